@@ -123,6 +123,28 @@ __device__ __forceinline__ void group_barrier(int a) {
   else asm volatile("bar.sync 2, 128;" ::: "memory");
 }
 
+// Hand-over of P and of the tensor turn through named barriers.  An mbarrier lives in shared
+// memory, whose bandwidth the MMA operands of Q K^T use up: an arrive or a try_wait there took
+// 120-270 clk, several times on every key tile's critical path; a named barrier takes 25-60 clk.
+// A named barrier has no bounded wait, so every role meets each of them a fixed number of times
+// (once per key tile of its segments), also after it has given up on an mbarrier.
+__device__ __forceinline__ void p_ready_arrive(int a) {   // softmax group a: P of a key tile is in TMEM
+  if (a == 0) asm volatile("bar.arrive 3, 160;" ::: "memory");
+  else asm volatile("bar.arrive 4, 160;" ::: "memory");
+}
+__device__ __forceinline__ void p_ready_sync(int a) {     // issuer a
+  if (a == 0) asm volatile("bar.sync 3, 160;" ::: "memory");
+  else asm volatile("bar.sync 4, 160;" ::: "memory");
+}
+__device__ __forceinline__ void turn_sync(int a) {        // issuer a waits for the tensor pipe
+  if (a == 0) asm volatile("bar.sync 5, 64;" ::: "memory");
+  else asm volatile("bar.sync 6, 64;" ::: "memory");
+}
+__device__ __forceinline__ void turn_pass(int a) {        // issuer a hands it to the other one
+  if (a == 0) asm volatile("bar.arrive 6, 64;" ::: "memory");
+  else asm volatile("bar.arrive 5, 64;" ::: "memory");
+}
+
 // Exponentials of 32 score columns (registers s) into 16 bf16 pairs (p) and the packed sums.
 __device__ __forceinline__ void exp_block32(const uint32_t* s, uint32_t* p, uint64_t c2, uint64_t nm2,
                                             uint64_t* acc) {
@@ -220,7 +242,7 @@ constexpr float kOptimisticLimit = 18446744073709551616.f;   // 2^64
 template <bool kMasked>
 __device__ __forceinline__ void softmax_row_tile(uint32_t t_S, uint32_t t_O, float c, int nvalid,
                                                  bool first, float& m_run, float& l_run,
-                                                 uint32_t bar_p_full, int trace_role, int trace_tile) {
+                                                 int a, int trace_role, int trace_tile) {
   if (first) m_run = max_row<kMasked>(t_S, nvalid);
   TRACE(trace_role, trace_tile, 2);
   uint32_t p0[32], p1[32];
@@ -249,7 +271,7 @@ __device__ __forceinline__ void softmax_row_tile(uint32_t t_S, uint32_t t_O, flo
   tmem_st32(t_S + 32, p1);   // P of keys 64..127 over score columns 32..63
   tc_wait_st();
   tc_fence_before();
-  mbar_arrive(bar_p_full);
+  p_ready_arrive(a);
   TRACE(trace_role, trace_tile, 5);
   l_run += sum;
 }
@@ -295,9 +317,7 @@ window_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
   const uint32_t bar_kv_full = sBar + 32;                    // [kStages] TMA -> both MMA warps
   const uint32_t bar_kv_empty = sBar + 32 + 8 * kStages;     // [kStages] both MMA warps -> TMA
   const uint32_t bar_s_full = sBar + 32 + 16 * kStages;      // [2]  MMA warp a -> softmax a
-  const uint32_t bar_p_full = bar_s_full + 16;               // [2]  softmax a -> MMA warp a (128 arrivals)
-  const uint32_t bar_o_final = bar_p_full + 16;              // [2]  MMA warp a -> softmax a
-  const uint32_t bar_mturn = bar_o_final + 16;               // [2]  MMA warp 1-a -> MMA warp a: your turn on the tensor pipe
+  const uint32_t bar_o_final = bar_s_full + 16;              // [2]  MMA warp a -> softmax a
   volatile uint32_t* tmem_slot = reinterpret_cast<volatile uint32_t*>(gen + kSmemBar + 224);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(gen + kSmemBar + 228);
   volatile int* merge_flag = reinterpret_cast<volatile int*>(gen + kSmemBar + 232);   // [2]
@@ -312,9 +332,7 @@ window_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
       mbar_init(bar_q_full + 8 * i, 1);
       mbar_init(bar_q_empty + 8 * i, 1);
       mbar_init(bar_s_full + 8 * i, 1);
-      mbar_init(bar_p_full + 8 * i, 128);
       mbar_init(bar_o_final + 8 * i, 1);
-      mbar_init(bar_mturn + 8 * i, 1);
     }
     for (int i = 0; i < kStages; ++i) {
       mbar_init(bar_kv_full + 8 * i, 1);
@@ -378,16 +396,19 @@ window_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
           }
         }
       }
-    } else if (warp <= 9 && lane == 0) {
+    } else if (warp <= 9) {
       // ------------------------------------------------------------ MMA issuer of query tile a
       // One issuing thread per query tile, on different scheduler partitions.  For each key
-      // tile: O_a += P_a V (two halves, as P arrives), then S_a = Q_a K_next^T.  Both warps
-      // walk the same K/V ring; a stage is released when both have retired it.
+      // tile: O_a += P_a V, then S_a = Q_a K_next^T.  Both warps walk the same K/V ring; a stage
+      // is released when both have retired it.  Lane 0 waits and issues; the whole warp meets
+      // the named barriers.
       const int a = warp - 8;
       Sched sched(p, static_cast<int>(blockIdx.x));
       Seg s;
-      uint32_t kv_it = 0, q_it = 0, sp_it = 0, mturn_it = 0;
+      uint32_t kv_it = 0, q_it = 0, turns = 0;
+      [[maybe_unused]] uint32_t sp_it = 0;   // key tiles so far (timeline stamps)
       bool ok = true;
+      const bool lead = lane == 0;
       const uint32_t idesc_pv = idesc_bf16_f32(kTileM, kHeadDim, 1);
       const uint32_t idesc_qk_full = idesc_bf16_f32(kTileM, kTileN, 0);
       // descriptors are built once; per instruction only the start-address field moves
@@ -395,7 +416,7 @@ window_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
       const uint64_t dk0 = smem_desc_sw128(sKV, 16, 1024);                  // stage 0 as a K tile
       const uint64_t dv0 = smem_desc_sw128(sKV, kHalfBytes, 1024);          // stage 0 as a V tile (MN-major)
       const uint32_t s_tmem = tmem_base + a * 128, o_tmem = tmem_base + 256 + a * 128;
-      const uint32_t my_s_full = bar_s_full + 8 * a, my_p_full = bar_p_full + 8 * a;
+      const uint32_t my_s_full = bar_s_full + 8 * a;
 
       // a ragged tile runs with N (for Q K^T) and K (for P V) rounded up to 16 keys
       auto issue_qk = [&](uint32_t stage, int valid) {
@@ -418,79 +439,78 @@ window_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
                    (accumulate || k > 0) ? 1u : 0u);
       };
 
-      while (ok && sched.next(s)) {
+      while (sched.next(s)) {
         const bool part = a < s.nq;   // a lone last query tile leaves warp 1 only the bookkeeping
         const int n = s.t1 - s.t0;
         const ValidKeys valid_of(p, s.b);
         int valid = valid_of(s.t0);  // real keys of the tile S is being computed for
         if (part) {
-          ok = w.wait(bar_q_full + 8 * a, q_it & 1);
-          if (!ok) break;
+          if (lead && ok) ok = w.wait(bar_q_full + 8 * a, q_it & 1);
           ++q_it;
         }
         uint32_t kst = kv_it % kStages;
-        ok = w.wait(bar_kv_full + 8 * kst, (kv_it / kStages) & 1);
-        if (!ok) break;
+        if (lead && ok) ok = w.wait(bar_kv_full + 8 * kst, (kv_it / kStages) & 1);
         ++kv_it;
-        if (part) {
-          tc_fence_after();
-          issue_qk(kst, valid);
-          // Q is free as soon as the item's last Q K^T has run: the producer fetches the next
-          // item's Q under this item's last exponentials and P V
-          if (n == 1) tc_commit(bar_q_empty + 8 * a);
-        } else {
-          mbar_arrive(bar_kv_empty + 8 * kst);
+        if (lead && ok) {
+          if (part) {
+            tc_fence_after();
+            issue_qk(kst, valid);
+            // Q is free as soon as the item's last Q K^T has run: the producer fetches the next
+            // item's Q under this item's last exponentials and P V
+            if (n == 1) tc_commit(bar_q_empty + 8 * a);
+          } else {
+            mbar_arrive(bar_kv_empty + 8 * kst);
+          }
         }
         for (int j = 0; j < n; ++j) {
           const int k_steps = (valid + 15) >> 4;
           const uint32_t vst = kv_it % kStages;
-          ok = w.wait(bar_kv_full + 8 * vst, (kv_it / kStages) & 1);
-          if (!ok) break;
+          if (lead && ok) ok = w.wait(bar_kv_full + 8 * vst, (kv_it / kStages) & 1);
           ++kv_it;
           const bool more = j + 1 < n;
           if (more) {
             valid = valid_of(s.t0 + j + 1);
             kst = kv_it % kStages;
-            ok = w.wait(bar_kv_full + 8 * kst, (kv_it / kStages) & 1);
-            if (!ok) break;
+            if (lead && ok) ok = w.wait(bar_kv_full + 8 * kst, (kv_it / kStages) & 1);
             ++kv_it;
           }
+          __syncwarp();
           if (part) {
             const uint64_t dv = dv0 + static_cast<uint64_t>((vst * kTileBytes) >> 4);
             TRACE(2 + a, sp_it, 0);
-            ok = w.wait(my_p_full, sp_it & 1);   // P of this tile is in TMEM, O rescaled if need be
-            if (!ok) break;
+            p_ready_sync(a);   // P of this tile is in TMEM, O rescaled if need be
             TRACE(2 + a, sp_it, 1);
             // The two issuers take turns with their P V + Q K^T chains: issued side by side the
             // chains would interleave in the tensor pipe and finish together, which pulls the
             // two query tiles into step; one after the other keeps them half a period apart.
             if (s.nq == 2) {
-              ok = w.wait(bar_mturn + 8 * a, (a == 0) ? ((mturn_it & 1) ^ 1) : (mturn_it & 1));
-              if (!ok) break;
+              if (a == 1 || turns > 0) turn_sync(a);
+              ++turns;
             }
             TRACE(2 + a, sp_it, 3);
-            tc_fence_after();
-            issue_pv_half(dv, 0, k_steps, j > 0);
-            issue_pv_half(dv, 1, k_steps, true);
-            TRACE(2 + a, sp_it, 4);
-            // the next S first (it is what the softmax warps wait for), the stage releases after it
-            if (more) issue_qk(kst, valid);
-            if (j + 2 == n) tc_commit(bar_q_empty + 8 * a);
-            tc_commit(bar_kv_empty + 8 * vst);
-            if (s.nq == 2) {
-              mbar_arrive(bar_mturn + 8 * (1 - a));
-              ++mturn_it;
+            if (lead && ok) {
+              tc_fence_after();
+              issue_pv_half(dv, 0, k_steps, j > 0);
+              issue_pv_half(dv, 1, k_steps, true);
+              TRACE(2 + a, sp_it, 4);
+              // the next S first (it is what the softmax warps wait for), the stage releases after it
+              if (more) issue_qk(kst, valid);
+              if (j + 2 == n) tc_commit(bar_q_empty + 8 * a);
+              tc_commit(bar_kv_empty + 8 * vst);
             }
+            __syncwarp();
+            if (s.nq == 2) turn_pass(a);
             TRACE(2 + a, sp_it, 5);
             ++sp_it;
-          } else {
+          } else if (lead && ok) {
             mbar_arrive(bar_kv_empty + 8 * vst);
             if (more) mbar_arrive(bar_kv_empty + 8 * kst);
           }
         }
-        if (!ok) break;
-        if (part) tc_commit(bar_o_final + 8 * a);
+        if (lead && ok && part) tc_commit(bar_o_final + 8 * a);
+        __syncwarp();
       }
+      if (a == 0 && turns > 0) turn_sync(0);   // the last turn that the other issuer passed back
     }
   } else {
     // ---------------------------------------------------------------- softmax warpgroups
@@ -501,7 +521,6 @@ window_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
     const int row = tid & 127;             // row inside the tile = TMEM lane
     const uint32_t t_lane = tmem_base + (static_cast<uint32_t>((warp & 3) * 32) << 16);
     const uint32_t t_S = t_lane + a * 128, t_O = t_lane + 256 + a * 128;
-    const uint32_t my_p_full = bar_p_full + 8 * a;
     volatile int* my_flag = merge_flag + a;
     Sched sched(p, static_cast<int>(blockIdx.x));
     Seg s;
@@ -509,25 +528,27 @@ window_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
     bool ok = true;
     int seg_no = 0;
     CTRACE(1);
-    // After a wait gave up (ok == false) a thread keeps walking its segments without working,
-    // so that it still meets its group at the barrier of the next split-item epilogue, where
-    // the whole group sees the abort flag and leaves together.
+    // After a wait gave up (ok == false) a thread keeps walking its segments without working, so
+    // that it still meets its group and its issuer at every named barrier.
     while (sched.next(s)) {
       if (a >= s.nq) continue;             // a lone last query tile: nothing for group 1
       float m_run = -INFINITY, l_run = 0.f;
       const ValidKeys valid_of(p, s.b);
-      for (int j = s.t0; j < s.t1 && ok; ++j) {
+      for (int j = s.t0; j < s.t1; ++j) {
         const int valid = valid_of(j);
         TRACE(a, it, 0);
-        ok = w.wait(bar_s_full + 8 * a, it & 1);
-        if (!ok) break;
+        if (ok) ok = w.wait(bar_s_full + 8 * a, it & 1);
+        if (!ok) {
+          p_ready_arrive(a);   // the issuer still counts on it
+          continue;
+        }
         tc_fence_after();
         if (it == 0) CTRACE(2);
         TRACE(a, it, 1);
         if (valid < kTileN)
-          softmax_row_tile<true>(t_S, t_O, p.scale_log2e, valid, j == s.t0, m_run, l_run, my_p_full, a, it);
+          softmax_row_tile<true>(t_S, t_O, p.scale_log2e, valid, j == s.t0, m_run, l_run, a, a, it);
         else
-          softmax_row_tile<false>(t_S, t_O, p.scale_log2e, kTileN, j == s.t0, m_run, l_run, my_p_full, a, it);
+          softmax_row_tile<false>(t_S, t_O, p.scale_log2e, kTileN, j == s.t0, m_run, l_run, a, a, it);
         ++it;
       }
       CTRACE(8 + seg_no);
@@ -584,7 +605,7 @@ window_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
           *my_flag = (seen == others) ? 1 : 0;
         }
         group_barrier(a);
-        if (*abort_flag) break;            // raised before the barrier by whoever gave up
+        if (*abort_flag) ok = false;       // somebody gave up: keep meeting the barriers, report nothing
         bool last = (*my_flag != 0);
         if (!last) {
           const int64_t mine = static_cast<int64_t>(2 * blockIdx.x + (s.first_in_worker ? 0 : 1)) * kPartFloats +
