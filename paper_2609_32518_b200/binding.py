@@ -1,4 +1,8 @@
-"""ctypes binding of libunstep.so: same names as the C ABI, argument marshalling only."""
+"""Binding of libunstep.so: same names as the C ABI, argument marshalling only.
+
+A call goes through the native marshalling module (csrc/marshal.cpp) when all its arguments have
+exactly the expected form; the module answers None for anything else, before anything is launched,
+and the general path in ctypes takes over and raises what there is to raise."""
 
 from __future__ import annotations
 
@@ -41,6 +45,7 @@ class Shape(ctypes.Structure):
 
 
 _lib = None
+_fast = None   # the native marshalling module, bound to the functions of _lib
 
 
 def lib() -> ctypes.CDLL:
@@ -92,6 +97,18 @@ def lib() -> ctypes.CDLL:
     return _lib
 
 
+def _native():
+    global _fast
+    if _fast is None:
+        L = lib()
+        mod = _build.load_marshal()
+        mod.bind(Shape, *(ctypes.cast(f, c_void_p).value for f in (
+            L.unstep_rope_table, L.unstep_rope_kv_append_sink, L.unstep_rmsnorm_rope_kv_append,
+            L.unstep_window_attn, L.unstep_window_attn_noalloc, L.unstep_window_attn_sink)))
+        _fast = mod
+    return _fast
+
+
 def strerror(code: int) -> str:
     return lib().unstep_strerror(int(code)).decode()
 
@@ -127,6 +144,15 @@ def _check(rc: int, where: str):
 
 def rope_table(shape: Shape, start_frame: int, cos, sin, stream=None):
     """unstep_rope_table: fill float32 cos/sin [L, 64] for the chunk starting at start_frame."""
+    rc = (_fast or _native()).rope_table(
+        shape, start_frame, cos, sin, stream)
+    if rc is None:
+        _general_rope_table(shape, start_frame, cos, sin, stream)
+    elif rc:
+        raise UnstepError(rc, "unstep_rope_table")
+
+
+def _general_rope_table(shape, start_frame, cos, sin, stream):
     import torch
     n = shape.chunk_tokens * 64
     _check(lib().unstep_rope_table(ctypes.byref(shape), int(start_frame),
@@ -138,6 +164,17 @@ def rope_table(shape: Shape, start_frame: int, cos, sin, stream=None):
 def rope_kv_append(shape: Shape, start_frame, q_in, k_in, v_in, cos, sin, q_out, ring_k, ring_v,
                    table_stream_stride: int = 0, stream=None):
     """unstep_rope_kv_append: rotate q/k, write k/v of the chunk into ring slots."""
+    rc = (_fast or _native()).append(
+        shape, 0, start_frame, q_in, k_in, v_in, cos, sin, q_out, ring_k, ring_v, table_stream_stride, stream)
+    if rc is None:
+        _general_rope_kv_append(shape, start_frame, q_in, k_in, v_in, cos, sin, q_out, ring_k, ring_v,
+                                table_stream_stride, stream)
+    elif rc:
+        raise UnstepError(rc, "unstep_rope_kv_append")
+
+
+def _general_rope_kv_append(shape, start_frame, q_in, k_in, v_in, cos, sin, q_out, ring_k, ring_v,
+                            table_stream_stride, stream):
     import torch
     bf = torch.bfloat16
     n = shape.batch * shape.chunk_tokens * shape.heads * shape.head_dim
@@ -155,6 +192,15 @@ def rope_kv_append(shape: Shape, start_frame, q_in, k_in, v_in, cos, sin, q_out,
 def window_attn(shape: Shape, start_frame, window_frames: int, q_rot, ring_k, ring_v, out,
                 stream=None):
     """unstep_window_attn: attention of the chunk's queries over the retained window."""
+    rc = (_fast or _native()).attn(
+        shape, start_frame, window_frames, q_rot, ring_k, ring_v, out, stream)
+    if rc is None:
+        _general_window_attn(shape, start_frame, window_frames, q_rot, ring_k, ring_v, out, stream)
+    elif rc:
+        raise UnstepError(rc, "unstep_window_attn")
+
+
+def _general_window_attn(shape, start_frame, window_frames, q_rot, ring_k, ring_v, out, stream):
     import torch
     bf = torch.bfloat16
     n = shape.batch * shape.chunk_tokens * shape.heads * shape.head_dim
@@ -173,6 +219,15 @@ def window_attn_noalloc(shape: Shape, start_frame, window_frames: int, q_rot, ri
     a deployment with a fixed footprint).  Its scratch is a fixed ~40 MB array inside the
     library; all calls on a device share it, so calls that may overlap on the GPU must be
     serialised by the caller.  Raises UnstepError(-5) when the problem exceeds the array."""
+    rc = (_fast or _native()).attn_noalloc(
+        shape, start_frame, window_frames, q_rot, ring_k, ring_v, out, stream)
+    if rc is None:
+        _general_window_attn_noalloc(shape, start_frame, window_frames, q_rot, ring_k, ring_v, out, stream)
+    elif rc:
+        raise UnstepError(rc, "unstep_window_attn_noalloc")
+
+
+def _general_window_attn_noalloc(shape, start_frame, window_frames, q_rot, ring_k, ring_v, out, stream):
     import torch
     bf = torch.bfloat16
     n = shape.batch * shape.chunk_tokens * shape.heads * shape.head_dim
@@ -187,6 +242,18 @@ def window_attn_noalloc(shape: Shape, start_frame, window_frames: int, q_rot, ri
 def rope_kv_append_sink(shape: Shape, sink_frames: int, start_frame, q_in, k_in, v_in, cos, sin, q_out,
                         cache_k, cache_v, table_stream_stride: int = 0, stream=None):
     """unstep_rope_kv_append_sink: the append with a sink prefix of `sink_frames` slots."""
+    rc = (_fast or _native()).append(
+        shape, sink_frames, start_frame, q_in, k_in, v_in, cos, sin, q_out, cache_k, cache_v,
+        table_stream_stride, stream)
+    if rc is None:
+        _general_rope_kv_append_sink(shape, sink_frames, start_frame, q_in, k_in, v_in, cos, sin, q_out,
+                                     cache_k, cache_v, table_stream_stride, stream)
+    elif rc:
+        raise UnstepError(rc, "unstep_rope_kv_append_sink")
+
+
+def _general_rope_kv_append_sink(shape, sink_frames, start_frame, q_in, k_in, v_in, cos, sin, q_out, cache_k,
+                                 cache_v, table_stream_stride, stream):
     import torch
     bf = torch.bfloat16
     n = shape.batch * shape.chunk_tokens * shape.heads * shape.head_dim
@@ -205,6 +272,18 @@ def rmsnorm_rope_kv_append(shape: Shape, sink_frames: int, start_frame, q_in, k_
                            eps: float, cos, sin, q_out, cache_k, cache_v, table_stream_stride: int = 0,
                            stream=None):
     """unstep_rmsnorm_rope_kv_append: RMSNorm of q and k, rotation and cache write in one kernel."""
+    rc = (_fast or _native()).norm_append(
+        shape, sink_frames, start_frame, q_in, k_in, v_in, gain_q, gain_k, eps, cos, sin, q_out, cache_k,
+        cache_v, table_stream_stride, stream)
+    if rc is None:
+        _general_rmsnorm_rope_kv_append(shape, sink_frames, start_frame, q_in, k_in, v_in, gain_q, gain_k,
+                                        eps, cos, sin, q_out, cache_k, cache_v, table_stream_stride, stream)
+    elif rc:
+        raise UnstepError(rc, "unstep_rmsnorm_rope_kv_append")
+
+
+def _general_rmsnorm_rope_kv_append(shape, sink_frames, start_frame, q_in, k_in, v_in, gain_q, gain_k, eps,
+                                    cos, sin, q_out, cache_k, cache_v, table_stream_stride, stream):
     import torch
     bf = torch.bfloat16
     n = shape.batch * shape.chunk_tokens * shape.heads * shape.head_dim
@@ -224,6 +303,17 @@ def rmsnorm_rope_kv_append(shape: Shape, sink_frames: int, start_frame, q_in, k_
 def window_attn_sink(shape: Shape, sink_frames: int, start_frame, recent_frames: int, sink_attend: int,
                      q_rot, cache_k, cache_v, out, stream=None):
     """unstep_window_attn_sink: attention over sink frames + the recent window."""
+    rc = (_fast or _native()).attn_sink(
+        shape, sink_frames, start_frame, recent_frames, sink_attend, q_rot, cache_k, cache_v, out, stream)
+    if rc is None:
+        _general_window_attn_sink(shape, sink_frames, start_frame, recent_frames, sink_attend, q_rot, cache_k,
+                                  cache_v, out, stream)
+    elif rc:
+        raise UnstepError(rc, "unstep_window_attn_sink")
+
+
+def _general_window_attn_sink(shape, sink_frames, start_frame, recent_frames, sink_attend, q_rot, cache_k,
+                              cache_v, out, stream):
     import torch
     bf = torch.bfloat16
     n = shape.batch * shape.chunk_tokens * shape.heads * shape.head_dim

@@ -1,10 +1,14 @@
-"""Builds libunstep.so (the C-ABI CUDA library) in-tree with nvcc for sm_100a."""
+"""Builds libunstep.so (the C-ABI CUDA library) in-tree with nvcc for sm_100a, and the native
+marshalling module of the Python binding with the host compiler."""
 
 from __future__ import annotations
 
+import importlib.machinery
+import importlib.util
 import os
 import shutil
 import subprocess
+import sysconfig
 
 PKG_DIR = os.path.dirname(os.path.abspath(__file__))
 ROOT = os.path.dirname(PKG_DIR)
@@ -24,7 +28,7 @@ def _nvcc() -> str:
 
 
 def _inputs():
-    files = [os.path.join(CSRC, f) for f in os.listdir(CSRC)]
+    files = [os.path.join(CSRC, f) for f in os.listdir(CSRC) if not f.endswith(".cpp")]
     files += [os.path.join(INCLUDE, f) for f in os.listdir(INCLUDE)]
     return files
 
@@ -32,8 +36,7 @@ def _inputs():
 # Diagnostic variants of the library, built beside the normal one as libunstep_<name>.so and
 # loaded instead of it when the environment variable UNSTEP_LIB_VARIANT names one.
 VARIANTS = {
-    "check": ["-DUNSTEP_CHECK"],
-    "abl3": ["-DNORM_ABL=3"],   # every global store bounds-checked, violations reported, never made
+    "check": ["-DUNSTEP_CHECK"],   # every global store bounds-checked, violations reported, never made
 }
 
 
@@ -68,6 +71,44 @@ def build(force: bool = False, verbose: bool = False, variant: str = "") -> str:
     if verbose:
         print(res.stderr)
     return path
+
+
+def marshal_path() -> str:
+    """The module is tied to the torch it was compiled against, so its name carries the version."""
+    import torch
+    return os.path.join(PKG_DIR, "_marshal_" + torch.__version__.replace("+", "_") + ".so")
+
+
+def build_marshal(force: bool = False) -> str:
+    """Compile csrc/marshal.cpp if it is missing or older than its sources; return its path."""
+    path = marshal_path()
+    inputs = [os.path.join(CSRC, "marshal.cpp"), os.path.join(INCLUDE, "unstep.h")]
+    if not force and os.path.exists(path) and all(os.path.getmtime(f) <= os.path.getmtime(path) for f in inputs):
+        return path
+    import torch
+    root = os.path.dirname(torch.__file__)
+    lib = os.path.join(root, "lib")
+    cuda = os.path.dirname(os.path.dirname(_nvcc()))
+    tmp = f"{path}.{os.getpid()}.tmp"
+    cmd = [os.environ.get("CXX", "g++"), "-O2", "-std=c++17", "-shared", "-fPIC", "-I", INCLUDE,
+           "-I", sysconfig.get_paths()["include"], "-I", os.path.join(root, "include"),
+           "-I", os.path.join(root, "include", "torch", "csrc", "api", "include"),
+           "-I", os.path.join(cuda, "include"), inputs[0], "-o", tmp, "-L", lib, "-ltorch_python",
+           "-ltorch_cpu", "-lc10", "-lc10_cuda", "-Wl,-rpath," + lib]
+    res = subprocess.run(cmd, capture_output=True, text=True)
+    if res.returncode != 0:
+        raise RuntimeError("building the marshalling module failed:\n" + res.stdout + res.stderr)
+    os.replace(tmp, path)
+    return path
+
+
+def load_marshal():
+    """Import the marshalling module (building it first if stale)."""
+    path = build_marshal()
+    loader = importlib.machinery.ExtensionFileLoader("_marshal", path)
+    module = importlib.util.module_from_spec(importlib.util.spec_from_file_location("_marshal", path, loader=loader))
+    loader.exec_module(module)
+    return module
 
 
 if __name__ == "__main__":
