@@ -1,20 +1,22 @@
 // RoPE coefficient table and the fused RoPE + KV-ring append (HBM-bound kernels).
 #include <cuda_bf16.h>
+#include <string.h>
+
+#include <cmath>
 
 #include "common.h"
 
 namespace unstep {
 
 // --------------------------------------------------------------------------
-// Table: one thread per (token, pair).  Angle and trig in double, one rounding.
+// Table.  Angle and trig in double, one rounding.
 // --------------------------------------------------------------------------
 struct TableParams {
-  int32_t start_frame, grid_h, grid_w, L;
+  int32_t start_frame, grid_h, grid_w, col_tiles;
   int32_t pairs_t, pairs_h;  // pairs_w = 64 - pairs_t - pairs_h
-  int32_t band_t, band_h, band_w;
-  double base;
-  int* status;       // status word and extent (floats) of each output, for checking builds
+  int* status;       // status word and extent (16-byte vectors) of each output, for checking builds
   int64_t extent;
+  double omega[kPairs];  // base^(-2i/d_band) of the 64 pairs
 };
 
 // cos and sin of position * omega in double, rounded once.
@@ -24,49 +26,80 @@ __device__ __forceinline__ float2 table_entry(double omega, int pos) {
   return make_float2(static_cast<float>(cs), static_cast<float>(sn));
 }
 
-// One block per (frame, token row).  The table is separable: a token's 64 coefficients are
-// 22 that depend on its frame only, 21 on its row only and 21 on its column only.  The block
-// evaluates those (22 + 21 + 21 * grid_w double-precision values) once into shared memory and
-// then writes its grid_w * 64 entries of cos and sin with coalesced stores (64 columns per pass).  Evaluating every
-// entry on its own costs 64 double pow/sincos per token instead of about 22.
-__global__ void __launch_bounds__(1024) rope_table_kernel(TableParams p, float* __restrict__ cos_out,
-                                                         float* __restrict__ sin_out) {
-  constexpr int kColsPerPass = 64;
-  __shared__ float2 band[kPairs + kColsPerPass * kPairs];   // frame/row part, then [column][pair]
-  __shared__ double omega[kPairs];                          // base^(-2i/d_band) of the 64 pairs
-  const int r = blockIdx.x, f = blockIdx.y;
-  const int pairs_w = kPairs - p.pairs_t - p.pairs_h;
-  const int n_fixed = p.pairs_t + p.pairs_h;
-  if (threadIdx.x < kPairs) {
-    const int j = threadIdx.x;
-    const int i = j < p.pairs_t ? j : (j < n_fixed ? j - p.pairs_t : j - n_fixed);
-    const int d = j < p.pairs_t ? p.band_t : (j < n_fixed ? p.band_h : p.band_w);
-    omega[j] = pow(p.base, -(2.0 * static_cast<double>(i)) / static_cast<double>(d));
+// One block per frame and tile of kTableRows x kTableCols tokens.  The table is separable: of a
+// token's 64 coefficients 22 depend on its frame only, 21 on its row only and 21 on its column
+// only, so a tile evaluates 22 + 8 * 21 + 8 * 21 = 358 double sincos for its 64 tokens (64 tokens
+// on their own: 4096), at most one per thread, and writes its entries from shared memory.  Bound by
+// the latency of launch, one sincos and one store: a block per whole token row, which evaluates
+// two per thread and the 64 frequencies by pow in each block, took 4.8 us at 3 x 45 x 80
+// tokens (5.5 MB), this takes 3.9 us.  The frequencies depend on the bands only and come from the host.
+constexpr int kTableRows = 8, kTableCols = 8, kTableThreads = 384;
+
+__global__ void __launch_bounds__(kTableThreads)
+rope_table_kernel(const __grid_constant__ TableParams p, float4* __restrict__ cos_out, float4* __restrict__ sin_out) {
+  __shared__ float2 band[kPairs * (kTableRows + kTableCols)];   // frame part, then [row][pair], then [column][pair]
+  const int row_tile = blockIdx.x / p.col_tiles, f = blockIdx.y;
+  const int r0 = row_tile * kTableRows, c0 = (blockIdx.x - row_tile * p.col_tiles) * kTableCols;
+  const int rows = min(kTableRows, p.grid_h - r0), cols = min(kTableCols, p.grid_w - c0);
+  const int n_fixed = p.pairs_t + p.pairs_h, pairs_w = kPairs - n_fixed;
+  const int row_part = p.pairs_t, col_part = row_part + rows * p.pairs_h;
+  for (int e = threadIdx.x; e < col_part + cols * pairs_w; e += kTableThreads) {
+    int j, pos;
+    if (e < row_part) {
+      j = e;
+      pos = p.start_frame + f;
+    } else if (e < col_part) {
+      const int r = (e - row_part) / p.pairs_h;
+      j = p.pairs_t + (e - row_part) - r * p.pairs_h;
+      pos = r0 + r;
+    } else {
+      const int c = (e - col_part) / pairs_w;
+      j = n_fixed + (e - col_part) - c * pairs_w;
+      pos = c0 + c;
+    }
+    band[e] = table_entry(p.omega[j], pos);
   }
   __syncthreads();
-  const int64_t row_base = (static_cast<int64_t>(f) * p.grid_h + r) * p.grid_w * kPairs;
-  for (int c0 = 0; c0 < p.grid_w; c0 += kColsPerPass) {
-    const int cols = min(kColsPerPass, p.grid_w - c0);
-    const int n_eval = n_fixed + cols * pairs_w;
-    for (int e = threadIdx.x; e < n_eval; e += blockDim.x) {
-      if (e < p.pairs_t) {
-        band[e] = table_entry(omega[e], p.start_frame + f);
-      } else if (e < n_fixed) {
-        band[e] = table_entry(omega[e], r);
-      } else {
-        const int c = (e - n_fixed) / pairs_w, i = (e - n_fixed) - c * pairs_w;
-        band[e] = table_entry(omega[n_fixed + i], c0 + c);
-      }
+  // a thread writes four pairs of a token; 16 threads write a token, so a warp stores 512 bytes of
+  // two neighbouring tokens
+  for (int i = threadIdx.x; i < rows * cols * (kPairs / 4); i += kTableThreads) {
+    const int token = i / (kPairs / 4), quad = i % (kPairs / 4);
+    const int r = token / cols, c = token - r * cols;
+    float2 v[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const int j = 4 * quad + u;
+      const int at = j < p.pairs_t ? j
+                     : j < n_fixed ? row_part + r * p.pairs_h + (j - p.pairs_t)
+                                   : col_part + c * pairs_w + (j - n_fixed);
+      v[u] = band[at];
     }
-    __syncthreads();
-    for (int idx = threadIdx.x; idx < cols * kPairs; idx += blockDim.x) {
-      const int c = idx >> 6, j = idx & 63;
-      const float2 v = j < n_fixed ? band[j] : band[n_fixed + c * pairs_w + (j - n_fixed)];
-      UNSTEP_STORE(cos_out, row_base + c0 * kPairs + idx, p.extent, v.x, p.status);
-      UNSTEP_STORE(sin_out, row_base + c0 * kPairs + idx, p.extent, v.y, p.status);
-    }
-    __syncthreads();
+    const int64_t dst = ((static_cast<int64_t>(f) * p.grid_h + r0 + r) * p.grid_w + c0 + c) * (kPairs / 4) + quad;
+    UNSTEP_STORE(cos_out, dst, p.extent, make_float4(v[0].x, v[1].x, v[2].x, v[3].x), p.status);
+    UNSTEP_STORE(sin_out, dst, p.extent, make_float4(v[0].y, v[1].y, v[2].y, v[3].y), p.status);
   }
+}
+
+// Frequencies of the 64 pairs; the last set is kept per thread (64 calls of pow cost about as much
+// as the launch).
+static const double* frequency_ladder(const unstep_shape_t* s) {
+  struct Ladder {
+    int32_t band_t = 0, band_h = 0, band_w = 0;
+    double base = 0.0, omega[kPairs];
+  };
+  static thread_local Ladder l;
+  if (l.band_t != s->band_t || l.band_h != s->band_h || l.band_w != s->band_w || l.base != s->rope_base) {
+    const int32_t bands[3] = {s->band_t, s->band_h, s->band_w};
+    int j = 0;
+    for (const int32_t d : bands)
+      for (int i = 0; i < d / 2; ++i)
+        l.omega[j++] = std::pow(s->rope_base, -(2.0 * static_cast<double>(i)) / static_cast<double>(d));
+    l.band_t = s->band_t;
+    l.band_h = s->band_h;
+    l.band_w = s->band_w;
+    l.base = s->rope_base;
+  }
+  return l.omega;
 }
 
 // --------------------------------------------------------------------------
@@ -344,22 +377,20 @@ extern "C" int unstep_rope_table(const unstep_shape_t* shape, int32_t start_fram
   if (!aligned16(cos_out) || !aligned16(sin_out)) return UNSTEP_ERR_INVALID_ARG;
   rc = check_device();
   if (rc != UNSTEP_OK) return rc;
+  if (shape->chunk_frames > 65535) return UNSTEP_ERR_INVALID_ARG;
   TableParams p;
   p.start_frame = start_frame;
   p.grid_h = shape->grid_h;
   p.grid_w = shape->grid_w;
-  p.L = shape->chunk_frames * shape->grid_h * shape->grid_w;
   p.pairs_t = shape->band_t / 2;
   p.pairs_h = shape->band_h / 2;
-  p.band_t = shape->band_t;
-  p.band_h = shape->band_h;
-  p.band_w = shape->band_w;
-  p.base = shape->rope_base;
   p.status = status_word();
-  p.extent = static_cast<int64_t>(p.L) * kPairs;
-  if (shape->chunk_frames > 65535) return UNSTEP_ERR_INVALID_ARG;
-  rope_table_kernel<<<dim3(shape->grid_h, shape->chunk_frames), 1024, 0,
-                      static_cast<cudaStream_t>(cuda_stream)>>>(p, cos_out, sin_out);
+  p.extent = static_cast<int64_t>(shape->chunk_frames) * shape->grid_h * shape->grid_w * (kPairs / 4);
+  memcpy(p.omega, frequency_ladder(shape), sizeof(p.omega));
+  p.col_tiles = (shape->grid_w + kTableCols - 1) / kTableCols;
+  const dim3 grid(p.col_tiles * ((shape->grid_h + kTableRows - 1) / kTableRows), shape->chunk_frames);
+  rope_table_kernel<<<grid, kTableThreads, 0, static_cast<cudaStream_t>(cuda_stream)>>>(
+      p, reinterpret_cast<float4*>(cos_out), reinterpret_cast<float4*>(sin_out));
   g_launches.fetch_add(1);
   return cudaGetLastError() == cudaSuccess ? UNSTEP_OK : UNSTEP_ERR_CUDA;
 }
