@@ -77,8 +77,9 @@ constexpr int kSmemKV = 2 * kTileBytes;
 constexpr int kSmemBar = kSmemKV + kStages * kTileBytes;
 constexpr int kAttnSmemBytes = kSmemBar + 256;
 
-// Partial result of one query tile of a split item: O[col][row] (unnormalised, relative to the
-// part's own reference maximum), then m[row], l[row].  Two tiles per slot, two slots per CTA.
+// Partial result of one query tile of a split item: O as [col / 4][row][col % 4] (unnormalised,
+// relative to the part's own reference maximum; a warp's 16-byte accesses are 512 consecutive
+// bytes), then (m, l)[row].  Two tiles per slot, two slots per CTA.
 constexpr int kPartTileFloats = 128 * 128 + 2 * 128;
 constexpr int kPartFloats = 2 * kPartTileFloats;
 struct Waiter {
@@ -553,6 +554,16 @@ window_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
       }
       CTRACE(8 + seg_no);
       // ---- epilogue of this group's query tile ----
+      const bool whole = (s.t0 == 0 && s.t1 == s.tiles);
+      // Part of a split item: the arrival counter, looked at under the wait for the last P V
+      auto counter = [&] { return p.counters + 2 * s.item + a; };
+      int seen = 0;
+      if (!whole && row == 0) {
+#ifdef UNSTEP_CHECK
+        if (2 * s.item + a >= p.extent_counters) atomicExch(p.status, static_cast<int>(UNSTEP_ERR_BOUNDS));
+#endif
+        asm volatile("ld.acquire.gpu.global.s32 %0, [%1];" : "=r"(seen) : "l"(counter()) : "memory");
+      }
       if (ok) {
         ok = w.wait(bar_o_final + 8 * a, seg_it & 1);
         ++seg_it;
@@ -572,7 +583,6 @@ window_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
           UNSTEP_STORE(out_v, d + i, p.extent_out, vv, p.status);
         }
       };
-      const bool whole = (s.t0 == 0 && s.t1 == s.tiles);
       if (whole) {
         // O / l -> bf16 -> out[b][n][h][:]: a thread writes its whole 256-byte row
         if (ok) {
@@ -595,40 +605,35 @@ window_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
         const int c_lo = first_part_worker(p, s);
         const int c_hi = last_part_worker(p, s);
         const int others = c_hi - c_lo;
-        int* counter = p.counters + 2 * s.item + a;
-#ifdef UNSTEP_CHECK
-        if (row == 0 && 2 * s.item + a >= p.extent_counters) atomicExch(p.status, static_cast<int>(UNSTEP_ERR_BOUNDS));
-#endif
-        if (row == 0 && ok) {
-          int seen;
-          asm volatile("ld.acquire.gpu.global.s32 %0, [%1];" : "=r"(seen) : "l"(counter) : "memory");
-          *my_flag = (seen == others) ? 1 : 0;
-        }
+        if (row == 0) *my_flag = (seen == others) ? 1 : 0;
         group_barrier(a);
         if (*abort_flag) ok = false;       // somebody gave up: keep meeting the barriers, report nothing
         bool last = (*my_flag != 0);
         if (!last) {
-          const int64_t mine = static_cast<int64_t>(2 * blockIdx.x + (s.first_in_worker ? 0 : 1)) * kPartFloats +
-                               a * kPartTileFloats;   // first float of this part in the scratch
+          const int64_t mine = (static_cast<int64_t>(2 * blockIdx.x + (s.first_in_worker ? 0 : 1)) * kPartFloats +
+                                a * kPartTileFloats);   // first float of this part in the scratch
+          float4* const part4 = reinterpret_cast<float4*>(p.part);
+          const int64_t mine4 = mine / 4 + row;
 #pragma unroll
           for (int q = 0; q < 4; ++q) {
             uint32_t o[32];
             tmem_ld32(t_O + q * 32, o);
             tc_wait_ld32(o);
 #pragma unroll
-            for (int i = 0; i < 32; ++i)
-              UNSTEP_STORE(p.part, mine + (q * 32 + i) * 128 + row, p.extent_part, __uint_as_float(o[i]), p.status);
+            for (int i = 0; i < 8; ++i)
+              UNSTEP_STORE(part4, mine4 + (q * 8 + i) * 128, p.extent_part / 4,
+                           make_float4(__uint_as_float(o[4 * i]), __uint_as_float(o[4 * i + 1]),
+                                       __uint_as_float(o[4 * i + 2]), __uint_as_float(o[4 * i + 3])),
+                           p.status);
           }
-          UNSTEP_STORE(p.part, mine + 128 * 128 + row, p.extent_part, m_run, p.status);
-          UNSTEP_STORE(p.part, mine + 128 * 128 + 128 + row, p.extent_part, l_run, p.status);
-          __threadfence();
-          group_barrier(a);   // all of this part is published; everyone has read the flag
+          UNSTEP_STORE(reinterpret_cast<float2*>(p.part), mine / 2 + 128 * 64 + row, p.extent_part / 2,
+                       make_float2(m_run, l_run), p.status);
+          group_barrier(a);   // all of this part is stored; everyone has read the flag
           if (row == 0) {
-            // release: the group's stores (fenced above, ordered before this thread by the barrier)
-            // become visible before the count; acquire: a merging part sees the other parts' stores
-            __threadfence();
-            const int before = atomicAdd(counter, 1);
-            __threadfence();
+            // release: the group's stores (ordered before this thread by the barrier) become visible
+            // before the count; acquire: a merging part sees the other parts' stores
+            int before;
+            asm volatile("atom.acq_rel.gpu.global.add.s32 %0, [%1], 1;" : "=r"(before) : "l"(counter()) : "memory");
             *my_flag = (before == others) ? 1 : 0;
           }
           group_barrier(a);
@@ -642,40 +647,60 @@ window_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
             return p.part + (static_cast<int64_t>(2 * c + part_slot(p, c, s.item_step0)) * kPartFloats +
                              a * kPartTileFloats);
           };
-          float m_all = m_run;
-          for (int c = c_lo; c <= c_hi; ++c)
-            if (c != me) m_all = fmaxf(m_all, __ldcg(part_of(c) + 128 * 128 + row));
-          float l_sum = 0.f;
-          for (int c = c_lo; c <= c_hi; ++c) {
-            const float* pc = part_of(c);
-            const float m_c = c == me ? m_run : __ldcg(pc + 128 * 128 + row);
-            const float l_c = c == me ? l_run : __ldcg(pc + 128 * 128 + 128 + row);
-            l_sum += l_c * ex2((m_c - m_all) * p.scale_log2e);
+          auto ml_of = [&](int c) -> float2 {
+            return c == me ? make_float2(m_run, l_run)
+                           : __ldcg(reinterpret_cast<const float2*>(part_of(c) + 128 * 128) + row);
+          };
+          float m_all = m_run, l_sum = 0.f;
+          if (others == 1) {   // the common case: one round trip
+            const float2 x = ml_of(c_lo), y = ml_of(c_hi);
+            m_all = fmaxf(x.x, y.x);
+            l_sum = x.y * ex2((x.x - m_all) * p.scale_log2e) + y.y * ex2((y.x - m_all) * p.scale_log2e);
+          } else {
+#pragma unroll 2
+            for (int c = c_lo; c <= c_hi; ++c) m_all = fmaxf(m_all, ml_of(c).x);
+#pragma unroll 2
+            for (int c = c_lo; c <= c_hi; ++c) {
+              const float2 x = ml_of(c);
+              l_sum += x.y * ex2((x.x - m_all) * p.scale_log2e);
+            }
           }
           const float inv_l = 1.f / l_sum;
 #pragma unroll 1
-          for (int q = 0; q < 4; ++q) {   // 32 output columns at a time
-            float acc[32];
+          for (int q = 0; q < 2; ++q) {   // 64 output columns at a time
+            float acc[64];
 #pragma unroll
-            for (int i = 0; i < 32; ++i) acc[i] = 0.f;
+            for (int i = 0; i < 64; ++i) acc[i] = 0.f;
             for (int c = c_lo; c <= c_hi; ++c) {
-              float v[32];
-              float m_c;
               if (c == me) {
-                tmem_ld32(t_O + 32 * q, reinterpret_cast<uint32_t*>(v));
-                tc_wait_ld32(reinterpret_cast<uint32_t*>(v));
-                m_c = m_run;
+                const float sc = ex2((m_run - m_all) * p.scale_log2e);
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                  uint32_t o[32];
+                  tmem_ld32(t_O + 64 * q + 32 * h, o);
+                  tc_wait_ld32(o);
+#pragma unroll
+                  for (int i = 0; i < 32; ++i) acc[32 * h + i] = fmaf(__uint_as_float(o[i]), sc, acc[32 * h + i]);
+                }
               } else {
-                const float* pc = part_of(c);
+                const float4* pc = reinterpret_cast<const float4*>(part_of(c)) + q * 16 * 128 + row;
+                float4 v[16];
 #pragma unroll
-                for (int i = 0; i < 32; ++i) v[i] = __ldcg(pc + (32 * q + i) * 128 + row);
-                m_c = __ldcg(pc + 128 * 128 + row);
+                for (int i = 0; i < 16; ++i) v[i] = __ldcg(pc + i * 128);
+                const float sc = ex2((ml_of(c).x - m_all) * p.scale_log2e);
+#pragma unroll
+                for (int i = 0; i < 16; ++i) {
+                  acc[4 * i] = fmaf(v[i].x, sc, acc[4 * i]);
+                  acc[4 * i + 1] = fmaf(v[i].y, sc, acc[4 * i + 1]);
+                  acc[4 * i + 2] = fmaf(v[i].z, sc, acc[4 * i + 2]);
+                  acc[4 * i + 3] = fmaf(v[i].w, sc, acc[4 * i + 3]);
+                }
               }
-              const float sc = ex2((m_c - m_all) * p.scale_log2e);
-#pragma unroll
-              for (int i = 0; i < 32; ++i) acc[i] = fmaf(v[i], sc, acc[i]);
             }
-            if (n < p.L) store_row(dst + 4 * q, acc, inv_l);
+            if (n < p.L) {
+              store_row(dst + 8 * q, acc, inv_l);
+              store_row(dst + 8 * q + 4, acc + 32, inv_l);
+            }
           }
         }
       }

@@ -19,7 +19,7 @@ namespace unstep {
 
 constexpr int kTileM = 128;                 // queries per tile (two tiles per work item)
 constexpr int kTileN = 128;                 // keys per tile
-constexpr int kMinStepsPerWorker = 4;       // a launch smaller than this per worker uses fewer workers
+constexpr int kMinStepsPerWorker = 4;       // shortest share of the remainder that may cross items
 
 struct AttnParams {
   int32_t Hn, L, T, C;
@@ -31,8 +31,10 @@ struct AttnParams {
   float scale_log2e;        // log2(e) / sqrt(128)
   int32_t items_per_stream; // Hn * q_pairs
   int32_t n_workers;        // workers of the launch (grid size, or clusters)
-  int32_t n_active;         // workers that take a share of the remainder: min(n_workers, steps / 4), >= 1
-  int32_t full_rounds;      // whole rounds per stream: items_per_stream / n_workers
+  int32_t full_rounds;      // whole rounds per stream, n_workers items each
+  int32_t leftover;         // items per stream behind the whole rounds: the remainder
+  int32_t parts;            // > 0: every item of the remainder is cut into this many parts, one per worker
+  int32_t n_active;         // parts == 0: workers that take a share of the remainder, >= 1
   int64_t total_steps;      // remainder: sum over the leftover items of their key tiles
   float* part;              // workspace: partial results of split items, kPartFloats per slot
   int* counters;            // workspace: arrivals per (item, query tile), zero between launches
@@ -58,7 +60,7 @@ struct Seg {
   int b, h, qp, nq, t0, t1;
   int tiles;             // key tiles of the whole item
   int item;              // item index inside the launch
-  int64_t item_step0;    // global step index of the item's first tile
+  int64_t item_step0;    // remainder: step index of the item's first tile, with p.parts its first worker
   bool first_in_worker;  // this segment starts the worker's range
 };
 
@@ -107,12 +109,14 @@ UNSTEP_HD TileInfo tile_info(const AttnParams& p, int b, int j) {
 //   1. Whole rounds: while a stream still has at least n_workers items, worker c takes item
 //      (round * n_workers + c) whole.  All workers walk the key tiles in step, so a K/V tile is
 //      fetched from HBM once and then hit in L2 by the other workers of the head.
-//   2. Remainder: the leftover items of all streams (fewer than n_workers per stream) form one
-//      sequence of (item, key tile) steps, and each of the first n_active workers takes an equal
-//      contiguous share of it (n_active <= total_steps, so no share is empty and the workers
-//      that hold parts of an item are exactly those between the owners of its first and last
-//      step).  An item that straddles a boundary is split along its keys; the parts are merged
-//      by whichever worker finishes last.
+//   2. Remainder: the leftover items of all streams (fewer than n_workers per stream), split along
+//      their keys in one of two ways (plan_launch chooses):
+//      - p.parts > 0: every item is cut into p.parts parts and each worker takes one of them;
+//      - p.parts == 0: the items form one sequence of (item, key tile) steps, and each of the first
+//        n_active workers takes an equal contiguous share of it (n_active <= total_steps, so no
+//        share is empty and the workers that hold parts of an item are exactly those between the
+//        owners of its first and last step).
+//      The parts of an item are merged by whichever worker finishes last.
 struct Sched {
   int64_t lo, hi, cur;
   int b_round, round;   // position in the whole rounds
@@ -128,8 +132,13 @@ struct Sched {
     return static_cast<int>(c);
   }
   UNSTEP_HD Sched(const AttnParams& prm, int worker) : me(worker), p(prm) {
-    lo = worker_lo(p, worker);
-    hi = worker_lo(p, worker + 1);
+    if (p.parts > 0) {   // cur: the worker's part, hi: one past it
+      lo = worker;
+      hi = worker < static_cast<int64_t>(p.n_streams) * p.leftover * p.parts ? lo + 1 : lo;
+    } else {
+      lo = worker_lo(p, worker);
+      hi = worker_lo(p, worker + 1);
+    }
     cur = lo;
     b_round = 0;
     round = 0;
@@ -157,6 +166,17 @@ struct Sched {
       ++b_round;
     }
     if (cur >= hi) return false;             // remainder
+    if (p.parts > 0) {
+      const int item = me / p.parts, part = me - item * p.parts;
+      const int b = item / p.leftover;
+      decode(s, b, p.full_rounds * p.n_workers + item - b * p.leftover);
+      s.t0 = s.tiles * part / p.parts;
+      s.t1 = s.tiles * (part + 1) / p.parts;
+      s.item_step0 = me - part;
+      s.first_in_worker = true;
+      cur = hi;
+      return true;
+    }
     int b = 0;
     while (b + 1 < p.n_streams && p.step_base[b + 1] <= cur) ++b;
     const int tiles = p.tiles[b];
@@ -176,12 +196,40 @@ struct Sched {
 // Parts of a split item: the workers that own its first and its last step, and the scratch slot
 // (0 or 1 of the two a worker has) in which worker c publishes its part of the item that starts
 // at global step item_step0.
-UNSTEP_HD int first_part_worker(const AttnParams& p, const Seg& s) { return Sched::worker_of(p, s.item_step0); }
+UNSTEP_HD int first_part_worker(const AttnParams& p, const Seg& s) {
+  return p.parts > 0 ? static_cast<int>(s.item_step0) : Sched::worker_of(p, s.item_step0);
+}
 UNSTEP_HD int last_part_worker(const AttnParams& p, const Seg& s) {
-  return Sched::worker_of(p, s.item_step0 + s.tiles - 1);
+  return p.parts > 0 ? static_cast<int>(s.item_step0) + p.parts - 1 : Sched::worker_of(p, s.item_step0 + s.tiles - 1);
 }
 UNSTEP_HD int part_slot(const AttnParams& p, int c, int64_t item_step0) {
-  return Sched::worker_lo(p, c) >= item_step0 ? 0 : 1;   // 0: the part starts the worker's range
+  return p.parts > 0 || Sched::worker_lo(p, c) >= item_step0 ? 0 : 1;   // 0: the part starts the worker's range
+}
+
+// How the remainder (`items` of `least` to `most` key tiles, `steps` in all) is split: the number of
+// parts per item, or 0 for `*shares` equal shares across the items.  Parts leave a worker with one
+// part of one item; shares give the workers less to do, but each then holds parts of two items, one
+// after the other, each with a hand-over, and an item falls into more parts.  The estimates (us)
+// are fitted to launches of 2 to 40 items of 6 to 85 key tiles on a B200: a step 1.6; a second part
+// 3.4, each further one 1.6; shares 6 and 2.2 for each part of an item.  Measured, us: 8 items x 43
+// steps 85 whole, 5 parts 38, 8 parts 39, 86 shares of 4 steps 44; 40 items x 16 steps 38 whole, 3
+// parts 30, 148 shares 44; 80 items x 37 steps behind a whole round: shares, 140 against 160 whole.
+inline int32_t remainder_parts(int64_t items, int64_t steps, int32_t least, int32_t most, int max_workers,
+                               int32_t* shares) {
+  int64_t n = steps / kMinStepsPerWorker;
+  n = n < 1 ? 1 : (n > max_workers ? max_workers : n);
+  *shares = static_cast<int32_t>(n);
+  const double share = static_cast<double>((steps + n - 1) / n);
+  double lowest = 1.6 * share + 6.0 + 2.2 * (static_cast<double>(steps) / static_cast<double>(items) / share + 1.0);
+  int32_t best = 0;
+  for (int32_t parts = 1; parts * items <= max_workers && parts <= least; ++parts) {
+    const double cost = 1.6 * ((most + parts - 1) / parts) + (parts > 1 ? 3.4 + 1.6 * (parts - 2) : 0.0);
+    if (cost < lowest) {
+      lowest = cost;
+      best = parts;
+    }
+  }
+  return best;
 }
 
 // Fills the per-launch part of `p` for streams [b0, b0 + nb): the attended frames of each stream
@@ -221,23 +269,28 @@ inline int plan_launch(AttnParams& p, const unstep_shape_t* shape, const int32_t
       p.tiles[i] = (n_sink + hi - lo) * p.tiles_per_frame;
     }
   }
-  // one worker per SM (or SM pair), fewer when the whole launch is small
-  int64_t all_steps = 0;
-  for (int i = 0; i < nb; ++i) all_steps += static_cast<int64_t>(p.items_per_stream) * p.tiles[i];
-  int64_t want = all_steps / kMinStepsPerWorker;
-  if (want < 1) want = 1;
-  p.n_workers = static_cast<int32_t>(want < max_workers ? want : max_workers);
-  p.full_rounds = p.items_per_stream / p.n_workers;
-  const int leftover = p.items_per_stream - p.full_rounds * p.n_workers;
+  // One worker per SM where there are whole rounds for all of them; a launch of fewer items than
+  // that is all remainder, and has the workers that the split asks for.
+  const int64_t all_items = static_cast<int64_t>(nb) * p.items_per_stream;
+  p.n_workers = max_workers;
+  p.full_rounds = all_items > max_workers ? p.items_per_stream / max_workers : 0;
+  p.leftover = p.items_per_stream - p.full_rounds * max_workers;
   int64_t steps = 0;
+  int32_t least = INT32_MAX, most = 0;
   for (int i = 0; i < nb; ++i) {
     p.step_base[i] = steps;
-    steps += static_cast<int64_t>(leftover) * p.tiles[i];
+    steps += static_cast<int64_t>(p.leftover) * p.tiles[i];
+    least = p.tiles[i] < least ? p.tiles[i] : least;
+    most = p.tiles[i] > most ? p.tiles[i] : most;
   }
   p.total_steps = steps;
-  int64_t active = steps / kMinStepsPerWorker;
-  if (active < 1) active = 1;
-  p.n_active = static_cast<int32_t>(active < p.n_workers ? active : p.n_workers);
+  p.parts = 0;
+  p.n_active = 1;
+  if (steps > 0) {
+    const int64_t items = static_cast<int64_t>(nb) * p.leftover;
+    p.parts = remainder_parts(items, steps, least, most, max_workers, &p.n_active);
+    if (p.full_rounds == 0) p.n_workers = p.parts > 0 ? static_cast<int32_t>(items) * p.parts : p.n_active;
+  }
   return UNSTEP_OK;
 }
 

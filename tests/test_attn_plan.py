@@ -98,3 +98,18 @@ def test_sink_prefix_and_bad_arguments():
         U.window_attn_plan(sh, [18], 7, 148)          # window longer than the ring
     with pytest.raises(U.UnstepError):
         U.window_attn_plan(sh, [18], 6, 0)            # no workers
+
+
+def test_launches_smaller_than_the_grid_cut_every_item_into_equal_parts():
+    # (batch, heads, grid, chunk frames, ring, window, starts) -> parts of every item
+    for b, heads, grid, fc, ring, win, starts, parts in [
+            (2, 5, (17, 23), 2, 7, 5, [12, 8], 3),     # items of 16 and of 17 key tiles
+            (1, 1, (20, 30), 3, 9, 9, [12], 5),
+            (3, 1, (11, 13), 3, 9, 9, [0, 6, 12], 3),  # items of 4 and of 11 key tiles
+            (1, 3, (9, 14), 1, 5, 5, [6], 1)]:         # whole items
+        sh = U.Shape.make(batch=b, heads=heads, chunk_frames=fc, grid_h=grid[0], grid_w=grid[1], ring_frames=ring)
+        segs = check_plan(sh, starts, win, 148)
+        assert {s[8] for s in segs} == {parts}
+        assert len(segs) == 1 + max(s[0] for s in segs)   # one segment per worker
+        for s in segs:
+            assert abs((s[6] - s[5]) - s[7] / parts) < 1

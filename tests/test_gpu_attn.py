@@ -268,3 +268,17 @@ def test_remainder_smaller_than_the_grid():
                     k_scale=4.0)
     # the two leftover items are the last two query pairs of the last head: rows 3328.. of head 9
     run(wl, rows_fn=lambda L: np.concatenate([W.sample_rows(L, per_tile=2), np.arange(3328, L, 7)]), heads=[0, 9])
+
+
+@pytest.mark.parametrize("batch,heads,grid,fc,ring,win,history,starts", [
+    (2, 5, (17, 23), 2, 7, 5, ((4, 6, 8, 10), (2, 4, 6)), (12, 8)),        # 3 parts, 16 and 17 key tiles
+    (1, 1, (20, 30), 3, 9, 9, ((3, 6, 9),), (12,)),                        # 5 parts
+    (3, 1, (11, 13), 3, 9, 9, ((), (0, 3), (3, 6, 9)), (0, 6, 12)),        # 3 parts, 4 and 11 key tiles
+    (2, 4, (16, 24), 1, 6, 6, (tuple(range(3, 9)), (0,)), (9, 1)),         # 4 parts, a lone query tile
+    (1, 3, (9, 14), 1, 5, 5, ((1, 2, 3, 4, 5),), (6,)),                    # whole items, frames below a tile
+])
+def test_items_cut_into_equal_parts(batch, heads, grid, fc, ring, win, history, starts):
+    sh = W.Shape(batch=batch, heads=heads, chunk_frames=fc, grid_h=grid[0], grid_w=grid[1], ring_frames=ring)
+    wl = W.Workload("parts", sh, seed=31, history_starts=history, measured_starts=starts, window_frames=(win,),
+                    k_scale=4.0)
+    run(wl)
