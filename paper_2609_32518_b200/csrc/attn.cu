@@ -350,6 +350,8 @@ window_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
+  // What comes before a role's grid_wait may run under the kernel before this one.  Every role waits
+  // there, so that no bounded wait counts that kernel's time.
   const Waiter w{abort_flag, kWaitCycles};
 
   if (warp >= 8) {
@@ -361,6 +363,7 @@ window_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
       prefetch_tensormap(&tm_v);
       prefetch_tensormap(&tm_kf);
       prefetch_tensormap(&tm_vf);
+      grid_wait();
       Sched sched(p, static_cast<int>(blockIdx.x));
       Seg s;
       uint32_t kv_it = 0, q_it[2] = {0, 0};
@@ -403,6 +406,7 @@ window_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
       // tile: O_a += P_a V, then S_a = Q_a K_next^T.  Both warps walk the same K/V ring; a stage
       // is released when both have retired it.  Lane 0 waits and issues; the whole warp meets
       // the named barriers.
+      grid_wait();
       const int a = warp - 8;
       Sched sched(p, static_cast<int>(blockIdx.x));
       Seg s;
@@ -518,6 +522,7 @@ window_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
     // Warps 0-3 own query tile 0, warps 4-7 query tile 1; a thread owns a row from the scores
     // to the output.  The groups never wait for each other.
     reg_alloc_softmax();
+    grid_wait();
     const int a = warp >> 2;               // query tile of this warpgroup
     const int row = tid & 127;             // row inside the tile = TMEM lane
     const uint32_t t_lane = tmem_base + (static_cast<uint32_t>((warp & 3) * 32) << 16);
@@ -873,6 +878,8 @@ using namespace unstep;
 // arrival counters.
 typedef int (*ScratchFn)(cudaStream_t st, size_t slots, size_t n_counters, Workspace* out);   // an unstep_status
 
+constexpr int kOverlapSteps = 64;   // key-tile steps per worker below which a launch overlaps the kernel before it
+
 // Validation, work split, tensor maps and launch shared by the attention entry points.
 // The cache has `sink_frames` slots in front of the ring (0 for the plain rolling window);
 // stream b attends frames [0, min(sink_attend, lo)) and [lo, hi), lo = max(0, hi - window_frames).
@@ -928,9 +935,15 @@ static int window_attn_run(const unstep_shape_t* shape, const int32_t* start_fra
         !make_map(&tm_v, vb, 5, rdims, rstr, 2) || !make_map(&tm_kf, kb, 4, fdims, fstr, 2) ||
         !make_map(&tm_vf, vb, 4, fdims, fstr, 2))
       return UNSTEP_ERR_CUDA;
-    window_attn_kernel<<<p.n_workers, kThreads, kAttnSmemBytes, st>>>(tm_q, tm_k, tm_v, tm_kf, tm_vf, p, ob);
+    // Set up under the append before it where the launch is short: five heads and two streams
+    // 36 -> 32 us with the append, 57 steps per worker 166.7 -> 164.7 us.  Long launches run at the
+    // power cap, where the saved 2 us of idling show as a lower clock: 256 key tiles and 133 steps
+    // per worker took 898 us overlapped and 886 not, four layers of 64 steps 1609 and 1601.
+    const bool brief = p.all_steps < static_cast<int64_t>(kOverlapSteps) * p.n_workers;
+    const cudaError_t err = launch_overlapped(brief, window_attn_kernel, p.n_workers, kThreads, kAttnSmemBytes, st, tm_q,
+                                              tm_k, tm_v, tm_kf, tm_vf, p, ob);
     g_launches.fetch_add(1);
-    if (cudaGetLastError() != cudaSuccess) return UNSTEP_ERR_CUDA;
+    if (err != cudaSuccess) return UNSTEP_ERR_CUDA;
   }
   return UNSTEP_OK;
 }

@@ -35,6 +35,7 @@ struct AttnParams {
   int32_t leftover;         // items per stream behind the whole rounds: the remainder
   int32_t parts;            // > 0: every item of the remainder is cut into this many parts, one per worker
   int32_t n_active;         // parts == 0: workers that take a share of the remainder, >= 1
+  int64_t all_steps;        // key tiles of all items of the launch
   int64_t total_steps;      // remainder: sum over the leftover items of their key tiles
   float* part;              // workspace: partial results of split items, kPartFloats per slot
   int* counters;            // workspace: arrivals per (item, query tile), zero between launches
@@ -276,9 +277,11 @@ inline int plan_launch(AttnParams& p, const unstep_shape_t* shape, const int32_t
   p.full_rounds = all_items > max_workers ? p.items_per_stream / max_workers : 0;
   p.leftover = p.items_per_stream - p.full_rounds * max_workers;
   int64_t steps = 0;
+  p.all_steps = 0;
   int32_t least = INT32_MAX, most = 0;
   for (int i = 0; i < nb; ++i) {
     p.step_base[i] = steps;
+    p.all_steps += static_cast<int64_t>(p.items_per_stream) * p.tiles[i];
     steps += static_cast<int64_t>(p.leftover) * p.tiles[i];
     least = p.tiles[i] < least ? p.tiles[i] : least;
     most = p.tiles[i] > most ? p.tiles[i] : most;

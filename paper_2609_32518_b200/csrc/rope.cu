@@ -60,6 +60,8 @@ rope_table_kernel(const __grid_constant__ TableParams p, float4* __restrict__ co
     band[e] = table_entry(p.omega[j], pos);
   }
   __syncthreads();
+  grid_launch_next();
+  grid_wait();   // the evaluation above overlaps the kernel before this one, the stores do not
   // a thread writes four pairs of a token; 16 threads write a token, so a warp stores 512 bytes of
   // two neighbouring tokens
   for (int i = threadIdx.x; i < rows * cols * (kPairs / 4); i += kTableThreads) {
@@ -141,6 +143,8 @@ rope_kv_append_kernel(AppendParams p, const uint4* q_in, const uint4* __restrict
                       const uint4* __restrict__ v_in, const float4* __restrict__ cos_t,
                       const float4* __restrict__ sin_t, uint4* q_out,
                       uint4* __restrict__ ring_k, uint4* __restrict__ ring_v) {
+  grid_launch_next();
+  grid_wait();
   const int b = blockIdx.y;
   const int64_t v = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
   if (v >= p.vec_per_stream) return;
@@ -222,6 +226,8 @@ rmsnorm_rope_kv_append_kernel(AppendParams p, float eps, const uint4* q_in, cons
                               const float4* __restrict__ gain_k, const float4* __restrict__ cos_t,
                               const float4* __restrict__ sin_t, uint4* q_out, uint4* __restrict__ ring_k,
                               uint4* __restrict__ ring_v) {
+  grid_launch_next();
+  grid_wait();
   const int b = blockIdx.y;
   const int lane = threadIdx.x & 31;
   const int n = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);   // token of this warp
@@ -303,6 +309,8 @@ rmsnorm_rope_kv_append_token_kernel(AppendParams p, float eps, const uint4* q_in
                                     const float4* __restrict__ sin_t, uint4* q_out, uint4* __restrict__ ring_k,
                                     uint4* __restrict__ ring_v) {
   __shared__ double part[2][8];
+  grid_launch_next();
+  grid_wait();
   const int b = blockIdx.y;
   const int n = blockIdx.x;   // token
   const int tid = threadIdx.x, nthr = blockDim.x;
@@ -389,10 +397,11 @@ extern "C" int unstep_rope_table(const unstep_shape_t* shape, int32_t start_fram
   memcpy(p.omega, frequency_ladder(shape), sizeof(p.omega));
   p.col_tiles = (shape->grid_w + kTableCols - 1) / kTableCols;
   const dim3 grid(p.col_tiles * ((shape->grid_h + kTableRows - 1) / kTableRows), shape->chunk_frames);
-  rope_table_kernel<<<grid, kTableThreads, 0, static_cast<cudaStream_t>(cuda_stream)>>>(
-      p, reinterpret_cast<float4*>(cos_out), reinterpret_cast<float4*>(sin_out));
+  const cudaError_t err = launch_overlapped(true, rope_table_kernel, grid, kTableThreads, 0,
+                                            static_cast<cudaStream_t>(cuda_stream), p,
+                                            reinterpret_cast<float4*>(cos_out), reinterpret_cast<float4*>(sin_out));
   g_launches.fetch_add(1);
-  return cudaGetLastError() == cudaSuccess ? UNSTEP_OK : UNSTEP_ERR_CUDA;
+  return err == cudaSuccess ? UNSTEP_OK : UNSTEP_ERR_CUDA;
 }
 
 static int rope_kv_append_run(const unstep_shape_t* shape, int32_t sink_frames,
@@ -437,13 +446,13 @@ static int rope_kv_append_run(const unstep_shape_t* shape, int32_t sink_frames,
     const int64_t in_off = static_cast<int64_t>(b0) * p.vec_per_stream;
     const int64_t ring_off = static_cast<int64_t>(b0) * p.ring_vec_per_stream;
     const int64_t tab_off = static_cast<int64_t>(b0) * table_stream_stride;
-    rope_kv_append_kernel<<<dim3(blocks, nb), 256, 0, st>>>(
-        p, static_cast<const uint4*>(q_in) + in_off, static_cast<const uint4*>(k_in) + in_off,
-        static_cast<const uint4*>(v_in) + in_off, reinterpret_cast<const float4*>(cos + tab_off),
+    const cudaError_t err = launch_overlapped(
+        true, rope_kv_append_kernel, dim3(blocks, nb), 256, 0, st, p, static_cast<const uint4*>(q_in) + in_off,
+        static_cast<const uint4*>(k_in) + in_off, static_cast<const uint4*>(v_in) + in_off, reinterpret_cast<const float4*>(cos + tab_off),
         reinterpret_cast<const float4*>(sin + tab_off), static_cast<uint4*>(q_out) + in_off,
         static_cast<uint4*>(ring_k) + ring_off, static_cast<uint4*>(ring_v) + ring_off);
     g_launches.fetch_add(1);
-    if (cudaGetLastError() != cudaSuccess) return UNSTEP_ERR_CUDA;
+    if (err != cudaSuccess) return UNSTEP_ERR_CUDA;
   }
   return UNSTEP_OK;
 }
@@ -526,21 +535,21 @@ extern "C" int unstep_rmsnorm_rope_kv_append(const unstep_shape_t* shape, int32_
       int per_thread = (p.vec_per_token + 95) / 96;
       if (per_thread > 4) per_thread = 4;
       const int threads = (((p.vec_per_token + per_thread - 1) / per_thread) + 31) & ~31;
-      const dim3 grid(static_cast<unsigned>(L), nb);
-      switch (per_thread) {
-        case 1: rmsnorm_rope_kv_append_token_kernel<1><<<grid, threads, 0, st>>>(p, eps, q, k, v, gq, gk, ct, sn, qo, rk, rv); break;
-        case 2: rmsnorm_rope_kv_append_token_kernel<2><<<grid, threads, 0, st>>>(p, eps, q, k, v, gq, gk, ct, sn, qo, rk, rv); break;
-        case 3: rmsnorm_rope_kv_append_token_kernel<3><<<grid, threads, 0, st>>>(p, eps, q, k, v, gq, gk, ct, sn, qo, rk, rv); break;
-        default: rmsnorm_rope_kv_append_token_kernel<4><<<grid, threads, 0, st>>>(p, eps, q, k, v, gq, gk, ct, sn, qo, rk, rv); break;
-      }
+      const auto kernel = per_thread == 1   ? rmsnorm_rope_kv_append_token_kernel<1>
+                          : per_thread == 2 ? rmsnorm_rope_kv_append_token_kernel<2>
+                          : per_thread == 3 ? rmsnorm_rope_kv_append_token_kernel<3>
+                                            : rmsnorm_rope_kv_append_token_kernel<4>;
+      const cudaError_t err = launch_overlapped(true, kernel, dim3(static_cast<unsigned>(L), nb), threads, 0, st, p, eps,
+                                                q, k, v, gq, gk, ct, sn, qo, rk, rv);
       g_launches.fetch_add(1);
-      if (cudaGetLastError() != cudaSuccess) return UNSTEP_ERR_CUDA;
+      if (err != cudaSuccess) return UNSTEP_ERR_CUDA;
       continue;
     }
     // wider tokens: one warp per token
-    rmsnorm_rope_kv_append_kernel<<<dim3(blocks, nb), 256, 0, st>>>(p, eps, q, k, v, gq, gk, ct, sn, qo, rk, rv);
+    const cudaError_t err = launch_overlapped(true, rmsnorm_rope_kv_append_kernel, dim3(blocks, nb), 256, 0, st, p, eps,
+                                              q, k, v, gq, gk, ct, sn, qo, rk, rv);
     g_launches.fetch_add(1);
-    if (cudaGetLastError() != cudaSuccess) return UNSTEP_ERR_CUDA;
+    if (err != cudaSuccess) return UNSTEP_ERR_CUDA;
   }
   return UNSTEP_OK;
 }
