@@ -429,7 +429,6 @@ window_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
         const uint32_t idesc = valid == kTileN ? idesc_qk_full : idesc_bf16_f32(kTileM, (valid + 15) & ~15, 0);
         mma_ss_k128(s_tmem, dq, dk, idesc, 0u);
         tc_commit(my_s_full);
-        tc_commit(bar_kv_empty + 8 * stage);
       };
       auto issue_pv_half = [&](uint64_t dv, int half, int k_steps, bool accumulate) {
         if (k_steps >= 4 * half + 4) {
@@ -460,6 +459,7 @@ window_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
           if (part) {
             tc_fence_after();
             issue_qk(kst, valid);
+            tc_commit(bar_kv_empty + 8 * kst);
             // Q is free as soon as the item's last Q K^T has run: the producer fetches the next
             // item's Q under this item's last exponentials and P V
             if (n == 1) tc_commit(bar_q_empty + 8 * a);
@@ -498,13 +498,17 @@ window_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
               issue_pv_half(dv, 0, k_steps, j > 0);
               issue_pv_half(dv, 1, k_steps, true);
               TRACE(2 + a, sp_it, 4);
-              // the next S first (it is what the softmax warps wait for), the stage releases after it
               if (more) issue_qk(kst, valid);
+            }
+            __syncwarp();
+            // The turn goes on before the commits that release the buffers (90-130 clk each): the other
+            // issuer's first MMA then follows this chain's last without a gap.
+            if (s.nq == 2) turn_pass(a);
+            if (lead && ok) {
+              if (more) tc_commit(bar_kv_empty + 8 * kst);
               if (j + 2 == n) tc_commit(bar_q_empty + 8 * a);
               tc_commit(bar_kv_empty + 8 * vst);
             }
-            __syncwarp();
-            if (s.nq == 2) turn_pass(a);
             TRACE(2 + a, sp_it, 5);
             ++sp_it;
           } else if (lead && ok) {
@@ -578,15 +582,20 @@ window_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
       uint4* const out_v = reinterpret_cast<uint4*>(out);
       const int64_t dst = ((static_cast<int64_t>(s.b) * p.L + n) * p.Hn + s.h) * (kHeadDim / 8);   // 16-byte vectors
       auto store_row = [&](int64_t d, const float* v, float inv_l) {   // 32 columns from vector d on
+        uint32_t w[16];
 #pragma unroll
-        for (int i = 0; i < 4; ++i) {
-          uint4 vv;
-          vv.x = pack_bf16x2(v[8 * i + 0] * inv_l, v[8 * i + 1] * inv_l);
-          vv.y = pack_bf16x2(v[8 * i + 2] * inv_l, v[8 * i + 3] * inv_l);
-          vv.z = pack_bf16x2(v[8 * i + 4] * inv_l, v[8 * i + 5] * inv_l);
-          vv.w = pack_bf16x2(v[8 * i + 6] * inv_l, v[8 * i + 7] * inv_l);
-          UNSTEP_STORE(out_v, d + i, p.extent_out, vv, p.status);
+        for (int i = 0; i < 16; ++i) w[i] = pack_bf16x2(v[2 * i] * inv_l, v[2 * i + 1] * inv_l);
+#ifndef UNSTEP_CHECK
+        if (p.out_wide) {   // whole 32-byte sectors
+          st_global_32(out_v + d, w);
+          st_global_32(out_v + d + 2, w + 8);
+          return;
         }
+#endif
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+          UNSTEP_STORE(out_v, d + i, p.extent_out, make_uint4(w[4 * i], w[4 * i + 1], w[4 * i + 2], w[4 * i + 3]),
+                       p.status);
       };
       if (whole) {
         // O / l -> bf16 -> out[b][n][h][:]: a thread writes its whole 256-byte row
@@ -648,23 +657,28 @@ window_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
           __threadfence();   // acquire side for every thread that reads the other parts below
           if (row == 0) UNSTEP_STORE(p.counters, 2 * s.item + a, p.extent_counters, 0, p.status);   // ready for the next launch
           const int me = static_cast<int>(blockIdx.x);
+          const int lo_slot = part_slot(p, c_lo, s.item_step0);   // every later part starts its worker's range
           auto part_of = [&](int c) -> const float* {
-            return p.part + (static_cast<int64_t>(2 * c + part_slot(p, c, s.item_step0)) * kPartFloats +
-                             a * kPartTileFloats);
+            return p.part + (static_cast<int64_t>(2 * c + (c == c_lo ? lo_slot : 0)) * kPartFloats + a * kPartTileFloats);
           };
           auto ml_of = [&](int c) -> float2 {
             return c == me ? make_float2(m_run, l_run)
                            : __ldcg(reinterpret_cast<const float2*>(part_of(c) + 128 * 128) + row);
           };
           float m_all = m_run, l_sum = 0.f;
-          if (others == 1) {   // the common case: one round trip
-            const float2 x = ml_of(c_lo), y = ml_of(c_hi);
-            m_all = fmaxf(x.x, y.x);
-            l_sum = x.y * ex2((x.x - m_all) * p.scale_log2e) + y.y * ex2((y.x - m_all) * p.scale_log2e);
+          if (others <= 3) {   // one round trip for all parts
+            float2 x[4];
+#pragma unroll
+            for (int i = 0; i < 4; ++i) x[i] = i <= others ? ml_of(c_lo + i) : make_float2(-INFINITY, 0.f);
+#pragma unroll
+            for (int i = 0; i < 4; ++i) m_all = fmaxf(m_all, x[i].x);
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+              if (i <= others) l_sum += x[i].y * ex2((x[i].x - m_all) * p.scale_log2e);
           } else {
-#pragma unroll 2
+#pragma unroll 4
             for (int c = c_lo; c <= c_hi; ++c) m_all = fmaxf(m_all, ml_of(c).x);
-#pragma unroll 2
+#pragma unroll 4
             for (int c = c_lo; c <= c_hi; ++c) {
               const float2 x = ml_of(c);
               l_sum += x.y * ex2((x.x - m_all) * p.scale_log2e);
@@ -916,6 +930,7 @@ static int window_attn_run(const unstep_shape_t* shape, const int32_t* start_fra
     p.part = ws.part;
     p.counters = ws.counters;
     p.status = status_word();
+    p.out_wide = (reinterpret_cast<uintptr_t>(out) & 31u) == 0;   // rows are multiples of 256 bytes
     p.extent_out = static_cast<int64_t>(nb) * p.L * p.Hn * (kHeadDim / 8);
     p.extent_part = static_cast<int64_t>(ws.slots) * kPartFloats;
     p.extent_counters = static_cast<int64_t>(ws.n_counters);

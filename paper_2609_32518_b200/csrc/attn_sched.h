@@ -36,10 +36,12 @@ struct AttnParams {
   int32_t parts;            // > 0: every item of the remainder is cut into this many parts, one per worker
   int32_t n_active;         // parts == 0: workers that take a share of the remainder, >= 1
   int64_t all_steps;        // key tiles of all items of the launch
+  int32_t narrow;           // 1: total_steps * n_active fits 32 bits, and so does every index of the split
   int64_t total_steps;      // remainder: sum over the leftover items of their key tiles
   float* part;              // workspace: partial results of split items, kPartFloats per slot
   int* counters;            // workspace: arrivals per (item, query tile), zero between launches
   int* status;              // status word; with the extents below, for checking builds
+  int32_t out_wide;         // 1: `out` is 32-byte aligned
   int64_t extent_out;       // 16-byte vectors of `out` that belong to this launch's streams
   int64_t extent_part;      // floats of `part`
   int64_t extent_counters;  // ints of `counters`
@@ -123,11 +125,17 @@ struct Sched {
   int b_round, round;   // position in the whole rounds
   int me;
   const AttnParams& p;
+  // (a * b) / c; a 64-bit division takes several hundred clk, a chain of them was 2 us of the
+  // epilogue of every part
+  UNSTEP_HD static int64_t mul_div(const AttnParams& p, int64_t a, int64_t b, int64_t c) {
+    if (p.narrow) return static_cast<uint32_t>(a) * static_cast<uint32_t>(b) / static_cast<uint32_t>(c);
+    return a * b / c;
+  }
   UNSTEP_HD static int64_t worker_lo(const AttnParams& p, int64_t c) {
-    return c >= p.n_active ? p.total_steps : p.total_steps * c / p.n_active;
+    return c >= p.n_active ? p.total_steps : mul_div(p, p.total_steps, c, p.n_active);
   }
   UNSTEP_HD static int worker_of(const AttnParams& p, int64_t step) {
-    int64_t c = step * p.n_active / p.total_steps;
+    int64_t c = mul_div(p, step, p.n_active, p.total_steps);
     while (c + 1 < p.n_active && worker_lo(p, c + 1) <= step) ++c;
     while (c > 0 && worker_lo(p, c) > step) --c;
     return static_cast<int>(c);
@@ -182,7 +190,7 @@ struct Sched {
     while (b + 1 < p.n_streams && p.step_base[b + 1] <= cur) ++b;
     const int tiles = p.tiles[b];
     const int64_t rel = cur - p.step_base[b];
-    const int left_item = static_cast<int>(rel / tiles);
+    const int left_item = static_cast<int>(mul_div(p, rel, 1, tiles));
     decode(s, b, p.full_rounds * p.n_workers + left_item);
     s.t0 = static_cast<int>(rel - static_cast<int64_t>(left_item) * tiles);
     const int64_t left = hi - cur;
@@ -289,9 +297,11 @@ inline int plan_launch(AttnParams& p, const unstep_shape_t* shape, const int32_t
   p.total_steps = steps;
   p.parts = 0;
   p.n_active = 1;
+  p.narrow = 1;
   if (steps > 0) {
     const int64_t items = static_cast<int64_t>(nb) * p.leftover;
     p.parts = remainder_parts(items, steps, least, most, max_workers, &p.n_active);
+    p.narrow = steps * p.n_active <= INT32_MAX;
     if (p.full_rounds == 0) p.n_workers = p.parts > 0 ? static_cast<int32_t>(items) * p.parts : p.n_active;
   }
   return UNSTEP_OK;

@@ -113,3 +113,26 @@ def test_launches_smaller_than_the_grid_cut_every_item_into_equal_parts():
         assert len(segs) == 1 + max(s[0] for s in segs)   # one segment per worker
         for s in segs:
             assert abs((s[6] - s[5]) - s[7] / parts) < 1
+
+
+def test_split_of_more_steps_than_32_bit_products_hold():
+    # 32 items of 8.4 million key tiles: shares across items in 64-bit arithmetic
+    frames = 262143
+    sh = U.Shape.make(batch=1, heads=2, chunk_frames=1, grid_h=64, grid_w=64, ring_frames=frames)
+    segs = U.window_attn_plan(sh, [frames - 1], frames, 148)
+    tiles = frames * 64 * 64 // 128
+    items = {}
+    for (w, b, h, qp, nq, t0, t1, n, parts, slot) in segs:
+        assert n == tiles and 0 <= t0 < t1 <= tiles
+        items.setdefault((h, qp), []).append((t0, t1, w, parts))
+    assert len(items) == 2 * 16
+    total = len(items) * tiles
+    for spans in items.values():
+        spans.sort()
+        assert [s[0] for s in spans] == [0] + [s[1] for s in spans[:-1]] and spans[-1][1] == tiles
+        assert all(s[3] == len(spans) for s in spans)
+        assert [s[2] for s in spans] == list(range(spans[0][2], spans[0][2] + len(spans)))
+    work = {}
+    for s in segs:
+        work[s[0]] = work.get(s[0], 0) + s[6] - s[5]
+    assert len(work) == 148 and max(work.values()) - min(work.values()) <= 1 and sum(work.values()) == total
