@@ -369,21 +369,24 @@ window_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
       uint32_t kv_it = 0, q_it[2] = {0, 0};
       bool ok = true;
       while (ok && sched.next(s)) {
-        for (int a = 0; a < s.nq && ok; ++a) {
+        auto load_q = [&](int a) {
+          if (!ok || a >= s.nq) return;
           ok = w.wait(bar_q_empty + 8 * a, (q_it[a] & 1) ^ 1);
-          if (!ok) break;
+          if (!ok) return;
           const uint32_t dst = sQ + a * kTileBytes, bar = bar_q_full + 8 * a;
           const int n0 = (2 * s.qp + a) * kTileM;
           mbar_expect_tx(bar, kTileBytes);
           tma_load_4d(dst, &tm_q, bar, 0, s.h, n0, s.b);
           tma_load_4d(dst + kHalfBytes, &tm_q, bar, 64, s.h, n0, s.b);
           ++q_it[a];
-        }
+        };
+        load_q(0);   // what the first S needs comes first: Q of tile 0, then K
         for (int j = s.t0; j < s.t1 && ok; ++j) {
           const TileInfo ti = tile_info(p, s.b, j);
           for (int kv = 0; kv < 2 && ok; ++kv) {
+            if (j == s.t0 && kv == 1) load_q(1);
             const uint32_t st = kv_it % kStages;
-            ok = w.wait(bar_kv_empty + 8 * st, ((kv_it / kStages) & 1) ^ 1);
+            if (ok) ok = w.wait(bar_kv_empty + 8 * st, ((kv_it / kStages) & 1) ^ 1);
             if (!ok) break;
             const uint32_t dst = sKV + st * kTileBytes, bar = bar_kv_full + 8 * st;
             mbar_expect_tx(bar, kTileBytes);
