@@ -179,7 +179,7 @@ __device__ __forceinline__ void mask_block32(uint32_t* s, int col0, int nvalid) 
 // exponentiated (a block keeps the MUFU pipe busy for 256 clk, longer than a TMEM load takes), so
 // that only the first block's load is exposed.  Leaves P (bf16 pairs) in p0 (keys 0..63) and p1
 // (keys 64..127) and returns the row's sum of P.
-template <bool kMasked>
+template <bool kMasked, int kCols>
 __device__ __forceinline__ float exp_row(uint32_t t_S, float c, float neg_ms, int nvalid, uint32_t* p0,
                                          uint32_t* p1) {
   const uint64_t c2 = pack_f32x2(c, c);
@@ -192,16 +192,18 @@ __device__ __forceinline__ float exp_row(uint32_t t_S, float c, float neg_ms, in
   mask_block32<kMasked>(a, 0, nvalid);
   exp_block32(a, p0, c2, nm2, acc);
   tc_wait_ld32(b);
-  tmem_ld32(t_S + 64, a);
+  if (kCols > 64) tmem_ld32(t_S + 64, a);
   mask_block32<kMasked>(b, 32, nvalid);
   exp_block32(b, p0 + 16, c2, nm2, acc);
-  tc_wait_ld32(a);
-  tmem_ld32(t_S + 96, b);
-  mask_block32<kMasked>(a, 64, nvalid);
-  exp_block32(a, p1, c2, nm2, acc);
-  tc_wait_ld32(b);
-  mask_block32<kMasked>(b, 96, nvalid);
-  exp_block32(b, p1 + 16, c2, nm2, acc);
+  if (kCols > 64) {
+    tc_wait_ld32(a);
+    tmem_ld32(t_S + 96, b);
+    mask_block32<kMasked>(a, 64, nvalid);
+    exp_block32(a, p1, c2, nm2, acc);
+    tc_wait_ld32(b);
+    mask_block32<kMasked>(b, 96, nvalid);
+    exp_block32(b, p1 + 16, c2, nm2, acc);
+  }
   const uint64_t t = add_f32x2(add_f32x2(acc[0], acc[1]), add_f32x2(acc[2], acc[3]));
   float t0, t1;
   unpack_f32x2(t, t0, t1);
@@ -209,54 +211,75 @@ __device__ __forceinline__ float exp_row(uint32_t t_S, float c, float neg_ms, in
 }
 
 // Row maximum of the 128 scores in TMEM.
-template <bool kMasked>
+template <bool kMasked, int kCols>
 __device__ __forceinline__ float max_row(uint32_t t_S, int nvalid) {
   uint32_t hi[64], lo[64];
-  tmem_ld32(t_S + 64, hi);
-  tmem_ld32(t_S + 96, hi + 32);
+  if (kCols > 64) {
+    tmem_ld32(t_S + 64, hi);
+    tmem_ld32(t_S + 96, hi + 32);
+  }
   tmem_ld32(t_S, lo);
   tmem_ld32(t_S + 32, lo + 32);
-  tc_wait_ld32(hi);
-  reg_fence32(hi + 32);
-  reg_fence32(lo);
+  tc_wait_ld32(lo);
   reg_fence32(lo + 32);
-  mask_block32<kMasked>(hi, 64, nvalid);
-  mask_block32<kMasked>(hi + 32, 96, nvalid);
   mask_block32<kMasked>(lo, 0, nvalid);
   mask_block32<kMasked>(lo + 32, 32, nvalid);
-  return fmaxf(fmaxf(max_block32(hi), max_block32(hi + 32)), fmaxf(max_block32(lo), max_block32(lo + 32)));
+  float m = fmaxf(max_block32(lo), max_block32(lo + 32));
+  if (kCols > 64) {
+    reg_fence32(hi);
+    reg_fence32(hi + 32);
+    mask_block32<kMasked>(hi, 64, nvalid);
+    mask_block32<kMasked>(hi + 32, 96, nvalid);
+    m = fmaxf(m, fmaxf(max_block32(hi), max_block32(hi + 32)));
+  }
+  return m;
 }
 
-// Only the first key tile of a segment looks for the row maximum before its exponentials.
-// Every later tile exponentiates against that reference straight away and looks at the row's sum
-// of P afterwards.  P is positive, so a sum of at most kOptimisticLimit = 2^64 means that no
-// score was more than 64 (log2 units) above the reference: P (bf16) and the float32 sums are as
-// accurate at that magnitude as near 1 (same relative precision, no overflow: 128 keys of 2^64
-// times |v| stay far below 2^127), and everything accumulated before such a jump is negligible
-// exactly as in the true softmax.  Otherwise (scores more than 64 above the first tile's maximum,
-// or an overflow to inf) the warp finds the tile's true maximum, rescales O and l, and redoes
-// the exponentials; the scores are still in TMEM, because P is only stored at the very end.
-// Scores are read from TMEM in blocks to keep the register count down; P (bf16 pairs)
-// overwrites score columns 0..63.
+// Only the first key tile of a segment looks for a reference before its exponentials, the maximum of
+// its first 32 scores (the whole row's would take another 350 clk a segment and is not needed: first
+// chunk of the 1.3B class 160.3 -> 158.8 us).  Every tile exponentiates against that reference straight
+// away and looks at the row's sum of P afterwards.  P is positive, so a sum of at most
+// kOptimisticLimit = 2^64 means that no score was more than 64 (log2 units) above the reference: P
+// (bf16) and the float32 sums are as accurate at that magnitude as near 1 (same relative precision, no
+// overflow: 128 keys of 2^64 times |v| stay far below 2^127), and everything accumulated before such a
+// jump is negligible exactly as in the true softmax.  Otherwise (scores more than 64 above the
+// reference, or an overflow to inf) the warp finds the tile's true maximum, rescales O and l, and
+// redoes the exponentials; the scores are still in TMEM, because P is only stored at the very end.
+// Scores are read from TMEM in blocks to keep the register count down; P (bf16 pairs) overwrites
+// score columns 0..63.  Tiles of at most 64 keys (frames of up to 64 tokens, the end of a run) leave the
+// other half of the columns alone: append and attention of a toy layer with 64-token frames 16.1 ->
+// 14.7 us.  The redo is the second round of a loop, so that each variant holds its exponentials once.
 constexpr float kOptimisticLimit = 18446744073709551616.f;   // 2^64
 
-template <bool kMasked>
+template <bool kMasked, int kCols>   // kCols: score columns that hold keys, 64 or 128
 __device__ __forceinline__ void softmax_row_tile(uint32_t t_S, uint32_t t_O, float c, int nvalid,
                                                  bool first, float& m_run, float& l_run,
                                                  int a, int trace_role, int trace_tile) {
-  if (first) m_run = max_row<kMasked>(t_S, nvalid);
+  if (first) {
+    uint32_t s[32];
+    tmem_ld32(t_S, s);
+    tc_wait_ld32(s);
+    mask_block32<kMasked>(s, 0, nvalid);
+    m_run = max_block32(s);
+  }
   TRACE(trace_role, trace_tile, 2);
   uint32_t p0[32], p1[32];
-  float sum = exp_row<kMasked>(t_S, c, -m_run * c, nvalid, p0, p1);
-  const bool redo = !first && !(sum <= kOptimisticLimit);   // also taken for inf and NaN
-  if (__any_sync(0xFFFFFFFFu, redo)) {
-    const float mx = max_row<kMasked>(t_S, nvalid);
+  float sum;
+  bool redone = false;
+#pragma unroll 1
+  for (;;) {   // at most twice
+    sum = exp_row<kMasked, kCols>(t_S, c, -m_run * c, nvalid, p0, p1);
+    const bool redo = !(sum <= kOptimisticLimit);   // also taken for inf and NaN
+    if (redone || !__any_sync(0xFFFFFFFFu, redo)) break;
+    redone = true;
+    const float mx = max_row<kMasked, kCols>(t_S, nvalid);
     float alpha = 1.f;
     if (mx > m_run) {
       alpha = ex2((m_run - mx) * c);
       m_run = mx;
       l_run *= alpha;
     }
+    // (on the first tile O is not valid yet; its P V overwrites it)
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
       uint32_t o[32];
@@ -266,10 +289,9 @@ __device__ __forceinline__ void softmax_row_tile(uint32_t t_S, uint32_t t_O, flo
       for (int i = 0; i < 32; ++i) o[i] = __float_as_uint(__uint_as_float(o[i]) * alpha);
       tmem_st32(t_O + q * 32, o);
     }
-    sum = exp_row<kMasked>(t_S, c, -m_run * c, nvalid, p0, p1);
   }
   tmem_st32(t_S, p0);        // P of keys 0..63 over score columns 0..31
-  tmem_st32(t_S + 32, p1);   // P of keys 64..127 over score columns 32..63
+  if (kCols > 64) tmem_st32(t_S + 32, p1);   // P of keys 64..127 over score columns 32..63
   tc_wait_st();
   tc_fence_before();
   p_ready_arrive(a);
@@ -558,10 +580,12 @@ window_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
         tc_fence_after();
         if (it == 0) CTRACE(2);
         TRACE(a, it, 1);
-        if (valid < kTileN)
-          softmax_row_tile<true>(t_S, t_O, p.scale_log2e, valid, j == s.t0, m_run, l_run, a, a, it);
+        if (valid <= 64)   // frames of at most half a tile, and the end of a run
+          softmax_row_tile<true, 64>(t_S, t_O, p.scale_log2e, valid, j == s.t0, m_run, l_run, a, a, it);
+        else if (valid < kTileN)
+          softmax_row_tile<true, kTileN>(t_S, t_O, p.scale_log2e, valid, j == s.t0, m_run, l_run, a, a, it);
         else
-          softmax_row_tile<false>(t_S, t_O, p.scale_log2e, kTileN, j == s.t0, m_run, l_run, a, a, it);
+          softmax_row_tile<false, kTileN>(t_S, t_O, p.scale_log2e, kTileN, j == s.t0, m_run, l_run, a, a, it);
         ++it;
       }
       CTRACE(8 + seg_no);

@@ -282,3 +282,33 @@ def test_items_cut_into_equal_parts(batch, heads, grid, fc, ring, win, history, 
     wl = W.Workload("parts", sh, seed=31, history_starts=history, measured_starts=starts, window_frames=(win,),
                     k_scale=4.0)
     run(wl)
+
+
+@pytest.mark.parametrize("grid,fc,ring,history,start,keys", [
+    ((8, 8), 2, 6, (0, 2), 4, (33, 63)),               # tiles of 64 keys: past the first 32 of a tile
+    ((8, 8), 2, 6, (0, 2), 4, (31,)),                  # the last key that the reference sees
+    ((10, 20), 1, 3, (0, 1), 2, (32, 100, 127)),       # full first tile
+    ((10, 20), 1, 3, (0, 1), 2, (128 + 40,)),          # second tile (flat)
+    ((10, 20), 1, 3, (0, 1), 2, (3 * 200 - 1,)),       # ragged last tile: 600 = 4 x 128 + 88
+    ((12, 15), 1, 3, (0, 1), 2, (3 * 180 - 1,)),       # ragged last tile of at most 64: 540 = 4 x 128 + 28
+    ((9, 14), 1, 4, (0, 1, 2), 3, (32, 125)),          # frames just below a tile
+])
+def test_keys_far_above_the_reference_wherever_they_sit(grid, fc, ring, history, start, keys):
+    # The reference of a segment is the maximum of the first 32 scores of its first tile.  Single keys
+    # 256 times larger score hundreds of log2 units above it (for about half of the rows).
+    sh = W.Shape(batch=1, heads=2, chunk_frames=fc, grid_h=grid[0], grid_w=grid[1], ring_frames=ring)
+    wl = W.Workload("far_keys", sh, seed=32, history_starts=(history,), measured_starts=(start,), window_frames=(ring,))
+    T = sh.tokens_per_frame
+    dev, ora = DevicePath(sh), OraclePath(sh)
+    q_dev = q_ref = None
+    for first in (*history, start):
+        q, k, v = W.batch_qkv(wl, [first])
+        k = k.copy()
+        for key in keys:
+            n = key - first * T
+            if 0 <= n < k.shape[1]:
+                k[:, n] = W.f32_to_bf16_bits(W.bf16_bits_to_f32(k[:, n]) * np.float32(256.0))
+        q_dev, q_ref = dev.append([first], q, k, v), ora.append([first], q, k, v)
+    assert np.array_equal(to_bits(q_dev), q_ref)
+    check(to_bits(dev.attend([start], ring, q_dev)), ora.attend([start], ring, q_ref), f"keys {keys}")
+    assert U.poll_status() == 0
