@@ -117,7 +117,23 @@ struct AppendParams {
   int32_t start[kMaxStreamsPerLaunch];  // start_frame[b]
   int* status;                     // status word and extents (16-byte vectors) of q_out and of the cache
   int64_t extent_act, extent_cache;     // of this launch's streams, for checking builds
+  int32_t prefetch;                // 1: the first blocks prefetch their inputs to L2
 };
+
+// A block that is set up while the kernel before it finishes has DRAM bring its inputs to L2 meanwhile.
+// The prefetch reads nothing: L2 is where that kernel's stores become visible, and the loads behind
+// grid_wait() find whatever is there by then.  Only the blocks that fit the GPU at once can be early,
+// and only launches of up to 64 MB of inputs ask for it: the append behind the norm of 4680 tokens x 12
+// heads (43 MB of inputs) 17.8 -> 16.6 us, the plain one in front of 4680 keys' attention 157.4 -> 156.9
+// with it; four streams (172 MB) 55.5 -> 55.8, so that they do without.
+constexpr int64_t kPrefetchVectors = (int64_t{64} << 20) / 16;
+constexpr int kEarlyBlocks = 2048;
+__device__ __forceinline__ bool early_block(const AppendParams& p) {
+  return threadIdx.x == 0 && p.prefetch && blockIdx.y * gridDim.x + blockIdx.x < kEarlyBlocks;
+}
+__device__ __forceinline__ void prefetch_l2(const uint4* p, int vectors) {
+  asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(p), "r"(vectors * 16) : "memory");
+}
 
 __device__ __forceinline__ uint32_t rotate_pair(uint32_t w, float c, float s) {
   const float xe = __uint_as_float(w << 16);
@@ -144,9 +160,17 @@ rope_kv_append_kernel(AppendParams p, const uint4* q_in, const uint4* __restrict
                       const float4* __restrict__ sin_t, uint4* q_out,
                       uint4* __restrict__ ring_k, uint4* __restrict__ ring_v) {
   grid_launch_next();
-  grid_wait();
   const int b = blockIdx.y;
   const int64_t v = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
+  if (early_block(p)) {
+    const int64_t first = static_cast<int64_t>(b) * p.vec_per_stream + v;
+    const int64_t left = p.vec_per_stream - v;
+    const int n = left < blockDim.x ? static_cast<int>(left) : static_cast<int>(blockDim.x);
+    prefetch_l2(q_in + first, n);
+    prefetch_l2(k_in + first, n);
+    prefetch_l2(v_in + first, n);
+  }
+  grid_wait();
   if (v >= p.vec_per_stream) return;
   const int n = static_cast<int>(v / p.vec_per_token);
   const int rem = static_cast<int>(v - static_cast<int64_t>(n) * p.vec_per_token);
@@ -310,7 +334,6 @@ rmsnorm_rope_kv_append_token_kernel(AppendParams p, float eps, const uint4* q_in
                                     uint4* __restrict__ ring_v) {
   __shared__ double part[2][8];
   grid_launch_next();
-  grid_wait();
   const int b = blockIdx.y;
   const int n = blockIdx.x;   // token
   const int tid = threadIdx.x, nthr = blockDim.x;
@@ -323,6 +346,12 @@ rmsnorm_rope_kv_append_token_kernel(AppendParams p, float eps, const uint4* q_in
   const int64_t tab_base = (static_cast<int64_t>(b) * p.table_stream_stride >> 2) +
                            static_cast<int64_t>(n) * (kPairs / 4);
 
+  if (early_block(p)) {
+    prefetch_l2(q_in + in_base, p.vec_per_token);
+    prefetch_l2(k_in + in_base, p.vec_per_token);
+    prefetch_l2(v_in + in_base, p.vec_per_token);
+  }
+  grid_wait();
   uint4 xq[kU], xk[kU], xv[kU];
 #pragma unroll
   for (int u = 0; u < kU; ++u) {
@@ -442,6 +471,7 @@ static int rope_kv_append_run(const unstep_shape_t* shape, int32_t sink_frames,
     for (int i = 0; i < nb; ++i) p.start[i] = start_frame[b0 + i];
     p.status = status_word();
     p.extent_act = nb * p.vec_per_stream;
+    p.prefetch = 3 * p.extent_act <= kPrefetchVectors;
     p.extent_cache = nb * p.ring_vec_per_stream;
     const int64_t in_off = static_cast<int64_t>(b0) * p.vec_per_stream;
     const int64_t ring_off = static_cast<int64_t>(b0) * p.ring_vec_per_stream;
@@ -514,6 +544,7 @@ extern "C" int unstep_rmsnorm_rope_kv_append(const unstep_shape_t* shape, int32_
     for (int i = 0; i < nb; ++i) p.start[i] = start_frame[b0 + i];
     p.status = status_word();
     p.extent_act = nb * p.vec_per_stream;
+    p.prefetch = 3 * p.extent_act <= kPrefetchVectors;
     p.extent_cache = nb * p.ring_vec_per_stream;
     const int64_t in_off = static_cast<int64_t>(b0) * p.vec_per_stream;
     const int64_t ring_off = static_cast<int64_t>(b0) * p.ring_vec_per_stream;
