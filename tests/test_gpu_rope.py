@@ -43,6 +43,21 @@ def test_table_matches_oracle_within_one_ulp(grid, fc, start):
         assert (gc[0] == 1.0).all() and (gs[0] == 0.0).all()
 
 
+@pytest.mark.parametrize("grid,fc,bands", [((1, 1), 1, (44, 42, 42)), ((7, 9), 2, (44, 42, 42)),
+                                           ((9, 8), 1, (2, 124, 2)), ((16, 17), 3, (124, 2, 2)),
+                                           ((8, 63), 1, (2, 2, 124)), ((2100, 1), 1, (44, 42, 42))])
+def test_table_at_the_edges_of_its_tiles_and_with_other_bands(grid, fc, bands):
+    # tiles of 8 x 8 tokens, 384 threads: whole tiles, remainders of 1 and 7, bands of one and of 62 pairs
+    sh = U.Shape.make(1, 1, fc, grid[0], grid[1], fc, bands=bands, rope_base=500.0)
+    cos = torch.full((sh.chunk_tokens, 64), float("nan"), dtype=torch.float32, device="cuda")
+    sin = torch.full_like(cos, float("nan"))
+    U.rope_table(sh, 5, cos, sin)
+    for got, want in zip((cos, sin), O.rope_table(5, fc, grid[0], grid[1], bands, 500.0)):
+        g = got.cpu().numpy()
+        close = (ulp_diff(g, want) <= 1) | (np.abs(g.astype(np.float64) - want.astype(np.float64)) < 1e-12)
+        assert close.all()
+
+
 def test_cfg1_append_bit_exact_and_sentinels():
     wl = W.WORKLOADS["cfg1"]
     dev, ora = DevicePath(wl.shape), OraclePath(wl.shape)
