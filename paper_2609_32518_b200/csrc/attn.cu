@@ -235,15 +235,16 @@ __device__ __forceinline__ float max_row(uint32_t t_S, int nvalid) {
   return m;
 }
 
-// Only the first key tile of a segment looks for a reference before its exponentials, the maximum of
-// its first 32 scores (the whole row's would take another 350 clk a segment and is not needed: first
-// chunk of the 1.3B class 160.3 -> 158.8 us).  Every tile exponentiates against that reference straight
-// away and looks at the row's sum of P afterwards.  P is positive, so a sum of at most
+// Only the first key tile of a segment looks for the row maximum before its exponentials.
+// (The maximum of 32 scores would do as a reference and saves 350 clk a segment, but then the largest
+// weight is no longer exactly 1 and rounds to bf16 like the others: against float64 the error of
+// peaked rows grew from 2.17e-3 to 2.32e-3.)  Every later tile exponentiates against that reference
+// straight away and looks at the row's sum of P afterwards.  P is positive, so a sum of at most
 // kOptimisticLimit = 2^64 means that no score was more than 64 (log2 units) above the reference: P
 // (bf16) and the float32 sums are as accurate at that magnitude as near 1 (same relative precision, no
 // overflow: 128 keys of 2^64 times |v| stay far below 2^127), and everything accumulated before such a
-// jump is negligible exactly as in the true softmax.  Otherwise (scores more than 64 above the
-// reference, or an overflow to inf) the warp finds the tile's true maximum, rescales O and l, and
+// jump is negligible exactly as in the true softmax.  Otherwise (scores more than 64 above the first
+// tile's maximum, or an overflow to inf) the warp finds the tile's true maximum, rescales O and l, and
 // redoes the exponentials; the scores are still in TMEM, because P is only stored at the very end.
 // Scores are read from TMEM in blocks to keep the register count down; P (bf16 pairs) overwrites
 // score columns 0..63.  Tiles of at most 64 keys (frames of up to 64 tokens, the end of a run) leave the
@@ -255,13 +256,7 @@ template <bool kMasked, int kCols>   // kCols: score columns that hold keys, 64 
 __device__ __forceinline__ void softmax_row_tile(uint32_t t_S, uint32_t t_O, float c, int nvalid,
                                                  bool first, float& m_run, float& l_run,
                                                  int a, int trace_role, int trace_tile) {
-  if (first) {
-    uint32_t s[32];
-    tmem_ld32(t_S, s);
-    tc_wait_ld32(s);
-    mask_block32<kMasked>(s, 0, nvalid);
-    m_run = max_block32(s);
-  }
+  if (first) m_run = max_row<kMasked, kCols>(t_S, nvalid);
   TRACE(trace_role, trace_tile, 2);
   uint32_t p0[32], p1[32];
   float sum;
@@ -269,7 +264,7 @@ __device__ __forceinline__ void softmax_row_tile(uint32_t t_S, uint32_t t_O, flo
 #pragma unroll 1
   for (;;) {   // at most twice
     sum = exp_row<kMasked, kCols>(t_S, c, -m_run * c, nvalid, p0, p1);
-    const bool redo = !(sum <= kOptimisticLimit);   // also taken for inf and NaN
+    const bool redo = !first && !(sum <= kOptimisticLimit);   // also taken for inf and NaN
     if (redone || !__any_sync(0xFFFFFFFFu, redo)) break;
     redone = true;
     const float mx = max_row<kMasked, kCols>(t_S, nvalid);
@@ -279,7 +274,6 @@ __device__ __forceinline__ void softmax_row_tile(uint32_t t_S, uint32_t t_O, flo
       m_run = mx;
       l_run *= alpha;
     }
-    // (on the first tile O is not valid yet; its P V overwrites it)
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
       uint32_t o[32];

@@ -286,7 +286,7 @@ def test_items_cut_into_equal_parts(batch, heads, grid, fc, ring, win, history, 
 
 @pytest.mark.parametrize("grid,fc,ring,history,start,keys", [
     ((8, 8), 2, 6, (0, 2), 4, (33, 63)),               # tiles of 64 keys: past the first 32 of a tile
-    ((8, 8), 2, 6, (0, 2), 4, (31,)),                  # the last key that the reference sees
+    ((8, 8), 2, 6, (0, 2), 4, (31, 64 + 40)),          # and in the tile behind it
     ((10, 20), 1, 3, (0, 1), 2, (32, 100, 127)),       # full first tile
     ((10, 20), 1, 3, (0, 1), 2, (128 + 40,)),          # second tile (flat)
     ((10, 20), 1, 3, (0, 1), 2, (3 * 200 - 1,)),       # ragged last tile: 600 = 4 x 128 + 88
@@ -294,8 +294,9 @@ def test_items_cut_into_equal_parts(batch, heads, grid, fc, ring, win, history, 
     ((9, 14), 1, 4, (0, 1, 2), 3, (32, 125)),          # frames just below a tile
 ])
 def test_keys_far_above_the_reference_wherever_they_sit(grid, fc, ring, history, start, keys):
-    # The reference of a segment is the maximum of the first 32 scores of its first tile.  Single keys
-    # 256 times larger score hundreds of log2 units above it (for about half of the rows).
+    # The reference of a segment is the maximum of its first tile.  Single keys 256 times larger score
+    # hundreds of log2 units above the others (for about half of the rows): in the first tile they must
+    # be found, in a later one the tile must be redone, in tiles of up to 64 keys and in full ones.
     sh = W.Shape(batch=1, heads=2, chunk_frames=fc, grid_h=grid[0], grid_w=grid[1], ring_frames=ring)
     wl = W.Workload("far_keys", sh, seed=32, history_starts=(history,), measured_starts=(start,), window_frames=(ring,))
     T = sh.tokens_per_frame
