@@ -973,8 +973,8 @@ static int window_attn_run(const unstep_shape_t* shape, const int32_t* start_fra
       return UNSTEP_ERR_CUDA;
     // Set up under the append before it where the launch is short: five heads and two streams
     // 36 -> 32 us with the append, 57 steps per worker 166.7 -> 164.7 us.  Long launches run at the
-    // power cap, where the saved 2 us of idling show as a lower clock: 256 key tiles and 133 steps
-    // per worker took 898 us overlapped and 886 not, four layers of 64 steps 1609 and 1601.
+    // power cap, where the saved 2 us of idling show as a lower clock: 394 steps per worker took 898 us
+    // overlapped and 886 not, six layers of 171 steps 2473 and 2411.
     const bool brief = p.all_steps < static_cast<int64_t>(kOverlapSteps) * p.n_workers;
     const cudaError_t err = launch_overlapped(brief, window_attn_kernel, p.n_workers, kThreads, kAttnSmemBytes, st, tm_q,
                                               tm_k, tm_v, tm_kf, tm_vf, p, ob);

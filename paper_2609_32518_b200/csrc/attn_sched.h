@@ -221,8 +221,8 @@ UNSTEP_HD int part_slot(const AttnParams& p, int c, int64_t item_step0) {
 // after the other, each with a hand-over, and an item falls into more parts.  The estimates (us)
 // are fitted to launches of 2 to 40 items of 6 to 85 key tiles on a B200: a step 1.6; a second part
 // 3.4, each further one 1.6; shares 6 and 2.2 for each part of an item.  Measured, us: 8 items x 43
-// steps 85 whole, 5 parts 38, 8 parts 39, 86 shares of 4 steps 44; 40 items x 16 steps 38 whole, 3
-// parts 30, 148 shares 44; 80 items x 37 steps behind a whole round: shares, 140 against 160 whole.
+// steps 82 whole, 5 parts 33, 6 parts 31, 8 parts 33, 86 shares of 4 steps 35; 40 items x 16 steps 35
+// whole, 3 parts 25, 148 shares 36; 80 items x 37 steps behind a whole round: shares.
 inline int32_t remainder_parts(int64_t items, int64_t steps, int32_t least, int32_t most, int max_workers,
                                int32_t* shares) {
   int64_t n = steps / kMinStepsPerWorker;
