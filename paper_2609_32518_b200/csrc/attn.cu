@@ -28,6 +28,7 @@
 #include "common.h"
 #include "ptx.cuh"
 #include "attn_sched.h"
+#include "handover.h"
 
 namespace unstep {
 
@@ -120,30 +121,35 @@ __device__ __forceinline__ void reg_alloc_softmax() { asm volatile("setmaxnreg.i
 // rescaled here without another wait.
 // --------------------------------------------------------------------------------------
 __device__ __forceinline__ void group_barrier(int a) {
-  if (a == 0) asm volatile("bar.sync 1, 128;" ::: "memory");
-  else asm volatile("bar.sync 2, 128;" ::: "memory");
+  asm volatile("bar.sync %0, 128;" ::"r"(kGroupBarrier + a) : "memory");
+}
+// The group barrier that also counts the threads with a true predicate: the same answer in every
+// thread, with nothing in memory that a warp ahead of the others could overwrite.
+__device__ __forceinline__ uint32_t group_count(int a, bool pred) {
+  uint32_t n;
+  asm volatile("{\n.reg .pred q;\nsetp.ne.u32 q, %2, 0;\nbar.red.popc.u32 %0, %1, 128, q;\n}"
+               : "=r"(n) : "r"(kGroupBarrier + a), "r"(static_cast<uint32_t>(pred)) : "memory");
+  return n;
 }
 
 // Hand-over of P and of the tensor turn through named barriers.  An mbarrier lives in shared
 // memory, whose bandwidth the MMA operands of Q K^T use up: an arrive or a try_wait there took
 // 120-270 clk, several times on every key tile's critical path; a named barrier takes 25-60 clk.
-// A named barrier has no bounded wait, so every role meets each of them a fixed number of times
-// (once per key tile of its segments), also after it has given up on an mbarrier.
-__device__ __forceinline__ void p_ready_arrive(int a) {   // softmax group a: P of a key tile is in TMEM
-  if (a == 0) asm volatile("bar.arrive 3, 160;" ::: "memory");
-  else asm volatile("bar.arrive 4, 160;" ::: "memory");
+// A named barrier has no bounded wait, so every warp keeps meeting them, once per key tile of its
+// segments, after it has given up on an mbarrier as well; handover.h says why all of them end.  The
+// turns alternate strictly between two warps that take and pass them whether or not they gave up.
+__device__ __forceinline__ void p_ready_sync(int a, uint32_t tile) {   // issuer a: P of group a's tile-th key tile is in TMEM
+  asm volatile("bar.sync %0, 160;" ::"r"(p_ready_barrier(a, tile)) : "memory");
 }
-__device__ __forceinline__ void p_ready_sync(int a) {     // issuer a
-  if (a == 0) asm volatile("bar.sync 3, 160;" ::: "memory");
-  else asm volatile("bar.sync 4, 160;" ::: "memory");
+__device__ __forceinline__ void p_ready_pass(int a, uint32_t tile, bool gave_up) {   // a warp of softmax group a
+  if (p_ready_waits(gave_up)) p_ready_sync(a, tile);
+  else asm volatile("bar.arrive %0, 160;" ::"r"(p_ready_barrier(a, tile)) : "memory");
 }
 __device__ __forceinline__ void turn_sync(int a) {        // issuer a waits for the tensor pipe
-  if (a == 0) asm volatile("bar.sync 5, 64;" ::: "memory");
-  else asm volatile("bar.sync 6, 64;" ::: "memory");
+  asm volatile("bar.sync %0, 64;" ::"r"(kTurnBarrier + a) : "memory");
 }
 __device__ __forceinline__ void turn_pass(int a) {        // issuer a hands it to the other one
-  if (a == 0) asm volatile("bar.arrive 6, 64;" ::: "memory");
-  else asm volatile("bar.arrive 5, 64;" ::: "memory");
+  asm volatile("bar.arrive %0, 64;" ::"r"(kTurnBarrier + 1 - a) : "memory");
 }
 
 // Exponentials of 32 score columns (registers s) into 16 bf16 pairs (p) and the packed sums.
@@ -255,9 +261,9 @@ constexpr float kOptimisticLimit = 18446744073709551616.f;   // 2^64
 template <bool kMasked, int kCols>   // kCols: score columns that hold keys, 64 or 128
 __device__ __forceinline__ void softmax_row_tile(uint32_t t_S, uint32_t t_O, float c, int nvalid,
                                                  bool first, float& m_run, float& l_run,
-                                                 int a, int trace_role, int trace_tile) {
+                                                 int a, uint32_t tile) {
   if (first) m_run = max_row<kMasked, kCols>(t_S, nvalid);
-  TRACE(trace_role, trace_tile, 2);
+  TRACE(a, tile, 2);
   uint32_t p0[32], p1[32];
   float sum;
   bool redone = false;
@@ -288,8 +294,8 @@ __device__ __forceinline__ void softmax_row_tile(uint32_t t_S, uint32_t t_O, flo
   if (kCols > 64) tmem_st32(t_S + 32, p1);   // P of keys 64..127 over score columns 32..63
   tc_wait_st();
   tc_fence_before();
-  p_ready_arrive(a);
-  TRACE(trace_role, trace_tile, 5);
+  p_ready_pass(a, tile, false);
+  TRACE(a, tile, 5);
   l_run += sum;
 }
 
@@ -337,7 +343,6 @@ window_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
   const uint32_t bar_o_final = bar_s_full + 16;              // [2]  MMA warp a -> softmax a
   volatile uint32_t* tmem_slot = reinterpret_cast<volatile uint32_t*>(gen + kSmemBar + 224);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(gen + kSmemBar + 228);
-  volatile int* merge_flag = reinterpret_cast<volatile int*>(gen + kSmemBar + 232);   // [2]
 
   const int tid = threadIdx.x;
   const int warp = tid >> 5;
@@ -430,7 +435,7 @@ window_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
       Sched sched(p, static_cast<int>(blockIdx.x));
       Seg s;
       uint32_t kv_it = 0, q_it = 0, turns = 0;
-      [[maybe_unused]] uint32_t sp_it = 0;   // key tiles so far (timeline stamps)
+      uint32_t sp_it = 0;   // key tiles so far
       bool ok = true;
       const bool lead = lane == 0;
       const uint32_t idesc_pv = idesc_bf16_f32(kTileM, kHeadDim, 1);
@@ -502,7 +507,7 @@ window_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
           if (part) {
             const uint64_t dv = dv0 + static_cast<uint64_t>((vst * kTileBytes) >> 4);
             TRACE(2 + a, sp_it, 0);
-            p_ready_sync(a);   // P of this tile is in TMEM, O rescaled if need be
+            p_ready_sync(a, sp_it);   // P of this tile is in TMEM, O rescaled if need be
             TRACE(2 + a, sp_it, 1);
             // The two issuers take turns with their P V + Q K^T chains: issued side by side the
             // chains would interleave in the tensor pipe and finish together, which pulls the
@@ -550,37 +555,36 @@ window_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
     const int row = tid & 127;             // row inside the tile = TMEM lane
     const uint32_t t_lane = tmem_base + (static_cast<uint32_t>((warp & 3) * 32) << 16);
     const uint32_t t_S = t_lane + a * 128, t_O = t_lane + 256 + a * 128;
-    volatile int* my_flag = merge_flag + a;
     Sched sched(p, static_cast<int>(blockIdx.x));
     Seg s;
     uint32_t it = 0, seg_it = 0;
     bool ok = true;
     int seg_no = 0;
     CTRACE(1);
-    // After a wait gave up (ok == false) a thread keeps walking its segments without working, so
-    // that it still meets its group and its issuer at every named barrier.
+    // After a wait gave up (ok == false) a warp keeps walking its segments without working, so that
+    // it still meets its group and its issuer at every named barrier.  ok is the same in all threads
+    // of a warp: barriers and TMEM accesses are instructions of the whole warp.
     while (sched.next(s)) {
       if (a >= s.nq) continue;             // a lone last query tile: nothing for group 1
       float m_run = -INFINITY, l_run = 0.f;
       const ValidKeys valid_of(p, s.b);
-      for (int j = s.t0; j < s.t1; ++j) {
+      for (int j = s.t0; j < s.t1; ++j, ++it) {
         const int valid = valid_of(j);
         TRACE(a, it, 0);
-        if (ok) ok = w.wait(bar_s_full + 8 * a, it & 1);
+        if (ok) ok = __all_sync(0xFFFFFFFFu, w.wait(bar_s_full + 8 * a, it & 1));
         if (!ok) {
-          p_ready_arrive(a);   // the issuer still counts on it
+          p_ready_pass(a, it, true);   // the issuer still counts on this warp
           continue;
         }
         tc_fence_after();
         if (it == 0) CTRACE(2);
         TRACE(a, it, 1);
         if (valid <= 64)   // frames of at most half a tile, and the end of a run
-          softmax_row_tile<true, 64>(t_S, t_O, p.scale_log2e, valid, j == s.t0, m_run, l_run, a, a, it);
+          softmax_row_tile<true, 64>(t_S, t_O, p.scale_log2e, valid, j == s.t0, m_run, l_run, a, it);
         else if (valid < kTileN)
-          softmax_row_tile<true, kTileN>(t_S, t_O, p.scale_log2e, valid, j == s.t0, m_run, l_run, a, a, it);
+          softmax_row_tile<true, kTileN>(t_S, t_O, p.scale_log2e, valid, j == s.t0, m_run, l_run, a, it);
         else
-          softmax_row_tile<false, kTileN>(t_S, t_O, p.scale_log2e, kTileN, j == s.t0, m_run, l_run, a, a, it);
-        ++it;
+          softmax_row_tile<false, kTileN>(t_S, t_O, p.scale_log2e, kTileN, j == s.t0, m_run, l_run, a, it);
       }
       CTRACE(8 + seg_no);
       // ---- epilogue of this group's query tile ----
@@ -595,7 +599,7 @@ window_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
         asm volatile("ld.acquire.gpu.global.s32 %0, [%1];" : "=r"(seen) : "l"(counter()) : "memory");
       }
       if (ok) {
-        ok = w.wait(bar_o_final + 8 * a, seg_it & 1);
+        ok = __all_sync(0xFFFFFFFFu, w.wait(bar_o_final + 8 * a, seg_it & 1));
         ++seg_it;
         tc_fence_after();
       }
@@ -640,11 +644,12 @@ window_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
         const int c_lo = first_part_worker(p, s);
         const int c_hi = last_part_worker(p, s);
         const int others = c_hi - c_lo;
-        if (row == 0) *my_flag = (seen == others) ? 1 : 0;
-        group_barrier(a);
-        if (*abort_flag) ok = false;       // somebody gave up: keep meeting the barriers, report nothing
-        bool last = (*my_flag != 0);
-        if (!last) {
+        // one thread says whether all others are in, the others whether their warp gave up (31 or
+        // more do then); a group that gave up publishes nothing
+        const uint32_t votes = group_count(a, row == 0 ? seen == others : !ok);
+        if (votes > 1) ok = false;
+        bool last = votes == 1;
+        if (ok && !last) {
           const int64_t mine = (static_cast<int64_t>(2 * blockIdx.x + (s.first_in_worker ? 0 : 1)) * kPartFloats +
                                 a * kPartTileFloats);   // first float of this part in the scratch
           float4* const part4 = reinterpret_cast<float4*>(p.part);
@@ -663,18 +668,16 @@ window_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
           }
           UNSTEP_STORE(reinterpret_cast<float2*>(p.part), mine / 2 + 128 * 64 + row, p.extent_part / 2,
                        make_float2(m_run, l_run), p.status);
-          group_barrier(a);   // all of this part is stored; everyone has read the flag
+          group_barrier(a);   // all of this part is stored
+          int before = -1;
           if (row == 0) {
             // release: the group's stores (ordered before this thread by the barrier) become visible
             // before the count; acquire: a merging part sees the other parts' stores
-            int before;
             asm volatile("atom.acq_rel.gpu.global.add.s32 %0, [%1], 1;" : "=r"(before) : "l"(counter()) : "memory");
-            *my_flag = (before == others) ? 1 : 0;
           }
-          group_barrier(a);
-          last = (*my_flag != 0);
+          last = group_count(a, before == others) != 0;
         }
-        if (last) {
+        if (ok && last) {
           __threadfence();   // acquire side for every thread that reads the other parts below
           if (row == 0) UNSTEP_STORE(p.counters, 2 * s.item + a, p.extent_counters, 0, p.status);   // ready for the next launch
           const int me = static_cast<int>(blockIdx.x);
