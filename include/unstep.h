@@ -119,14 +119,17 @@ int unstep_rope_kv_append(const unstep_shape_t* shape, const int32_t* start_fram
  *   out           : bf16 [B, L, Hn, 128], written.
  * Scratch: work items that are split across thread blocks exchange partial results through a
  * buffer the library keeps per (device, stream).  The first call on a stream creates it with
- * cudaMalloc (about 40 MB): make that call outside any stream capture.  Calls on one stream
- * share the buffer safely; calls on different streams use different buffers.  A buffer is replaced
- * by a larger one when a later call on its stream needs more (more SMs or more work items).
+ * cudaMalloc (two slots per SM, about 40 MB, whatever the problem): make that call outside any stream
+ * capture.  Calls on one stream share the buffer safely; calls on different streams use different
+ * buffers.  Only the arrival counters depend on the problem: 8 bytes per work item (stream, head, pair
+ * of 128-query tiles; up to 32 streams), independent of the start frames and the window.  The first
+ * call of a stream with more than 2048 work items, and any later one with more than there is room
+ * for, gets a larger array (again by cudaMalloc, outside any capture); the former one is kept, and
+ * together they are at most twice the largest.  Everything is freed by unstep_shutdown() only.
  * CUDA graphs: a call captured into a graph freezes the addresses of the capture stream's buffer
- * into the graph.  Such a graph is invalid after unstep_shutdown() and after a larger problem was
- * run on the capture stream (both free the buffer), and its replays must not overlap on the GPU
- * with each other or with direct calls on the capture stream.  Capture all graphs that may replay
- * back to back on one stream, after one uncaptured call of the largest problem on that stream.
+ * into the graph.  Such a graph is invalid after unstep_shutdown(), and its replays must not overlap
+ * on the GPU with each other or with direct calls on the capture stream.  Capture all graphs that may
+ * replay back to back on one stream, after one uncaptured call on that stream with the most work items.
  */
 int unstep_window_attn(const unstep_shape_t* shape, const int32_t* start_frame,
                        int32_t window_frames, const void* q_rot, const void* ring_k,

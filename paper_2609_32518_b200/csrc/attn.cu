@@ -847,37 +847,54 @@ static const DeviceInfo& device_info() {
 }
 
 // Scratch for split items, one per (device, stream): calls on one stream run in order and may
-// share it; calls on different streams may overlap on the GPU and must not.  Allocated on first
-// use and kept; it only grows.
+// share it; calls on different streams may overlap on the GPU and must not.  Captured graphs hold
+// its addresses, so nothing is given back before unstep_shutdown().  The partial results have two
+// slots per SM whatever the launch: the workers of a launch go up and down with the start frame (one
+// to all SMs), and a buffer sized by them would move under graphs captured before.  The counters
+// go by the work items of the shape and at least double when they grow, so the arrays they have
+// left behind are together no larger than the one in use.
 struct Workspace {
   float* part = nullptr;
   int* counters = nullptr;
   size_t slots = 0, n_counters = 0;
 };
+constexpr size_t kLeastCounters = 4096;
+constexpr int kMaxGrowths = 32;
+struct StreamScratch {
+  Workspace ws;
+  Workspace left[kMaxGrowths];   // counters of former calls; captured graphs may still count in them
+  int n_left = 0;
+};
 static std::mutex g_ws_mutex;
-static std::map<std::pair<int, cudaStream_t>, Workspace> g_workspaces;
+static std::map<std::pair<int, cudaStream_t>, StreamScratch> g_workspaces;
 
 static int get_workspace(cudaStream_t st, size_t slots, size_t n_counters, Workspace* out) {
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess) return UNSTEP_ERR_CUDA;
   std::lock_guard<std::mutex> lock(g_ws_mutex);
-  Workspace& ws = g_workspaces[std::make_pair(dev, st)];
-  if (ws.slots < slots) {
-    if (ws.part != nullptr && cudaFree(ws.part) != cudaSuccess) return UNSTEP_ERR_CUDA;
-    ws.part = nullptr;
-    ws.slots = 0;
-    if (cudaMalloc(&ws.part, slots * kPartFloats * sizeof(float)) != cudaSuccess) return UNSTEP_ERR_CUDA;
+  StreamScratch& s = g_workspaces[std::make_pair(dev, st)];
+  Workspace& ws = s.ws;
+  if (ws.part == nullptr) {
+    if (cudaMalloc(&ws.part, slots * kPartFloats * sizeof(float)) != cudaSuccess) {
+      ws.part = nullptr;
+      return UNSTEP_ERR_CUDA;
+    }
     ws.slots = slots;
   }
   if (ws.n_counters < n_counters) {
-    if (ws.counters != nullptr && cudaFree(ws.counters) != cudaSuccess) return UNSTEP_ERR_CUDA;
-    ws.counters = nullptr;
-    ws.n_counters = 0;
-    if (cudaMalloc(&ws.counters, n_counters * sizeof(int)) != cudaSuccess) return UNSTEP_ERR_CUDA;
+    size_t n = ws.n_counters > 0 ? 2 * ws.n_counters : kLeastCounters;
+    while (n < n_counters) n *= 2;
+    int* counters = nullptr;
+    if (s.n_left == kMaxGrowths || cudaMalloc(&counters, n * sizeof(int)) != cudaSuccess) return UNSTEP_ERR_CUDA;
     // cleared on the caller's stream, so that the clear is ordered before the kernel that follows
     // (a non-blocking stream is not ordered against the legacy default stream)
-    if (cudaMemsetAsync(ws.counters, 0, n_counters * sizeof(int), st) != cudaSuccess) return UNSTEP_ERR_CUDA;
-    ws.n_counters = n_counters;
+    if (cudaMemsetAsync(counters, 0, n * sizeof(int), st) != cudaSuccess) {
+      cudaFree(counters);
+      return UNSTEP_ERR_CUDA;
+    }
+    if (ws.counters != nullptr) s.left[s.n_left++] = ws;
+    ws.counters = counters;
+    ws.n_counters = n;
   }
   *out = ws;
   return UNSTEP_OK;
@@ -888,9 +905,12 @@ static void reset_workspace_counters() {
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess) return;
   std::lock_guard<std::mutex> lock(g_ws_mutex);
-  for (auto& kv : g_workspaces)
-    if (kv.first.first == dev && kv.second.counters != nullptr)
-      cudaMemset(kv.second.counters, 0, kv.second.n_counters * sizeof(int));
+  for (auto& kv : g_workspaces) {
+    if (kv.first.first != dev) continue;
+    const StreamScratch& s = kv.second;
+    if (s.ws.counters != nullptr) cudaMemset(s.ws.counters, 0, s.ws.n_counters * sizeof(int));
+    for (int i = 0; i < s.n_left; ++i) cudaMemset(s.left[i].counters, 0, s.left[i].n_counters * sizeof(int));
+  }
 }
 
 // Device address of g_status on the current device, looked up once per device.
@@ -912,8 +932,8 @@ int* status_word() {
 
 using namespace unstep;
 
-// Hands out the scratch of one launch: `slots` partial-result slots and `n_counters` zeroed
-// arrival counters.
+// Hands out the scratch of one launch: `slots` partial-result slots (two per SM) and at least
+// `n_counters` zeroed arrival counters.
 typedef int (*ScratchFn)(cudaStream_t st, size_t slots, size_t n_counters, Workspace* out);   // an unstep_status
 
 constexpr int kOverlapSteps = 64;   // key-tile steps per worker below which a launch overlaps the kernel before it
@@ -949,7 +969,7 @@ static int window_attn_run(const unstep_shape_t* shape, const int32_t* start_fra
     rc = plan_launch(p, shape, start_frame + b0, nb, window_frames, sink_frames, sink_attend, info.sm_count);
     if (rc != UNSTEP_OK) return rc;
     Workspace ws;
-    rc = scratch(st, 2 * static_cast<size_t>(p.n_workers), 2 * static_cast<size_t>(nb) * p.items_per_stream, &ws);
+    rc = scratch(st, 2 * static_cast<size_t>(info.sm_count), 2 * static_cast<size_t>(nb) * p.items_per_stream, &ws);
     if (rc != UNSTEP_OK) return rc;
     p.part = ws.part;
     p.counters = ws.counters;
@@ -1132,8 +1152,10 @@ extern "C" void unstep_shutdown(void) {
   for (auto& kv : g_workspaces) {
     if (cudaSetDevice(kv.first.first) != cudaSuccess) continue;
     cudaDeviceSynchronize();
-    if (kv.second.part != nullptr) cudaFree(kv.second.part);
-    if (kv.second.counters != nullptr) cudaFree(kv.second.counters);
+    const StreamScratch& s = kv.second;
+    if (s.ws.part != nullptr) cudaFree(s.ws.part);
+    if (s.ws.counters != nullptr) cudaFree(s.ws.counters);
+    for (int i = 0; i < s.n_left; ++i) cudaFree(s.left[i].counters);
   }
   g_workspaces.clear();
   cudaSetDevice(cur);

@@ -44,7 +44,8 @@ class ChunkStepper:
         # Every graph of this stepper is captured on this one stream.  The attention call keeps its
         # scratch per stream and a capture freezes the scratch pointers into the graph, so one
         # capture stream means one scratch for all graphs (replays of one stepper run one after
-        # the other on the caller's stream and may share it).
+        # the other on the caller's stream and may share it).  The scratch of a shape is the same at
+        # every start frame, so a later capture leaves the earlier graphs' addresses alone.
         self._capture_stream = torch.cuda.Stream(device=self.device)
 
     def table(self, start_frame: int):

@@ -136,3 +136,15 @@ def test_split_of_more_steps_than_32_bit_products_hold():
     for s in segs:
         work[s[0]] = work.get(s[0], 0) + s[6] - s[5]
     assert len(work) == 148 and max(work.values()) - min(work.values()) <= 1 and sum(work.values()) == total
+
+
+def test_workers_rise_and_fall_along_a_clip_within_the_grid():
+    # scratch has two slots for each of the grid's workers, whatever the start frame
+    workers = {}
+    for heads, fc, starts in [(3, 3, (0, 3, 18)), (1, 1, (0, 18, 19, 20))]:
+        sh = U.Shape.make(batch=1, heads=heads, chunk_frames=fc, grid_h=30, grid_w=52, ring_frames=21)
+        for start in starts:
+            segs = check_plan(sh, [start], 21, 148)
+            workers[heads, start] = 1 + max(s[0] for s in segs)
+    assert workers[3, 0] < workers[3, 3] and workers[1, 20] < workers[1, 19]
+    assert max(workers.values()) <= 148
