@@ -36,7 +36,7 @@ struct AttnParams {
   int32_t parts;            // > 0: every item of the remainder is cut into this many parts, one per worker
   int32_t n_active;         // parts == 0: workers that take a share of the remainder, >= 1
   int64_t all_steps;        // key tiles of all items of the launch
-  int32_t narrow;           // 1: total_steps * n_active fits 32 bits, and so does every index of the split
+  int32_t narrow;           // 1: total_steps * n_active fits 32 bits, and so does every index of the shares
   int64_t total_steps;      // remainder: sum over the leftover items of their key tiles
   float* part;              // workspace: partial results of split items, kPartFloats per slot
   int* counters;            // workspace: arrivals per (item, query tile), zero between launches
@@ -179,8 +179,10 @@ struct Sched {
       const int item = me / p.parts, part = me - item * p.parts;
       const int b = item / p.leftover;
       decode(s, b, p.full_rounds * p.n_workers + item - b * p.leftover);
-      s.t0 = s.tiles * part / p.parts;
-      s.t1 = s.tiles * (part + 1) / p.parts;
+      // tiles * part / parts without that product, which passes 32 bits for items of many tiles
+      const uint32_t each = s.tiles / p.parts, over = s.tiles - each * p.parts;
+      s.t0 = static_cast<int>(each * part + over * part / p.parts);
+      s.t1 = static_cast<int>(each * (part + 1) + over * (part + 1) / p.parts);
       s.item_step0 = me - part;
       s.first_in_worker = true;
       cur = hi;
