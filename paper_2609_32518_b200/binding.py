@@ -2,7 +2,8 @@
 
 A call goes through the native marshalling module (csrc/marshal.cpp) when all its arguments have
 exactly the expected form; the module answers None for anything else, before anything is launched,
-and the general path in ctypes takes over and raises what there is to raise."""
+and the general path in ctypes takes over and raises what there is to raise.  Where the module cannot
+be built or loaded (no host compiler, no headers), every call takes the general path."""
 
 from __future__ import annotations
 
@@ -45,7 +46,14 @@ class Shape(ctypes.Structure):
 
 
 _lib = None
-_fast = None   # the native marshalling module, bound to the functions of _lib
+_fast = None   # the native marshalling module, bound to the functions of _lib, or a _NoMarshal
+
+
+class _NoMarshal:
+    """Stands in for the marshalling module: no call is of its form."""
+
+    def __getattr__(self, name):
+        return lambda *args: None
 
 
 def lib() -> ctypes.CDLL:
@@ -101,7 +109,13 @@ def _native():
     global _fast
     if _fast is None:
         L = lib()
-        mod = _build.load_marshal()
+        try:
+            mod = _build.load_marshal()
+        except (ImportError, OSError, RuntimeError) as e:
+            import warnings
+            warnings.warn(f"calls are marshalled by ctypes, 8-10 us each: {e}", RuntimeWarning, stacklevel=3)
+            _fast = _NoMarshal()
+            return _fast
         mod.bind(Shape, *(ctypes.cast(f, c_void_p).value for f in (
             L.unstep_rope_table, L.unstep_rope_kv_append_sink, L.unstep_rmsnorm_rope_kv_append,
             L.unstep_window_attn, L.unstep_window_attn_noalloc, L.unstep_window_attn_sink)))

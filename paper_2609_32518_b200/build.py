@@ -74,9 +74,10 @@ def build(force: bool = False, verbose: bool = False, variant: str = "") -> str:
 
 
 def marshal_path() -> str:
-    """The module is tied to the torch it was compiled against, so its name carries the version."""
+    """The module is tied to the torch and the Python it was compiled against, so its name carries both."""
     import torch
-    return os.path.join(PKG_DIR, "_marshal_" + torch.__version__.replace("+", "_") + ".so")
+    return os.path.join(PKG_DIR, "_marshal_" + torch.__version__.replace("+", "_") +
+                        (sysconfig.get_config_var("EXT_SUFFIX") or ".so"))
 
 
 def build_marshal(force: bool = False) -> str:

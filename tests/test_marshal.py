@@ -60,6 +60,49 @@ def test_malformed_calls_end_in_the_general_path():
     assert native.attn(sh, [1, 2], 4.0, t["q"], t["ck"], t["cv"], t["out"], None) is None
 
 
+@pytest.mark.parametrize("broken", ["no compiler", "no nvcc", "module does not load"])
+def test_calls_do_without_the_module(broken, monkeypatch, tmp_path):
+    if broken == "module does not load":
+        (tmp_path / "m.so").write_bytes(b"not a library")
+        monkeypatch.setattr(binding._build, "build_marshal", lambda force=False: str(tmp_path / "m.so"))
+    else:
+        monkeypatch.setattr(binding._build, "marshal_path", lambda: str(tmp_path / "absent.so"))
+        if broken == "no compiler":
+            monkeypatch.setenv("CXX", str(tmp_path / "no-such-compiler"))
+        else:
+            def no_nvcc():
+                raise RuntimeError("nvcc not found")
+            monkeypatch.setattr(binding._build, "_nvcc", no_nvcc)
+    binding.lib()
+    monkeypatch.setattr(binding, "_fast", None)
+    sh, t = buffers("cpu")
+    with pytest.warns(RuntimeWarning, match="marshalled by ctypes"):
+        with pytest.raises(TypeError, match="expected a CUDA tensor"):   # the general path's answer
+            U.rope_table(sh, 7, t["cos"], t["sin"])
+    for name, args in calls(sh, t, 0).items():                           # and no second warning
+        with pytest.raises(TypeError, match="expected a CUDA tensor"):
+            getattr(U, name)(*args)
+
+
+def test_the_file_of_the_module_names_torch_and_python():
+    import sysconfig
+    path = binding._build.marshal_path()
+    assert path.endswith(sysconfig.get_config_var("EXT_SUFFIX")) and torch.__version__.split("+")[0] in path
+
+
+@pytest.mark.gpu
+def test_well_formed_calls_take_the_module():
+    for sink in (0, 2):
+        sh, t = buffers("cuda", sink)
+        native, made = binding._native(), calls(sh, t, sink)
+        s, ap = made["rmsnorm_rope_kv_append"], made["rope_kv_append_sink"]
+        assert native.norm_append(*s) == 0 and native.append(*ap) == 0 and native.attn_sink(*made["window_attn_sink"]) == 0
+        if sink == 0:
+            assert native.rope_table(*made["rope_table"]) == 0
+            assert native.attn(*made["window_attn"]) == 0 and native.attn_noalloc(*made["window_attn_noalloc"]) == 0
+    assert U.poll_status() == 0
+
+
 @pytest.mark.gpu
 @pytest.mark.parametrize("sink", [0, 2])
 def test_same_results_as_the_general_path(sink):
