@@ -284,6 +284,12 @@ int64_t unstep_launch_count(void);
  * UNSTEP_ERR_BOUNDS once.  Shows that the checks are armed; nothing faults.
  */
 int unstep_selftest_bounds_check(int32_t* device_buf5, void* cuda_stream);
+/*
+ * The same for the 32-byte stores: two threads store 32 bytes each into the first 48 bytes of
+ * `device_buf16` (DEVICE int32 [16], 32-byte aligned).  The second store is half outside and skipped
+ * whole: the first eight elements become 7, the others keep their values.
+ */
+int unstep_selftest_bounds_check_wide(int32_t* device_buf16, void* cuda_stream);
 #endif
 
 #ifdef UNSTEP_TRACE

@@ -610,13 +610,11 @@ window_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
         uint32_t w[16];
 #pragma unroll
         for (int i = 0; i < 16; ++i) w[i] = pack_bf16x2(v[2 * i] * inv_l, v[2 * i + 1] * inv_l);
-#ifndef UNSTEP_CHECK
         if (p.out_wide) {   // whole 32-byte sectors
-          st_global_32(out_v + d, w);
-          st_global_32(out_v + d + 2, w + 8);
+          UNSTEP_STORE_32(out_v, d, p.extent_out, w, p.status);
+          UNSTEP_STORE_32(out_v, d + 2, p.extent_out, w + 8, p.status);
           return;
         }
-#endif
 #pragma unroll
         for (int i = 0; i < 4; ++i)
           UNSTEP_STORE(out_v, d + i, p.extent_out, make_uint4(w[4 * i], w[4 * i + 1], w[4 * i + 2], w[4 * i + 3]),
@@ -1120,6 +1118,11 @@ namespace unstep {
 __global__ void check_probe_kernel(int* buf, int* status) {
   UNSTEP_STORE(buf, threadIdx.x, 4, 7, status);
 }
+// Two 32-byte stores into three 16-byte vectors: the second one is half outside and must be skipped whole.
+__global__ void check_probe_wide_kernel(int* buf, int* status) {
+  const uint32_t w[8] = {7, 7, 7, 7, 7, 7, 7, 7};
+  UNSTEP_STORE_32(reinterpret_cast<uint4*>(buf), 2 * threadIdx.x, 3, w, status);
+}
 }  // namespace unstep
 
 extern "C" int unstep_selftest_bounds_check(int32_t* device_buf5, void* cuda_stream) {
@@ -1129,6 +1132,17 @@ extern "C" int unstep_selftest_bounds_check(int32_t* device_buf5, void* cuda_str
   int* st = status_word();
   if (st == nullptr) return UNSTEP_ERR_CUDA;
   check_probe_kernel<<<1, 5, 0, static_cast<cudaStream_t>(cuda_stream)>>>(device_buf5, st);
+  g_launches.fetch_add(1);
+  return cudaGetLastError() == cudaSuccess ? UNSTEP_OK : UNSTEP_ERR_CUDA;
+}
+
+extern "C" int unstep_selftest_bounds_check_wide(int32_t* device_buf16, void* cuda_stream) {
+  if (device_buf16 == nullptr || (reinterpret_cast<uintptr_t>(device_buf16) & 31u) != 0) return UNSTEP_ERR_INVALID_ARG;
+  const int rc = check_device();
+  if (rc != UNSTEP_OK) return rc;
+  int* st = status_word();
+  if (st == nullptr) return UNSTEP_ERR_CUDA;
+  check_probe_wide_kernel<<<1, 2, 0, static_cast<cudaStream_t>(cuda_stream)>>>(device_buf16, st);
   g_launches.fetch_add(1);
   return cudaGetLastError() == cudaSuccess ? UNSTEP_OK : UNSTEP_ERR_CUDA;
 }

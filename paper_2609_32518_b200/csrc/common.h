@@ -22,7 +22,8 @@ int* status_word();
 // A checking build (-DUNSTEP_CHECK) tests every global store of the kernels against the extent of
 // the buffer it belongs to; a store outside is skipped and recorded in the status word (no trap),
 // so that a wrong index shows up as UNSTEP_ERR_BOUNDS instead of silent corruption.  This stands
-// in for a memory checker where none can be run.  In a normal build the macro is the plain store.
+// in for a memory checker where none can be run.  In a normal build the macros are the plain stores.
+// UNSTEP_STORE_32 stores 32 bytes, two 16-byte vectors of `base` from vector `idx` on.
 #ifdef UNSTEP_CHECK
 #define UNSTEP_STORE(base, idx, extent, value, status)                                  \
   do {                                                                                  \
@@ -30,8 +31,15 @@ int* status_word();
     if (idx_ >= 0 && idx_ < static_cast<long long>(extent)) (base)[idx_] = (value);     \
     else atomicExch((status), static_cast<int>(UNSTEP_ERR_BOUNDS));                     \
   } while (0)
+#define UNSTEP_STORE_32(base, idx, extent, words, status)                               \
+  do {                                                                                  \
+    const long long idx_ = static_cast<long long>(idx);                                 \
+    if (idx_ >= 0 && idx_ + 2 <= static_cast<long long>(extent)) ptx::st_global_32((base) + idx_, (words)); \
+    else atomicExch((status), static_cast<int>(UNSTEP_ERR_BOUNDS));                     \
+  } while (0)
 #else
 #define UNSTEP_STORE(base, idx, extent, value, status) ((base)[idx] = (value))
+#define UNSTEP_STORE_32(base, idx, extent, words, status) ptx::st_global_32((base) + (idx), (words))
 #endif
 
 inline bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }

@@ -313,3 +313,21 @@ def test_keys_far_above_the_reference_wherever_they_sit(grid, fc, ring, history,
     assert np.array_equal(to_bits(q_dev), q_ref)
     check(to_bits(dev.attend([start], ring, q_dev)), ora.attend([start], ring, q_ref), f"keys {keys}")
     assert U.poll_status() == 0
+
+
+@pytest.mark.parametrize("heads,grid,ring", [(2, (8, 8), 6), (12, (30, 52), 9)])   # parts, and whole items as well
+def test_result_at_an_address_of_16_bytes(heads, grid, ring):
+    # rows are stored 32 bytes at a time where the result is 32-byte aligned, 16 bytes otherwise
+    sh = U.Shape.make(1, heads, 3, grid[0], grid[1], ring)
+    gen = torch.Generator(device="cuda").manual_seed(3)
+    dims, cache = (1, sh.chunk_tokens, heads, 128), (1, ring, sh.tokens_per_frame, heads, 128)
+    q, ck, cv = (torch.randn(d, generator=gen, device="cuda").to(torch.bfloat16) for d in (dims, cache, cache))
+    want = torch.empty_like(q)
+    U.window_attn(sh, [ring - 3], ring, q, ck, cv, want)
+    raw = torch.full((q.numel() + 16,), 0x7FA5, dtype=torch.int16, device="cuda")
+    out = raw[8:-8].view(torch.bfloat16).view(dims)
+    assert out.data_ptr() % 32 == 16 and want.data_ptr() % 32 == 0
+    U.window_attn(sh, [ring - 3], ring, q, ck, cv, out)
+    assert torch.equal(out.view(torch.int16), want.view(torch.int16))
+    assert bool((raw[:8] == 0x7FA5).all()) and bool((raw[-8:] == 0x7FA5).all())
+    assert U.poll_status() == 0

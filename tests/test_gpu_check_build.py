@@ -37,21 +37,21 @@ def _child():
     class Guarded:
         """A bf16 device buffer of `numel` elements between two sentinel bands."""
 
-        def __init__(self, shape, fill=0x7FC1):
-            self.n = int(np.prod(shape))
-            self.raw = torch.full((self.n + 2 * GUARD,), BAND, dtype=torch.int16, device="cuda")
-            self.raw[GUARD:GUARD + self.n] = fill
-            self.t = self.raw[GUARD:GUARD + self.n].view(torch.bfloat16).view(shape)
+        def __init__(self, shape, fill=0x7FC1, offset=0):
+            self.n, self.lo = int(np.prod(shape)), GUARD + offset
+            self.raw = torch.full((self.n + 2 * GUARD + offset,), BAND, dtype=torch.int16, device="cuda")
+            self.raw[self.lo:self.lo + self.n] = fill
+            self.t = self.raw[self.lo:self.lo + self.n].view(torch.bfloat16).view(shape)
             assert self.t.data_ptr() % 16 == 0 and self.t.is_contiguous()
 
         def intact(self):
-            lo, hi = self.raw[:GUARD], self.raw[GUARD + self.n:]
+            lo, hi = self.raw[:self.lo], self.raw[self.lo + self.n:]
             return bool((lo == BAND).all()) and bool((hi == BAND).all())
 
         def bits(self):
             return self.t.contiguous().view(torch.int16).cpu().numpy().view(np.uint16)
 
-    def run(wl, extra_history=(), sink=0, sink_attend=0, norm=False):
+    def run(wl, extra_history=(), sink=0, sink_attend=0, norm=False, out_offset=0):
         sh = wl.shape
         abi = abi_shape(sh)
         cache_shape = (sh.batch, sink + sh.ring_frames, sh.tokens_per_frame, sh.heads, sh.head_dim)
@@ -118,7 +118,8 @@ def _child():
             append(starts)
         q_out, q_ref = append(wl.measured_starts)
         for wf in wl.window_frames:
-            out = Guarded(act_shape)
+            out = Guarded(act_shape, offset=out_offset)   # 8 elements: 16-byte stores of the result, else 32-byte ones
+            assert (out.t.data_ptr() % 32 == 0) == (out_offset % 16 == 0)
             starts = [int(s) for s in wl.measured_starts]
             if sink:
                 U.window_attn_sink(abi, sink, starts, wf, sink_attend, q_out.t, ck.t, cv.t, out.t)
@@ -143,6 +144,14 @@ def _child():
     assert probe.cpu().tolist() == [7, 7, 7, 7, 0]
     assert U.poll_status() == -6 and U.poll_status() == 0
 
+    wide = torch.zeros(16, dtype=torch.int32, device="cuda")
+    lib.unstep_selftest_bounds_check_wide.argtypes = [ctypes.c_void_p, ctypes.c_void_p]
+    lib.unstep_selftest_bounds_check_wide.restype = ctypes.c_int
+    assert lib.unstep_selftest_bounds_check_wide(ctypes.c_void_p(wide.data_ptr()), None) == 0
+    torch.cuda.synchronize()
+    assert wide.cpu().tolist() == [7] * 8 + [0] * 8
+    assert U.poll_status() == -6 and U.poll_status() == 0
+
     cfg1 = W.WORKLOADS["cfg1"]
     run(cfg1, extra_history=[[0], [2]])
     w = W.WORKLOADS["cfg1_wrapped"]
@@ -151,6 +160,8 @@ def _child():
     sh = W.Shape(batch=2, heads=3, chunk_frames=3, grid_h=8, grid_w=25, ring_frames=7)
     run(W.Workload("ragged", sh, seed=22, history_starts=((), ()), measured_starts=(12, 3),
                    window_frames=(7, 5, 3), k_scale=4.0), extra_history=[[0, 0], [3, 0], [6, 0], [9, 0]])
+    run(W.Workload("ragged_narrow", sh, seed=23, history_starts=((), ()), measured_starts=(12, 3),
+                   window_frames=(7, 3)), extra_history=[[0, 0], [3, 0], [6, 0], [9, 0]], out_offset=8)
     # 35 and 37 streams: more than one launch carries, frames shorter than a tile
     for nstreams, seed in ((35, 24), (37, 33)):
         sh = W.Shape(batch=nstreams, heads=1, chunk_frames=1, grid_h=4, grid_w=10, ring_frames=4)
@@ -181,6 +192,7 @@ def test_checking_build_compiles_and_exports_its_selftest():
     from paper_2609_32518_b200 import build as B
     lib = ctypes.CDLL(B.build(variant="check"))
     assert hasattr(lib, "unstep_selftest_bounds_check") and hasattr(lib, "unstep_window_attn")
+    assert hasattr(lib, "unstep_selftest_bounds_check_wide")
     import paper_2609_32518_b200 as U
     assert not hasattr(U.lib(), "unstep_selftest_bounds_check")      # the normal build carries no checks
     assert "store" in U.strerror(-6)
