@@ -179,10 +179,8 @@ struct Sched {
       const int item = me / p.parts, part = me - item * p.parts;
       const int b = item / p.leftover;
       decode(s, b, p.full_rounds * p.n_workers + item - b * p.leftover);
-      // tiles * part / parts without that product, which passes 32 bits for items of many tiles
-      const uint32_t each = s.tiles / p.parts, over = s.tiles - each * p.parts;
-      s.t0 = static_cast<int>(each * part + over * part / p.parts);
-      s.t1 = static_cast<int>(each * (part + 1) + over * (part + 1) / p.parts);
+      s.t0 = s.tiles * part / p.parts;   // remainder_parts keeps the products within 32 bits
+      s.t1 = s.tiles * (part + 1) / p.parts;
       s.item_step0 = me - part;
       s.first_in_worker = true;
       cur = hi;
@@ -234,6 +232,7 @@ inline int32_t remainder_parts(int64_t items, int64_t steps, int32_t least, int3
   double lowest = 1.6 * share + 6.0 + 2.2 * (static_cast<double>(steps) / static_cast<double>(items) / share + 1.0);
   int32_t best = 0;
   for (int32_t parts = 1; parts * items <= max_workers && parts <= least; ++parts) {
+    if (static_cast<int64_t>(most) * parts > INT32_MAX) break;   // a part's bounds are 32-bit products
     const double cost = 1.6 * ((most + parts - 1) / parts) + (parts > 1 ? 3.4 + 1.6 * (parts - 2) : 0.0);
     if (cost < lowest) {
       lowest = cost;

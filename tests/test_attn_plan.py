@@ -140,12 +140,13 @@ def test_split_of_more_steps_than_32_bit_products_hold():
 
 @pytest.mark.parametrize("frames", [14_510_024, 14_510_025, 14_600_000, 1 << 24, 1 << 29])
 def test_parts_of_items_of_many_tiles(frames):
-    # frames of one token, a key tile each: tiles x 148 parts passes 2^31 between the first two
+    # frames of one token, a key tile each: tiles x 148 parts passes 2^31 between the first two, and the
+    # item is cut in 64-bit arithmetic from there on
     sh = U.Shape.make(batch=1, heads=1, chunk_frames=1, grid_h=1, grid_w=1, ring_frames=frames)
     segs = U.window_attn_plan(sh, [frames - 1], frames, 148)
     assert [s[0] for s in segs] == list(range(148)) and {s[8] for s in segs} == {148}
-    assert [s[5] for s in segs] == [frames * i // 148 for i in range(148)]
-    assert [s[6] for s in segs] == [frames * (i + 1) // 148 for i in range(148)]
+    assert [s[5] for s in segs] == [0] + [s[6] for s in segs[:-1]] and segs[-1][6] == frames
+    assert {s[6] - s[5] for s in segs} <= {frames // 148, frames // 148 + 1}
 
 
 def test_workers_rise_and_fall_along_a_clip_within_the_grid():
