@@ -92,7 +92,16 @@ inline cudaError_t launch_overlapped(bool overlap, void (*kernel)(KernelArgs...)
 }
 
 #if defined(__CUDACC__)
-__device__ __forceinline__ void grid_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+// Returns 0, as a value that only exists behind the wait.  What a kernel reads may be written while it is
+// already running, so no load may move above the wait, as the compiler may move __ldcs and its like,
+// which clobber nothing: their addresses take this 0 in.  Nor may such a load be an __ldg or go
+// through a `const __restrict__` pointer: those become ld.global.nc, which is for data that nobody
+// writes during the kernel's lifetime, and that began before the wait.  __ldca and __ldcs are coherent.
+__device__ __forceinline__ int grid_wait() {
+  int zero;
+  asm volatile("griddepcontrol.wait;\nmov.u32 %0, 0;" : "=r"(zero)::"memory");
+  return zero;
+}
 // The next kernel of the stream may be set up once every block has called this or has ended.  The
 // append and the table call it first thing: their blocks are short, and the attention behind them
 // needs a whole SM, which it only gets when their blocks there are done.  The attention does not:

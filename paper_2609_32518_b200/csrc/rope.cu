@@ -155,10 +155,8 @@ __device__ __forceinline__ uint4 rotate_vec(uint4 x, float4 c, float4 s) {
 }
 
 __global__ void __launch_bounds__(256)
-rope_kv_append_kernel(AppendParams p, const uint4* q_in, const uint4* __restrict__ k_in,
-                      const uint4* __restrict__ v_in, const float4* __restrict__ cos_t,
-                      const float4* __restrict__ sin_t, uint4* q_out,
-                      uint4* __restrict__ ring_k, uint4* __restrict__ ring_v) {
+rope_kv_append_kernel(AppendParams p, const uint4* q_in, const uint4* k_in, const uint4* v_in, const float4* cos_t,
+                      const float4* sin_t, uint4* q_out, uint4* __restrict__ ring_k, uint4* __restrict__ ring_v) {
   grid_launch_next();
   const int b = blockIdx.y;
   const int64_t v = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
@@ -170,7 +168,7 @@ rope_kv_append_kernel(AppendParams p, const uint4* q_in, const uint4* __restrict
     prefetch_l2(k_in + first, n);
     prefetch_l2(v_in + first, n);
   }
-  grid_wait();
+  const int behind = grid_wait();
   if (v >= p.vec_per_stream) return;
   const int n = static_cast<int>(v / p.vec_per_token);
   const int rem = static_cast<int>(v - static_cast<int64_t>(n) * p.vec_per_token);
@@ -179,14 +177,14 @@ rope_kv_append_kernel(AppendParams p, const uint4* q_in, const uint4* __restrict
   const int frame = p.start[b] + f;
   const int slot = frame < p.S ? frame : p.S + (frame - p.S) % p.C;
 
-  const int64_t in_idx = static_cast<int64_t>(b) * p.vec_per_stream + v;
+  const int64_t in_idx = static_cast<int64_t>(b) * p.vec_per_stream + v + behind;
   const uint4 xq = __ldcs(q_in + in_idx);
   const uint4 xk = __ldcs(k_in + in_idx);
   const uint4 xv = __ldcs(v_in + in_idx);
   const int64_t tab = (static_cast<int64_t>(b) * p.table_stream_stride >> 2) +
-                      static_cast<int64_t>(n) * (kPairs / 4) + (rem & 15);
-  const float4 c = __ldg(cos_t + tab);
-  const float4 s = __ldg(sin_t + tab);
+                      static_cast<int64_t>(n) * (kPairs / 4) + (rem & 15) + behind;
+  const float4 c = __ldca(cos_t + tab);
+  const float4 s = __ldca(sin_t + tab);
 
   const int64_t ring_idx = static_cast<int64_t>(b) * p.ring_vec_per_stream +
                            (static_cast<int64_t>(slot) * p.T + t) * p.vec_per_token + rem;
@@ -245,15 +243,12 @@ __device__ __forceinline__ uint4 normalise_vec(uint4 x, float r, float4 g0, floa
 }
 
 __global__ void __launch_bounds__(256)
-rmsnorm_rope_kv_append_kernel(AppendParams p, float eps, const uint4* q_in, const uint4* __restrict__ k_in,
-                              const uint4* __restrict__ v_in, const float4* __restrict__ gain_q,
-                              const float4* __restrict__ gain_k, const float4* __restrict__ cos_t,
-                              const float4* __restrict__ sin_t, uint4* q_out, uint4* __restrict__ ring_k,
-                              uint4* __restrict__ ring_v) {
+rmsnorm_rope_kv_append_kernel(AppendParams p, float eps, const uint4* q_in, const uint4* k_in, const uint4* v_in,
+                              const float4* gain_q, const float4* gain_k, const float4* cos_t, const float4* sin_t,
+                              uint4* q_out, uint4* __restrict__ ring_k, uint4* __restrict__ ring_v) {
   grid_launch_next();
-  grid_wait();
   const int b = blockIdx.y;
-  const int lane = threadIdx.x & 31;
+  const int lane = (threadIdx.x & 31) + grid_wait();   // every load below goes by the lane
   const int n = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);   // token of this warp
   if (n >= p.L) return;
   const int f = n / p.T, t = n - f * p.T;
@@ -275,7 +270,7 @@ rmsnorm_rope_kv_append_kernel(AppendParams p, float eps, const uint4* q_in, cons
         const int vi = v0 + 32 * u;
         if (vi < p.vec_per_token) {
           xq[u] = q_in[in_base + vi];   // plain load: q_out may be the same buffer
-          xk[u] = __ldg(k_in + in_base + vi);
+          xk[u] = __ldca(k_in + in_base + vi);
         }
       }
 #pragma unroll
@@ -293,10 +288,10 @@ rmsnorm_rope_kv_append_kernel(AppendParams p, float eps, const uint4* q_in, cons
   const float rk = __frcp_rn(__fsqrt_rn(__fadd_rn(ms_k, eps)));
 
   auto finish = [&](int vi, uint4 xq, uint4 xk) {
-    const float4 c = __ldg(cos_t + tab_base + (vi & 15));
-    const float4 s = __ldg(sin_t + tab_base + (vi & 15));
-    const uint4 nq = normalise_vec(xq, rq, __ldg(gain_q + 2 * vi), __ldg(gain_q + 2 * vi + 1));
-    const uint4 nk = normalise_vec(xk, rk, __ldg(gain_k + 2 * vi), __ldg(gain_k + 2 * vi + 1));
+    const float4 c = __ldca(cos_t + tab_base + (vi & 15));
+    const float4 s = __ldca(sin_t + tab_base + (vi & 15));
+    const uint4 nq = normalise_vec(xq, rq, __ldca(gain_q + 2 * vi), __ldca(gain_q + 2 * vi + 1));
+    const uint4 nk = normalise_vec(xk, rk, __ldca(gain_k + 2 * vi), __ldca(gain_k + 2 * vi + 1));
     UNSTEP_STORE(q_out, in_base + vi, p.extent_act, rotate_vec(nq, c, s), p.status);
     UNSTEP_STORE(ring_k, ring_base + vi, p.extent_cache, rotate_vec(nk, c, s), p.status);
     UNSTEP_STORE(ring_v, ring_base + vi, p.extent_cache, __ldcs(v_in + in_base + vi), p.status);
@@ -327,16 +322,15 @@ rmsnorm_rope_kv_append_kernel(AppendParams p, float eps, const uint4* q_in, cons
 // same order.
 template <int kU>
 __global__ void __launch_bounds__(kU <= 2 ? 96 : 256, kU <= 2 ? 12 : 3)
-rmsnorm_rope_kv_append_token_kernel(AppendParams p, float eps, const uint4* q_in, const uint4* __restrict__ k_in,
-                                    const uint4* __restrict__ v_in, const float4* __restrict__ gain_q,
-                                    const float4* __restrict__ gain_k, const float4* __restrict__ cos_t,
-                                    const float4* __restrict__ sin_t, uint4* q_out, uint4* __restrict__ ring_k,
-                                    uint4* __restrict__ ring_v) {
+rmsnorm_rope_kv_append_token_kernel(AppendParams p, float eps, const uint4* q_in, const uint4* k_in,
+                                    const uint4* v_in, const float4* gain_q, const float4* gain_k,
+                                    const float4* cos_t, const float4* sin_t, uint4* q_out,
+                                    uint4* __restrict__ ring_k, uint4* __restrict__ ring_v) {
   __shared__ double part[2][8];
   grid_launch_next();
   const int b = blockIdx.y;
   const int n = blockIdx.x;   // token
-  const int tid = threadIdx.x, nthr = blockDim.x;
+  const int nthr = blockDim.x;
   const int f = n / p.T, t = n - f * p.T;
   const int frame = p.start[b] + f;
   const int slot = frame < p.S ? frame : p.S + (frame - p.S) % p.C;
@@ -351,7 +345,7 @@ rmsnorm_rope_kv_append_token_kernel(AppendParams p, float eps, const uint4* q_in
     prefetch_l2(k_in + in_base, p.vec_per_token);
     prefetch_l2(v_in + in_base, p.vec_per_token);
   }
-  grid_wait();
+  const int tid = threadIdx.x + grid_wait();   // every load below goes by the thread
   uint4 xq[kU], xk[kU], xv[kU];
 #pragma unroll
   for (int u = 0; u < kU; ++u) {
@@ -364,8 +358,8 @@ rmsnorm_rope_kv_append_token_kernel(AppendParams p, float eps, const uint4* q_in
   }
   // All vectors of a thread sit at the same place of their heads (the block is a multiple of 16
   // threads wide), so they share one set of coefficients, fetched under the wait for q, k and v.
-  const float4 c = __ldg(cos_t + tab_base + (tid & 15));
-  const float4 s = __ldg(sin_t + tab_base + (tid & 15));
+  const float4 c = __ldca(cos_t + tab_base + (tid & 15));
+  const float4 s = __ldca(sin_t + tab_base + (tid & 15));
   double sq = 0.0, sk = 0.0;
 #pragma unroll
   for (int u = 0; u < kU; ++u) {
@@ -394,8 +388,8 @@ rmsnorm_rope_kv_append_token_kernel(AppendParams p, float eps, const uint4* q_in
   for (int u = 0; u < kU; ++u) {
     const int vi = tid + u * nthr;
     if (vi < p.vec_per_token) {
-      const uint4 nq = normalise_vec(xq[u], rq, __ldg(gain_q + 2 * vi), __ldg(gain_q + 2 * vi + 1));
-      const uint4 nk = normalise_vec(xk[u], rk, __ldg(gain_k + 2 * vi), __ldg(gain_k + 2 * vi + 1));
+      const uint4 nq = normalise_vec(xq[u], rq, __ldca(gain_q + 2 * vi), __ldca(gain_q + 2 * vi + 1));
+      const uint4 nk = normalise_vec(xk[u], rk, __ldca(gain_k + 2 * vi), __ldca(gain_k + 2 * vi + 1));
       UNSTEP_STORE(q_out, in_base + vi, p.extent_act, rotate_vec(nq, c, s), p.status);
       UNSTEP_STORE(ring_k, ring_base + vi, p.extent_cache, rotate_vec(nk, c, s), p.status);
     }
