@@ -219,9 +219,11 @@ int unstep_window_attn_noalloc(const unstep_shape_t* shape, const int32_t* start
  *
  * The launch is cut into work items (stream, head, pair of 128-query tiles); an item has one step
  * per 128-key tile of its window.  Each of at most `max_workers` workers (one per SM) first takes
- * whole items round-robin; what is left over is one sequence of steps cut into equal contiguous
- * shares, so an item there may be split along its keys into parts that different workers compute
- * and the last one to finish merges.
+ * whole items round-robin (a launch of no more items than workers has no such rounds).  What is left
+ * over is split along the keys in one of two ways, whichever is estimated to be shorter: every item
+ * into the same number of parts (one or more), one part per worker; or all its steps as one sequence
+ * cut into equal contiguous shares, one per worker, so that an item falls into as many parts as shares
+ * touch it.  The parts of an item are merged by the worker that finishes last.
  *
  *   segs     : HOST int32 [max_segs][10], written (may be NULL when max_segs is 0).  One row per
  *              segment in the order the worker walks them: worker, stream, head, query pair,

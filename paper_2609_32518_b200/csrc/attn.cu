@@ -106,8 +106,8 @@ struct Waiter {
 };
 
 // The CTA owns 384 x 168 registers; 128 x 72 for the service warps + 256 x 216 for the softmax
-// warps uses exactly that (an increase that the pool cannot satisfy would wait forever).  216 is
-// what the softmax warps need to run without spills.
+// warps uses exactly that (an increase that the pool cannot satisfy would wait forever).  With 216 the
+// softmax warps spill one register (ptxas: 4 bytes of stores, 12 of loads).
 constexpr int kRegsService = 72, kRegsSoftmax = 216;
 static_assert(128 * kRegsService + 256 * kRegsSoftmax <= 384 * 168, "register redistribution exceeds the CTA's allocation");
 static_assert(kRegsService == 72 && kRegsSoftmax == 216, "keep the setmaxnreg literals below in step");
@@ -992,10 +992,14 @@ static int window_attn_run(const unstep_shape_t* shape, const int32_t* start_fra
         !make_map(&tm_v, vb, 5, rdims, rstr, 2) || !make_map(&tm_kf, kb, 4, fdims, fstr, 2) ||
         !make_map(&tm_vf, vb, 4, fdims, fstr, 2))
       return UNSTEP_ERR_CUDA;
-    // Set up under the append before it where the launch is short: five heads and two streams
-    // 36 -> 32 us with the append, 57 steps per worker 166.7 -> 164.7 us.  Long launches run at the
-    // power cap, where the saved 2 us of idling show as a lower clock: 394 steps per worker took 898 us
-    // overlapped and 886 not, six layers of 171 steps 2473 and 2411.
+    // Set up under the append before it where the launch is short.  Append and attention, us not
+    // overlapped -> overlapped, by steps per worker: in runs of 20 (full clock) 24: 78.9 -> 76.5, 35:
+    // 94.6 -> 92.6, 57: 143.1 -> 142.3, 114: 242.0 -> 240.6, 226: 446.1 -> 445.5, 394: 754.9 -> 763.7; run
+    // on end at the power cap 24: 80.2 -> 79.8 (1912 -> 1867 MHz), 57: 155.2 -> 155.8 (1792 -> 1776), 114:
+    // 276.7 -> 276.6 (1702 -> 1688), 169: 395.4 -> 398.6 (1680 -> 1652), 394: 880.4 -> 895.9 (1635 -> 1605).
+    // The overlap saves 1.5-6 thousand cycles of a launch at any length; at the cap the clock falls for
+    // the idling it takes away.  The line lies about where the gain of short runs (0.6 % at 57 steps) has
+    // come down to the loss of runs at the cap (0.4 %).
     const bool brief = p.all_steps < static_cast<int64_t>(kOverlapSteps) * p.n_workers;
     const cudaError_t err = launch_overlapped(brief, window_attn_kernel, p.n_workers, kThreads, kAttnSmemBytes, st, tm_q,
                                               tm_k, tm_v, tm_kf, tm_vf, p, ob);

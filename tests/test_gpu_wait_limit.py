@@ -1,5 +1,6 @@
 """Bounded device-side waits: a wait that can never be satisfied gives up, reports it through
-the status word and leaves the context usable (no trap, no hang)."""
+the status word and leaves the context usable (no trap, no hang).  The probe is the wait alone; what the
+attention kernel's roles do behind a wait that gave up is shown on the CPU (test_hand_over.py)."""
 
 import time
 
@@ -36,5 +37,5 @@ def test_shutdown_frees_scratch_and_the_library_keeps_working():
     before = torch.cuda.mem_get_info()[0]
     U.shutdown()
     after = torch.cuda.mem_get_info()[0]
-    assert after >= before                      # the scratch (tens of MB) went back to the driver
+    assert after >= before + (30 << 20)         # the scratch (39 MB a stream) went back to the driver
     run(W.WORKLOADS["cfg1_wrapped"])            # and is made again on demand
