@@ -50,7 +50,7 @@ L2_BYTES = 126e6
 # captures of that kernel at that workload (the L2 state at the start of the launch differs)
 ATTN_DRAM_TRAFFIC = {"bytes": 336_867_072, "capture": "profiles/window_attn_cfg2_ncu_full.txt",
                      "range_over_captures_mb": [286, 402],
-                     "note": "cold L2 (every step on another working set); 286 MB when the cache of the step before is reused"}
+                     "note": "one launch under ncu, which replays it: parts of K and V may be in L2 when it begins"}
 
 
 def load_peaks():
