@@ -48,7 +48,7 @@ L2_BYTES = 126e6
 # dram__bytes_read.sum + dram__bytes_write.sum of one window_attn launch at cfg2 from the ncu
 # capture summarised in profiles/window_attn_cfg2_ncu_full.txt, and the range seen over all
 # captures of that kernel at that workload (the L2 state at the start of the launch differs)
-ATTN_DRAM_TRAFFIC = {"bytes": 336_867_072, "capture": "profiles/window_attn_cfg2_ncu_full.txt",
+ATTN_DRAM_TRAFFIC = {"bytes": 336_592_128, "capture": "profiles/window_attn_cfg2_ncu_full.txt",
                      "range_over_captures_mb": [286, 402],
                      "note": "one launch under ncu, which replays it: parts of K and V may be in L2 when it begins"}
 
