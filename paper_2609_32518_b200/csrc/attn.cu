@@ -3,14 +3,23 @@
 // Persistent, warp-specialised kernel, one CTA per SM:
 //   warps 0-3   softmax of query tile 0, one thread per query row
 //   warps 4-7   softmax of query tile 1
-//   warp  8, 9  tcgen05.mma issuers of query tile 0 and 1 (one lane each); warp 8 owns TMEM
+//   warp  8     issues S = Q K^T of both query tiles; owns TMEM
+//   warp  9     issues O += P V of both query tiles
 //   warp  10    TMA producer (one lane)
 // A work item is (stream, head, pair of 128-query tiles): both tiles share every K/V
-// tile.  The two tiles run half a period apart: while one is in its exponentials (MUFU
-// pipe) the other's P V and next Q K^T run on the tensor core.  A small token ring keeps
-// them apart: the MMA issuers take turns on the tensor pipe.  S = Q K^T and O += P V
-// accumulate in TMEM; P (bf16) is written back over S and fed to the second MMA straight
-// from TMEM.
+// tile.  S, P (bf16) and O live in TMEM: one S for both query tiles in turn, a P and an O for each.
+// A softmax group takes its scores into registers at once and gives S back, so that the tensor core
+// computes the other tile's scores, and then this tile's next ones, while the exponentials run; P V
+// follows when P is there.  So the next scores are there when a group is done with its tile, and the
+// two groups share the MUFU pipe without waiting for the tensor core.  (With an S for each tile and P over
+// S, a tile's next Q K^T had to wait for its P V: exponentials, hand-over, P V and Q K^T were one
+// chain of ~3500 clk per key tile.  12 heads, 4680 queries, 32760 keys: 1422 -> 1184 thousand
+// cycles, 878 -> 800 us run on end at the power cap, 754 -> 693 us in a burst.)
+//
+// What a group does per key tile is as long as the period, so it counts how fast it is fetched: its
+// loop over the full tiles is kept short and free of taken branches (rare cases are out of line, one
+// masked variant takes first and ragged tiles).  The same pipeline with the variants side by side in one loop
+// waited 640 clk per key tile for instructions and took 1425 thousand cycles.
 //
 // The attended frames are at most three runs of consecutive cache slots (sink prefix, ring
 // up to its end, ring from its start).  Key tiles are cut from the runs through a flat
@@ -70,7 +79,8 @@ constexpr int kHalfBytes = 128 * 64 * 2;    // one TMA box: 128 rows x 64 bf16 (
 constexpr int kTileBytes = 2 * kHalfBytes;  // 128 x 128 bf16
 constexpr int kStages = 5;                  // 32 KB buffers shared by the K and V tiles
 constexpr int kThreads = 384;
-constexpr int kTmemCols = 512;              // S0 | S1 | O0 | O1, 128 fp32 columns each
+constexpr int kTmemCols = 512;
+constexpr int kTmemS = 0, kTmemP = 128, kTmemO = 256;   // S (128 columns) | P0 | P1 (64 each) | O0 | O1 (128 each)
 constexpr long long kWaitCycles = 2000000000LL;  // about a second: then give up, never hang
 
 constexpr int kSmemQ = 0;
@@ -89,8 +99,12 @@ struct Waiter {
   // Bounded wait: the hardware parks the thread between polls; the clock and the CTA's abort
   // flag are only looked at every 32 polls so that a waiting warp leaves the issue slots alone.
   __device__ __forceinline__ bool wait(uint32_t bar, uint32_t parity) const {
-    if (mbar_try_wait(bar, parity)) return true;
+    if (__builtin_expect(mbar_try_wait(bar, parity) != 0, 1)) return true;
+    return wait_long(bar, parity);
+  }
+  __device__ __forceinline__ bool wait_long(uint32_t bar, uint32_t parity) const {
     const long long t0 = clock64();
+#pragma unroll 1
     for (uint32_t spin = 1;; ++spin) {
       if (mbar_try_wait_hint(bar, parity, 2000u)) return true;
       if ((spin & 31u) == 0u) {
@@ -103,11 +117,14 @@ struct Waiter {
       }
     }
   }
+  // The same by all lanes of a warp, with the warp's answer.
+  __device__ __forceinline__ bool wait_warp(uint32_t bar, uint32_t parity) const {
+    return __all_sync(0xFFFFFFFFu, wait(bar, parity));
+  }
 };
 
 // The CTA owns 384 x 168 registers; 128 x 72 for the service warps + 256 x 216 for the softmax
-// warps uses exactly that (an increase that the pool cannot satisfy would wait forever).  With 216 the
-// softmax warps spill one register (ptxas: 4 bytes of stores, 12 of loads).
+// warps uses exactly that (an increase that the pool cannot satisfy would wait forever).  Nothing spills.
 constexpr int kRegsService = 72, kRegsSoftmax = 216;
 static_assert(128 * kRegsService + 256 * kRegsSoftmax <= 384 * 168, "register redistribution exceeds the CTA's allocation");
 static_assert(kRegsService == 72 && kRegsSoftmax == 216, "keep the setmaxnreg literals below in step");
@@ -116,9 +133,7 @@ __device__ __forceinline__ void reg_alloc_softmax() { asm volatile("setmaxnreg.i
 
 // --------------------------------------------------------------------------------------
 // Softmax of one 128 x 128 score tile with one thread per query row (a warpgroup per query
-// tile); no data crosses threads.  The caller has seen S of this tile complete, which (the
-// tensor pipe runs in issue order) also means the previous P V into O has landed, so O may be
-// rescaled here without another wait.
+// tile); no data crosses threads.
 // --------------------------------------------------------------------------------------
 __device__ __forceinline__ void group_barrier(int a) {
   asm volatile("bar.sync %0, 128;" ::"r"(kGroupBarrier + a) : "memory");
@@ -132,24 +147,24 @@ __device__ __forceinline__ uint32_t group_count(int a, bool pred) {
   return n;
 }
 
-// Hand-over of P and of the tensor turn through named barriers.  An mbarrier lives in shared
+// Hand-over of P to the P V issuer, and of the read S back to the Q K^T issuer, through named barriers.  An mbarrier lives in shared
 // memory, whose bandwidth the MMA operands of Q K^T use up: an arrive or a try_wait there took
 // 120-270 clk, several times on every key tile's critical path; a named barrier takes 25-60 clk.
 // A named barrier has no bounded wait, so every warp keeps meeting them, once per key tile of its
-// segments, after it has given up on an mbarrier as well; handover.h says why all of them end.  The
-// turns alternate strictly between two warps that take and pass them whether or not they gave up.
-__device__ __forceinline__ void p_ready_sync(int a, uint32_t tile) {   // issuer a: P of group a's tile-th key tile is in TMEM
+// segments, after it has given up on an mbarrier as well; handover.h says why all of them end.
+__device__ __forceinline__ void p_ready_sync(int a, uint32_t tile) {   // P V issuer: P of group a's tile-th key tile is in TMEM
   asm volatile("bar.sync %0, 160;" ::"r"(p_ready_barrier(a, tile)) : "memory");
 }
 __device__ __forceinline__ void p_ready_pass(int a, uint32_t tile, bool gave_up) {   // a warp of softmax group a
   if (p_ready_waits(gave_up)) p_ready_sync(a, tile);
   else asm volatile("bar.arrive %0, 160;" ::"r"(p_ready_barrier(a, tile)) : "memory");
 }
-__device__ __forceinline__ void turn_sync(int a) {        // issuer a waits for the tensor pipe
-  asm volatile("bar.sync %0, 64;" ::"r"(kTurnBarrier + a) : "memory");
+__device__ __forceinline__ void s_free_sync(int a, uint32_t tile) {   // Q K^T issuer: group a has read S of its tile-th key tile
+  asm volatile("bar.sync %0, 160;" ::"r"(s_free_barrier(a, tile)) : "memory");
 }
-__device__ __forceinline__ void turn_pass(int a) {        // issuer a hands it to the other one
-  asm volatile("bar.arrive %0, 64;" ::"r"(kTurnBarrier + 1 - a) : "memory");
+__device__ __forceinline__ void s_free_pass(int a, uint32_t tile, bool gave_up) {   // a warp of softmax group a
+  if (p_ready_waits(gave_up)) s_free_sync(a, tile);
+  else asm volatile("bar.arrive %0, 160;" ::"r"(s_free_barrier(a, tile)) : "memory");
 }
 
 // Exponentials of 32 score columns (registers s) into 16 bf16 pairs (p) and the packed sums.
@@ -180,123 +195,88 @@ __device__ __forceinline__ void mask_block32(uint32_t* s, int col0, int nvalid) 
   }
 }
 
-// Exponentials of the 128 scores of a row (TMEM columns t_S .. t_S + 127) against the reference
-// maximum: the scores come in blocks of 32 columns, each fetched while the block before it is
-// exponentiated (a block keeps the MUFU pipe busy for 256 clk, longer than a TMEM load takes), so
-// that only the first block's load is exposed.  Leaves P (bf16 pairs) in p0 (keys 0..63) and p1
-// (keys 64..127) and returns the row's sum of P.
-template <bool kMasked, int kCols>
-__device__ __forceinline__ float exp_row(uint32_t t_S, float c, float neg_ms, int nvalid, uint32_t* p0,
-                                         uint32_t* p1) {
-  const uint64_t c2 = pack_f32x2(c, c);
-  const uint64_t nm2 = pack_f32x2(neg_ms, neg_ms);
-  uint64_t acc[4] = {0ull, 0ull, 0ull, 0ull};
-  uint32_t a[32], b[32];
-  tmem_ld32(t_S, a);
-  tc_wait_ld32(a);
-  tmem_ld32(t_S + 32, b);
-  mask_block32<kMasked>(a, 0, nvalid);
-  exp_block32(a, p0, c2, nm2, acc);
-  tc_wait_ld32(b);
-  if (kCols > 64) tmem_ld32(t_S + 64, a);
-  mask_block32<kMasked>(b, 32, nvalid);
-  exp_block32(b, p0 + 16, c2, nm2, acc);
-  if (kCols > 64) {
-    tc_wait_ld32(a);
-    tmem_ld32(t_S + 96, b);
-    mask_block32<kMasked>(a, 64, nvalid);
-    exp_block32(a, p1, c2, nm2, acc);
-    tc_wait_ld32(b);
-    mask_block32<kMasked>(b, 96, nvalid);
-    exp_block32(b, p1 + 16, c2, nm2, acc);
-  }
-  const uint64_t t = add_f32x2(add_f32x2(acc[0], acc[1]), add_f32x2(acc[2], acc[3]));
-  float t0, t1;
-  unpack_f32x2(t, t0, t1);
-  return t0 + t1;
-}
+// One key tile of a row: scores from TMEM (columns t_S ..) into registers, S given back, exponentials against
+// the row's reference maximum, P (bf16 pairs, keys 0.. from column t_P on) handed over.  False if a wait gave up;
+// S has been given back then, P has not been passed.
+//
+// The reference is the maximum of the segment's first key tile, so that the largest weight there is exactly 1 (with
+// the maximum of 32 scores the error of peaked rows against float64 grew from 2.17e-3 to 2.32e-3).  It moves
+// only where a later tile has a score more than kJump = 64 (log2 units) above it: up to there P (bf16)
+// and the float32 sums are as accurate as near 1 (same relative precision, no overflow: 32760 keys of 2^64
+// times |v| stay far below 2^127), and what was accumulated before such a jump is negligible exactly as in
+// the true softmax.  The scores have left TMEM by the time a sum of P could tell, so the maximum is looked
+// for in front: 64 three-input maxima in the shadow of the other group's exponentials.
+//
+// P may be stored, and O rescaled, once the P V of the tile before has run.  That barrier, and the one of the next
+// tile's scores, are looked at once, ahead of time: the look takes 100-200 clk under the MMAs' traffic, and
+// almost always finds what it looks for.
+// Tiles of at most 64 keys (frames of up to 64 tokens, the end of a run) leave the other half of the columns
+// alone.
+constexpr float kJump = 64.f;
 
-// Row maximum of the 128 scores in TMEM.
-template <bool kMasked, int kCols>
-__device__ __forceinline__ float max_row(uint32_t t_S, int nvalid) {
-  uint32_t hi[64], lo[64];
-  if (kCols > 64) {
-    tmem_ld32(t_S + 64, hi);
-    tmem_ld32(t_S + 96, hi + 32);
-  }
-  tmem_ld32(t_S, lo);
-  tmem_ld32(t_S + 32, lo + 32);
-  tc_wait_ld32(lo);
-  reg_fence32(lo + 32);
-  mask_block32<kMasked>(lo, 0, nvalid);
-  mask_block32<kMasked>(lo + 32, 32, nvalid);
-  float m = fmaxf(max_block32(lo), max_block32(lo + 32));
-  if (kCols > 64) {
-    reg_fence32(hi);
-    reg_fence32(hi + 32);
-    mask_block32<kMasked>(hi, 64, nvalid);
-    mask_block32<kMasked>(hi + 32, 96, nvalid);
-    m = fmaxf(m, fmaxf(max_block32(hi), max_block32(hi + 32)));
-  }
-  return m;
-}
-
-// Only the first key tile of a segment looks for the row maximum before its exponentials.
-// (The maximum of 32 scores would do as a reference and saves 350 clk a segment, but then the largest
-// weight is no longer exactly 1 and rounds to bf16 like the others: against float64 the error of
-// peaked rows grew from 2.17e-3 to 2.32e-3.)  Every later tile exponentiates against that reference
-// straight away and looks at the row's sum of P afterwards.  P is positive, so a sum of at most
-// kOptimisticLimit = 2^64 means that no score was more than 64 (log2 units) above the reference: P
-// (bf16) and the float32 sums are as accurate at that magnitude as near 1 (same relative precision, no
-// overflow: 128 keys of 2^64 times |v| stay far below 2^127), and everything accumulated before such a
-// jump is negligible exactly as in the true softmax.  Otherwise (scores more than 64 above the first
-// tile's maximum, or an overflow to inf) the warp finds the tile's true maximum, rescales O and l, and
-// redoes the exponentials; the scores are still in TMEM, because P is only stored at the very end.
-// Scores are read from TMEM in blocks to keep the register count down; P (bf16 pairs) overwrites
-// score columns 0..63.  Tiles of at most 64 keys (frames of up to 64 tokens, the end of a run) leave the
-// other half of the columns alone: append and attention of a toy layer with 64-token frames 16.1 ->
-// 14.7 us.  The redo is the second round of a loop, so that each variant holds its exponentials once.
-constexpr float kOptimisticLimit = 18446744073709551616.f;   // 2^64
-
-template <bool kMasked, int kCols>   // kCols: score columns that hold keys, 64 or 128
-__device__ __forceinline__ void softmax_row_tile(uint32_t t_S, uint32_t t_O, float c, int nvalid,
-                                                 bool first, float& m_run, float& l_run,
-                                                 int a, uint32_t tile) {
-  if (first) m_run = max_row<kMasked, kCols>(t_S, nvalid);
+template <bool kMasked, int kCols, bool kTight>   // kCols: score columns that hold keys, 64 or 128; kTight: not a segment's first tile
+__device__ __forceinline__ bool softmax_row_tile(uint32_t t_S, uint32_t t_P, uint32_t t_O, float c, int nvalid,
+                                                 bool first, float& m_run, float& l_run, int a, uint32_t tile,
+                                                 const Waiter& w, uint32_t bar_pv, uint32_t bar_s, uint32_t& s_seen) {
+  uint32_t s[kCols], p[kCols / 2];
+#pragma unroll
+  for (int q = 0; q < kCols / 32; ++q) tmem_ld32(t_S + 32 * q, s + 32 * q);
+  tc_wait_ld32(s);
+#pragma unroll
+  for (int q = 1; q < kCols / 32; ++q) reg_fence32(s + 32 * q);
+  tc_fence_before();
+  s_free_pass(a, tile, false);
   TRACE(a, tile, 2);
-  uint32_t p0[32], p1[32];
-  float sum;
-  bool redone = false;
-#pragma unroll 1
-  for (;;) {   // at most twice
-    sum = exp_row<kMasked, kCols>(t_S, c, -m_run * c, nvalid, p0, p1);
-    const bool redo = !first && !(sum <= kOptimisticLimit);   // also taken for inf and NaN
-    if (redone || !__any_sync(0xFFFFFFFFu, redo)) break;
-    redone = true;
-    const float mx = max_row<kMasked, kCols>(t_S, nvalid);
+#pragma unroll
+  for (int q = 0; q < kCols / 32; ++q) mask_block32<kMasked>(s + 32 * q, 32 * q, nvalid);
+  float mx = max_block32(s);
+#pragma unroll
+  for (int q = 1; q < kCols / 32; ++q) mx = fmaxf(mx, max_block32(s + 32 * q));
+  if (!kTight && first) {
+    m_run = mx;
+  } else if (__builtin_expect(__any_sync(0xFFFFFFFFu, (mx - m_run) * c > kJump), 0)) {
+    if (!w.wait_warp(bar_pv, (tile - 1) & 1)) return false;
+    tc_fence_after();
     float alpha = 1.f;
     if (mx > m_run) {
       alpha = ex2((m_run - mx) * c);
       m_run = mx;
       l_run *= alpha;
     }
+#pragma unroll 1
+    for (int q = 0; q < 16; ++q) {
+      uint32_t o[8];
+      tmem_ld8(t_O + q * 8, o);
+      tc_wait_ld8(o);
 #pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      uint32_t o[32];
-      tmem_ld32(t_O + q * 32, o);
-      tc_wait_ld32(o);
-#pragma unroll
-      for (int i = 0; i < 32; ++i) o[i] = __float_as_uint(__uint_as_float(o[i]) * alpha);
-      tmem_st32(t_O + q * 32, o);
+      for (int i = 0; i < 8; ++i) o[i] = __float_as_uint(__uint_as_float(o[i]) * alpha);
+      tmem_st8(t_O + q * 8, o);
     }
   }
-  tmem_st32(t_S, p0);        // P of keys 0..63 over score columns 0..31
-  if (kCols > 64) tmem_st32(t_S + 32, p1);   // P of keys 64..127 over score columns 32..63
+  const uint64_t c2 = pack_f32x2(c, c), nm2 = pack_f32x2(-m_run * c, -m_run * c);
+  uint64_t acc[4] = {0ull, 0ull, 0ull, 0ull};
+  TRACE(a, tile, 3);
+#pragma unroll
+  for (int q = 0; q < kCols / 32 - 1; ++q) exp_block32(s + 32 * q, p + 16 * q, c2, nm2, acc);
+  uint32_t pv_seen = mbar_test(bar_pv, (tile - 1) & 1);
+  exp_block32(s + kCols - 32, p + kCols / 2 - 16, c2, nm2, acc);
+  if ((kTight || !first) && __builtin_expect(!__all_sync(0xFFFFFFFFu, pv_seen), 0)) {
+    if (!w.wait_warp(bar_pv, (tile - 1) & 1)) return false;
+  }
+  tc_fence_after();
+  TRACE(a, tile, 4);
+  if (kCols > 64) tmem_st32(t_P, p);
+  s_seen = mbar_test(bar_s, (tile + 1) & 1);
+  tmem_st32(t_P + kCols / 2 - 32, p + kCols / 2 - 32);
   tc_wait_st();
   tc_fence_before();
   p_ready_pass(a, tile, false);
   TRACE(a, tile, 5);
-  l_run += sum;
+  const uint64_t t2 = add_f32x2(add_f32x2(acc[0], acc[1]), add_f32x2(acc[2], acc[3]));
+  float t0, t1;
+  unpack_f32x2(t2, t0, t1);
+  l_run += t0 + t1;
+  return true;
 }
 
 // Real keys of key tile j of a stream, without the divisions of tile_info: only the last tile of a
@@ -313,6 +293,15 @@ struct ValidKeys {
       j_last[r] = any ? end - 1 : -1;
       v_last[r] = p.run_rows[b][r] - kTileN * (end - begin - 1);
     }
+  }
+  // first tile from j on that is ragged, at most `end`
+  __device__ __forceinline__ int full_until(int j, int end) const {
+    if (dflt < kTileN) return j;
+    int k = end;
+#pragma unroll
+    for (int r = 0; r < 3; ++r)
+      if (j_last[r] >= j && j_last[r] < k && v_last[r] < kTileN) k = j_last[r];
+    return k;
   }
   __device__ __forceinline__ int operator()(int j) const {
     return j == j_last[0] ? v_last[0] : (j == j_last[1] ? v_last[1] : (j == j_last[2] ? v_last[2] : dflt));
@@ -335,17 +324,17 @@ window_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
   const uint32_t sKV = smem_base + kSmemKV;
   const uint32_t sBar = smem_base + kSmemBar;
   // mbarriers (8 bytes each)
-  const uint32_t bar_q_full = sBar;                          // [2]  TMA -> MMA warp a
-  const uint32_t bar_q_empty = sBar + 16;                    // [2]  MMA warp a -> TMA
-  const uint32_t bar_kv_full = sBar + 32;                    // [kStages] TMA -> both MMA warps
-  const uint32_t bar_kv_empty = sBar + 32 + 8 * kStages;     // [kStages] both MMA warps -> TMA
-  const uint32_t bar_s_full = sBar + 32 + 16 * kStages;      // [2]  MMA warp a -> softmax a
-  const uint32_t bar_o_final = bar_s_full + 16;              // [2]  MMA warp a -> softmax a
+  const uint32_t bar_q_full = sBar;                          // [2]  TMA -> Q K^T issuer
+  const uint32_t bar_q_empty = sBar + 16;                    // [2]  Q K^T issuer -> TMA
+  const uint32_t bar_kv_full = sBar + 32;                    // [kStages] TMA -> the issuer that reads the stage
+  const uint32_t bar_kv_empty = sBar + 32 + 8 * kStages;     // [kStages] that issuer -> TMA
+  const uint32_t bar_s_full = sBar + 32 + 16 * kStages;      // [2]  Q K^T issuer -> softmax a
+  const uint32_t bar_pv_done = bar_s_full + 16;              // [2]  P V issuer -> softmax a
   volatile uint32_t* tmem_slot = reinterpret_cast<volatile uint32_t*>(gen + kSmemBar + 224);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(gen + kSmemBar + 228);
 
   const int tid = threadIdx.x;
-  const int warp = tid >> 5;
+  const int warp = __shfl_sync(0xFFFFFFFFu, tid >> 5, 0);   // the same in all lanes, and known to be
   const int lane = tid & 31;
   CTRACE(0);
 
@@ -354,11 +343,11 @@ window_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
       mbar_init(bar_q_full + 8 * i, 1);
       mbar_init(bar_q_empty + 8 * i, 1);
       mbar_init(bar_s_full + 8 * i, 1);
-      mbar_init(bar_o_final + 8 * i, 1);
+      mbar_init(bar_pv_done + 8 * i, 1);
     }
     for (int i = 0; i < kStages; ++i) {
       mbar_init(bar_kv_full + 8 * i, 1);
-      mbar_init(bar_kv_empty + 8 * i, 2);
+      mbar_init(bar_kv_empty + 8 * i, 1);
     }
     *abort_flag = 0;
     mbar_fence_init();
@@ -370,7 +359,7 @@ window_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
-  const uint32_t tmem_base = *tmem_slot;
+  const uint32_t tmem_base = __shfl_sync(0xFFFFFFFFu, *tmem_slot, 0);
   // What comes before a role's grid_wait may run under the kernel before this one.  Every role waits
   // there, so that no bounded wait counts that kernel's time.
   const Waiter w{abort_flag, kWaitCycles};
@@ -401,163 +390,145 @@ window_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
           tma_load_4d(dst + kHalfBytes, &tm_q, bar, 64, s.h, n0, s.b);
           ++q_it[a];
         };
-        load_q(0);   // what the first S needs comes first: Q of tile 0, then K
-        for (int j = s.t0; j < s.t1 && ok; ++j) {
-          const TileInfo ti = tile_info(p, s.b, j);
-          for (int kv = 0; kv < 2 && ok; ++kv) {
-            if (j == s.t0 && kv == 1) load_q(1);
-            const uint32_t st = kv_it % kStages;
-            if (ok) ok = w.wait(bar_kv_empty + 8 * st, ((kv_it / kStages) & 1) ^ 1);
-            if (!ok) break;
-            const uint32_t dst = sKV + st * kTileBytes, bar = bar_kv_full + 8 * st;
-            mbar_expect_tx(bar, kTileBytes);
-            if (ti.framed) {
-              const CUtensorMap* tm = kv == 0 ? &tm_k : &tm_v;
-              tma_load_5d(dst, tm, bar, 0, s.h, ti.tok0, ti.slot, s.b);
-              tma_load_5d(dst + kHalfBytes, tm, bar, 64, s.h, ti.tok0, ti.slot, s.b);
-            } else {
-              const CUtensorMap* tm = kv == 0 ? &tm_kf : &tm_vf;
-              tma_load_4d(dst, tm, bar, 0, s.h, ti.row, s.b);
-              tma_load_4d(dst + kHalfBytes, tm, bar, 64, s.h, ti.row, s.b);
-            }
-            ++kv_it;
+        auto load_kv = [&](const TileInfo& ti, int kv) {
+          const uint32_t st = kv_it % kStages;
+          if (ok) ok = w.wait(bar_kv_empty + 8 * st, ((kv_it / kStages) & 1) ^ 1);
+          if (!ok) return;
+          const uint32_t dst = sKV + st * kTileBytes, bar = bar_kv_full + 8 * st;
+          mbar_expect_tx(bar, kTileBytes);
+          if (ti.framed) {
+            const CUtensorMap* tm = kv == 0 ? &tm_k : &tm_v;
+            tma_load_5d(dst, tm, bar, 0, s.h, ti.tok0, ti.slot, s.b);
+            tma_load_5d(dst + kHalfBytes, tm, bar, 64, s.h, ti.tok0, ti.slot, s.b);
+          } else {
+            const CUtensorMap* tm = kv == 0 ? &tm_kf : &tm_vf;
+            tma_load_4d(dst, tm, bar, 0, s.h, ti.row, s.b);
+            tma_load_4d(dst + kHalfBytes, tm, bar, 64, s.h, ti.row, s.b);
           }
+          ++kv_it;
+        };
+        load_q(0);   // what the first S needs comes first: Q of tile 0, then K
+        TileInfo ti = tile_info(p, s.b, s.t0);
+        load_kv(ti, 0);
+        load_q(1);
+        for (int j = s.t0; j < s.t1 && ok; ++j) {
+          TileInfo tn = ti;
+          if (j + 1 < s.t1) {
+            tn = tile_info(p, s.b, j + 1);
+            load_kv(tn, 0);
+          }
+          load_kv(ti, 1);
+          ti = tn;
         }
       }
-    } else if (warp <= 9) {
-      // ------------------------------------------------------------ MMA issuer of query tile a
-      // One issuing thread per query tile, on different scheduler partitions.  For each key
-      // tile: O_a += P_a V, then S_a = Q_a K_next^T.  Both warps walk the same K/V ring; a stage
-      // is released when both have retired it.  Lane 0 waits and issues; the whole warp meets
-      // the named barriers.
+    } else if (warp == 8) {
+      // ------------------------------------------------------------ Q K^T issuer
+      // The K and V tiles come in the order in which they are used: K of tile 0, then K of tile j + 1 and V
+      // of tile j.  The whole warp runs the code (the loops stay rolled: instruction fetch is scarce).
       grid_wait();
-      const int a = warp - 8;
       Sched sched(p, static_cast<int>(blockIdx.x));
       Seg s;
-      uint32_t kv_it = 0, q_it = 0, turns = 0;
-      uint32_t sp_it = 0;   // key tiles so far
+      uint32_t kv_base = 0, n0 = 0, n1 = 0, q0 = 0, q1 = 0;   // tiles and items per group
+      int before = -1;   // group whose scores are in S
       bool ok = true;
-      const bool lead = lane == 0;
-      const uint32_t idesc_pv = idesc_bf16_f32(kTileM, kHeadDim, 1);
-      const uint32_t idesc_qk_full = idesc_bf16_f32(kTileM, kTileN, 0);
-      // descriptors are built once; per instruction only the start-address field moves
-      const uint64_t dq = smem_desc_sw128(sQ + a * kTileBytes, 16, 1024);   // Q tile a, K-major
-      const uint64_t dk0 = smem_desc_sw128(sKV, 16, 1024);                  // stage 0 as a K tile
-      const uint64_t dv0 = smem_desc_sw128(sKV, kHalfBytes, 1024);          // stage 0 as a V tile (MN-major)
-      const uint32_t s_tmem = tmem_base + a * 128, o_tmem = tmem_base + 256 + a * 128;
-      const uint32_t my_s_full = bar_s_full + 8 * a;
-
-      // a ragged tile runs with N (for Q K^T) and K (for P V) rounded up to 16 keys
-      auto issue_qk = [&](uint32_t stage, int valid) {
-        const uint64_t dk = dk0 + static_cast<uint64_t>((stage * kTileBytes) >> 4);
-        const uint32_t idesc = valid == kTileN ? idesc_qk_full : idesc_bf16_f32(kTileM, (valid + 15) & ~15, 0);
-        mma_ss_k128(s_tmem, dq, dk, idesc, 0u);
-        tc_commit(my_s_full);
-      };
-      auto issue_pv_half = [&](uint64_t dv, int half, int k_steps, bool accumulate) {
-        if (k_steps >= 4 * half + 4) {
-          mma_ts_k64(o_tmem, s_tmem + 32 * half, dv + static_cast<uint64_t>(512 * half), idesc_pv,
-                     accumulate ? 1u : 0u);
-          return;
-        }
-#pragma unroll
-        for (int k = 4 * half; k < 4 * half + 4; ++k)
-          if (k < k_steps)
-            mma_ts(o_tmem, s_tmem + k * 8, dv + static_cast<uint64_t>((k * 2048) >> 4), idesc_pv,
-                   (accumulate || k > 0) ? 1u : 0u);
-      };
-
+      const uint32_t idesc_full = idesc_bf16_f32(kTileM, kTileN, 0);
+      const uint64_t dq = smem_desc_sw128(sQ, 16, 1024);    // Q tile 0, K-major
+      const uint64_t dk0 = smem_desc_sw128(sKV, 16, 1024);  // stage 0 as a K tile
       while (sched.next(s)) {
-        const bool part = a < s.nq;   // a lone last query tile leaves warp 1 only the bookkeeping
         const int n = s.t1 - s.t0;
         const ValidKeys valid_of(p, s.b);
-        int valid = valid_of(s.t0);  // real keys of the tile S is being computed for
-        if (part) {
-          if (lead && ok) ok = w.wait(bar_q_full + 8 * a, q_it & 1);
-          ++q_it;
-        }
-        uint32_t kst = kv_it % kStages;
-        if (lead && ok) ok = w.wait(bar_kv_full + 8 * kst, (kv_it / kStages) & 1);
-        ++kv_it;
-        if (lead && ok) {
-          if (part) {
-            tc_fence_after();
-            issue_qk(kst, valid);
-            tc_commit(bar_kv_empty + 8 * kst);
-            // Q is free as soon as the item's last Q K^T has run: the producer fetches the next
-            // item's Q under this item's last exponentials and P V
-            if (n == 1) tc_commit(bar_q_empty + 8 * a);
-          } else {
-            mbar_arrive(bar_kv_empty + 8 * kst);
-          }
-        }
         for (int j = 0; j < n; ++j) {
-          const int k_steps = (valid + 15) >> 4;
-          const uint32_t vst = kv_it % kStages;
-          if (lead && ok) ok = w.wait(bar_kv_full + 8 * vst, (kv_it / kStages) & 1);
-          ++kv_it;
-          const bool more = j + 1 < n;
-          if (more) {
-            valid = valid_of(s.t0 + j + 1);
-            kst = kv_it % kStages;
-            if (lead && ok) ok = w.wait(bar_kv_full + 8 * kst, (kv_it / kStages) & 1);
-            ++kv_it;
-          }
-          __syncwarp();
-          if (part) {
-            const uint64_t dv = dv0 + static_cast<uint64_t>((vst * kTileBytes) >> 4);
-            TRACE(2 + a, sp_it, 0);
-            p_ready_sync(a, sp_it);   // P of this tile is in TMEM, O rescaled if need be
-            TRACE(2 + a, sp_it, 1);
-            // The two issuers take turns with their P V + Q K^T chains: issued side by side the
-            // chains would interleave in the tensor pipe and finish together, which pulls the
-            // two query tiles into step; one after the other keeps them half a period apart.
-            if (s.nq == 2) {
-              if (a == 1 || turns > 0) turn_sync(a);
-              ++turns;
-            }
-            TRACE(2 + a, sp_it, 3);
-            if (lead && ok) {
+          const uint32_t it = kv_base + (j > 0 ? 2 * j - 1 : 0), st = it % kStages;   // K's place in the order
+          const int valid = valid_of(s.t0 + j);
+          const uint32_t idesc = valid == kTileN ? idesc_full : idesc_bf16_f32(kTileM, (valid + 15) & ~15, 0);
+          const uint64_t dk = dk0 + static_cast<uint64_t>((st * kTileBytes) >> 4);
+#pragma unroll 1
+          for (int a = 0; a < s.nq; ++a) {
+            if (ok && j == 0) ok = w.wait_warp(bar_q_full + 8 * a, (a == 0 ? q0 : q1) & 1);
+            if (ok && a == 0) ok = w.wait_warp(bar_kv_full + 8 * st, (it / kStages) & 1);
+            TRACE(2, n0 + n1, 0);
+            if (before >= 0) s_free_sync(before, (before == 0 ? n0 : n1) - 1);
+            TRACE(2, n0 + n1, 1);
+            if (ok) {
               tc_fence_after();
-              issue_pv_half(dv, 0, k_steps, j > 0);
-              issue_pv_half(dv, 1, k_steps, true);
-              TRACE(2 + a, sp_it, 4);
-              if (more) issue_qk(kst, valid);
+              mma_ss_k128(tmem_base + kTmemS, dq + static_cast<uint64_t>((a * kTileBytes) >> 4), dk, idesc, 0u);
             }
-            __syncwarp();
-            // The turn goes on before the commits that release the buffers (90-130 clk each): the other
-            // issuer's first MMA then follows this chain's last without a gap.
-            if (s.nq == 2) turn_pass(a);
-            if (lead && ok) {
-              if (more) tc_commit(bar_kv_empty + 8 * kst);
-              if (j + 2 == n) tc_commit(bar_q_empty + 8 * a);
-              tc_commit(bar_kv_empty + 8 * vst);
+            if (ok) {
+              tc_commit(bar_s_full + 8 * a);
+              if (a == s.nq - 1) tc_commit(bar_kv_empty + 8 * st);
+              if (j == n - 1) tc_commit(bar_q_empty + 8 * a);
             }
-            TRACE(2 + a, sp_it, 5);
-            ++sp_it;
-          } else if (lead && ok) {
-            mbar_arrive(bar_kv_empty + 8 * vst);
-            if (more) mbar_arrive(bar_kv_empty + 8 * kst);
+            TRACE(2, n0 + n1, 2);
+            if (j == 0) ++(a == 0 ? q0 : q1);
+            ++(a == 0 ? n0 : n1);
+            before = a;
           }
         }
-        if (lead && ok && part) tc_commit(bar_o_final + 8 * a);
-        __syncwarp();
+        kv_base += 2 * n;
       }
-      if (a == 0 && turns > 0) turn_sync(0);   // the last turn that the other issuer passed back
+      if (before >= 0) s_free_sync(before, (before == 0 ? n0 : n1) - 1);
+    } else if (warp == 9) {
+      // ------------------------------------------------------------ P V issuer
+      // The commits that free a stage come behind those that a softmax group waits for, but for the segment's last one:
+      // behind that the kernel may end.
+      grid_wait();
+      Sched sched(p, static_cast<int>(blockIdx.x));
+      Seg s;
+      uint32_t kv_base = 0, n0 = 0, n1 = 0;
+      bool ok = true;
+      const uint32_t idesc_pv = idesc_bf16_f32(kTileM, kHeadDim, 1);
+      const uint64_t dv0 = smem_desc_sw128(sKV, kHalfBytes, 1024);          // stage 0 as a V tile (MN-major)
+      while (sched.next(s)) {
+        const int n = s.t1 - s.t0;
+        const ValidKeys valid_of(p, s.b);
+        for (int j = 0; j < n; ++j) {
+          const uint32_t it = kv_base + (j + 1 < n ? 2 * j + 2 : 2 * n - 1), st = it % kStages;
+          const int k_steps = (valid_of(s.t0 + j) + 15) >> 4;
+          const uint64_t dv = dv0 + static_cast<uint64_t>((st * kTileBytes) >> 4);
+          if (ok) ok = w.wait_warp(bar_kv_full + 8 * st, (it / kStages) & 1);
+#pragma unroll 1
+          for (int a = 0; a < s.nq; ++a) {
+            const uint32_t o_tmem = tmem_base + kTmemO + a * 128, p_tmem = tmem_base + kTmemP + a * 64;
+            TRACE(3, n0 + n1, 0);
+            p_ready_sync(a, a == 0 ? n0 : n1);   // P of this tile is in TMEM, O rescaled if need be
+            TRACE(3, n0 + n1, 1);
+            if (ok) {
+              tc_fence_after();
+              if (k_steps == 8) {
+                mma_ts_k64(o_tmem, p_tmem, dv, idesc_pv, j > 0 ? 1u : 0u);
+                mma_ts_k64(o_tmem, p_tmem + 32, dv + 512u, idesc_pv, 1u);
+              } else {
+#pragma unroll 1
+                for (int k = 0; k < k_steps; ++k)
+                  mma_ts(o_tmem, p_tmem + k * 8, dv + static_cast<uint64_t>(k * 128), idesc_pv, (j > 0 || k > 0) ? 1u : 0u);
+              }
+            }
+            if (ok) {
+              const bool last_of_stage = a == s.nq - 1;
+              if (last_of_stage && j == n - 1) tc_commit(bar_kv_empty + 8 * st);
+              tc_commit(bar_pv_done + 8 * a);
+              if (last_of_stage && j < n - 1) tc_commit(bar_kv_empty + 8 * st);
+            }
+            TRACE(3, n0 + n1, 2);
+            ++(a == 0 ? n0 : n1);
+          }
+        }
+        kv_base += 2 * n;
+      }
     }
   } else {
     // ---------------------------------------------------------------- softmax warpgroups
     // Warps 0-3 own query tile 0, warps 4-7 query tile 1; a thread owns a row from the scores
-    // to the output.  The groups never wait for each other.
+    // to the output.
     reg_alloc_softmax();
     grid_wait();
     const int a = warp >> 2;               // query tile of this warpgroup
     const int row = tid & 127;             // row inside the tile = TMEM lane
     const uint32_t t_lane = tmem_base + (static_cast<uint32_t>((warp & 3) * 32) << 16);
-    const uint32_t t_S = t_lane + a * 128, t_O = t_lane + 256 + a * 128;
+    const uint32_t t_S = t_lane + kTmemS, t_P = t_lane + kTmemP + a * 64, t_O = t_lane + kTmemO + a * 128;
     Sched sched(p, static_cast<int>(blockIdx.x));
     Seg s;
-    uint32_t it = 0, seg_it = 0;
+    uint32_t it = 0, s_seen = 0;
     bool ok = true;
     int seg_no = 0;
     CTRACE(1);
@@ -568,23 +539,47 @@ window_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
       if (a >= s.nq) continue;             // a lone last query tile: nothing for group 1
       float m_run = -INFINITY, l_run = 0.f;
       const ValidKeys valid_of(p, s.b);
-      for (int j = s.t0; j < s.t1; ++j, ++it) {
-        const int valid = valid_of(j);
-        TRACE(a, it, 0);
-        if (ok) ok = __all_sync(0xFFFFFFFFu, w.wait(bar_s_full + 8 * a, it & 1));
-        if (!ok) {
-          p_ready_pass(a, it, true);   // the issuer still counts on this warp
-          continue;
+      const uint32_t pv = bar_pv_done + 8 * a, sb = bar_s_full + 8 * a;
+      // scores of tile `it`: true unless the wait gave up, in which case the issuers still count on this warp
+      auto scores = [&](uint32_t tile) {
+        if (ok && __builtin_expect(!__all_sync(0xFFFFFFFFu, s_seen), 0)) ok = w.wait_warp(sb, tile & 1);
+        s_seen = 0;
+        if (__builtin_expect(!ok, 0)) {
+          s_free_pass(a, tile, true);
+          p_ready_pass(a, tile, true);
+          return false;
         }
         tc_fence_after();
-        if (it == 0) CTRACE(2);
-        TRACE(a, it, 1);
-        if (valid <= 64)   // frames of at most half a tile, and the end of a run
-          softmax_row_tile<true, 64>(t_S, t_O, p.scale_log2e, valid, j == s.t0, m_run, l_run, a, it);
-        else if (valid < kTileN)
-          softmax_row_tile<true, kTileN>(t_S, t_O, p.scale_log2e, valid, j == s.t0, m_run, l_run, a, it);
-        else
-          softmax_row_tile<false, kTileN>(t_S, t_O, p.scale_log2e, kTileN, j == s.t0, m_run, l_run, a, it);
+        return true;
+      };
+      int j = s.t0;
+#pragma unroll 1
+      while (j < s.t1) {
+        {   // the segment's first tile, or a ragged one
+          const int valid = valid_of(j);
+          TRACE(a, it, 0);
+          if (scores(it)) {
+            TRACE(a, it, 1);
+            const bool first = j == s.t0;
+            if (valid <= 64)   // frames of at most half a tile, and the end of a run
+              ok = softmax_row_tile<true, 64, false>(t_S, t_P, t_O, p.scale_log2e, valid, first, m_run, l_run, a, it, w, pv, sb, s_seen);
+            else
+              ok = softmax_row_tile<true, kTileN, false>(t_S, t_P, t_O, p.scale_log2e, valid, first, m_run, l_run, a, it, w, pv, sb, s_seen);
+            if (!ok) p_ready_pass(a, it, true);
+          }
+          ++j;
+          ++it;
+        }
+        const int jf = valid_of.full_until(j, s.t1);
+#pragma unroll 1
+        for (; j < jf; ++j, ++it) {
+          TRACE(a, it, 0);
+          if (scores(it)) {
+            TRACE(a, it, 1);
+            ok = softmax_row_tile<false, kTileN, true>(t_S, t_P, t_O, p.scale_log2e, kTileN, false, m_run, l_run, a, it, w, pv, sb, s_seen);
+            if (__builtin_expect(!ok, 0)) p_ready_pass(a, it, true);
+          }
+        }
       }
       CTRACE(8 + seg_no);
       // ---- epilogue of this group's query tile ----
@@ -599,8 +594,7 @@ window_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
         asm volatile("ld.acquire.gpu.global.s32 %0, [%1];" : "=r"(seen) : "l"(counter()) : "memory");
       }
       if (ok) {
-        ok = __all_sync(0xFFFFFFFFu, w.wait(bar_o_final + 8 * a, seg_it & 1));
-        ++seg_it;
+        ok = w.wait_warp(bar_pv_done + 8 * a, (it - 1) & 1);
         tc_fence_after();
       }
       const int n = (2 * s.qp + a) * kTileM + row;

@@ -40,6 +40,19 @@ __device__ __forceinline__ uint32_t mbar_try_wait(uint32_t bar, uint32_t parity)
   return ok;
 }
 
+// one look, without waiting
+__device__ __forceinline__ uint32_t mbar_test(uint32_t bar, uint32_t parity) {
+  uint32_t ok;
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t"
+      "mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+      "selp.u32 %0, 1, 0, p;\n\t}"
+      : "=r"(ok)
+      : "r"(bar), "r"(parity)
+      : "memory");
+  return ok;
+}
+
 // try_wait that lets the hardware park the thread for up to `ns` nanoseconds
 __device__ __forceinline__ uint32_t mbar_try_wait_hint(uint32_t bar, uint32_t parity, uint32_t ns) {
   uint32_t ok;
@@ -97,19 +110,25 @@ __device__ __forceinline__ void tc_fence_after() {
 __device__ __forceinline__ void tc_wait_st() {
   asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
 }
-// All tcgen05.mma issued so far by this thread arrive on `bar` when they complete.
+// tcgen05.mma and tcgen05.commit are executed by a whole, converged warp, and each names one elected lane
+// (always the same one) by a predicate on the instruction itself: the operands of an MMA come from uniform
+// registers, and only code that the whole warp runs keeps them there.  Eight MMAs take 150-180 clk to
+// issue this way and run back to back (64 clk each); issued by one lane inside a branch they take 390 clk, and
+// chains of eight with their commits 690 instead of 513.
+// All tcgen05.mma issued so far by that lane arrive on `bar` when they complete.
 __device__ __forceinline__ void tc_commit(uint32_t bar) {
-  asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
-                   bar)
-               : "memory");
+  asm volatile(
+      "{\n\t.reg .pred pe;\n\telect.sync _|pe, 0xffffffff;\n\t"
+      "@pe tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n\t}" ::"r"(bar)
+      : "memory");
 }
 // D[tmem] (+)= A[tmem] * B[smem desc]
 __device__ __forceinline__ void mma_ts(uint32_t d_tmem, uint32_t a_tmem, uint64_t b_desc,
                                        uint32_t idesc, uint32_t accumulate) {
   asm volatile(
-      "{\n\t.reg .pred p;\n\t"
-      "setp.ne.b32 p, %4, 0;\n\t"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n\t}"
+      "{\n\t.reg .pred p, pe;\n\t"
+      "setp.ne.b32 p, %4, 0;\n\telect.sync _|pe, 0xffffffff;\n\t"
+      "@pe tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n\t}"
       ::"r"(d_tmem), "r"(a_tmem), "l"(b_desc), "r"(idesc), "r"(accumulate)
       : "memory");
 }
@@ -123,24 +142,24 @@ __device__ __forceinline__ void mma_ss_k128(uint32_t d_tmem, uint64_t a_desc, ui
   const uint32_t a_lo = static_cast<uint32_t>(a_desc), a_hi = static_cast<uint32_t>(a_desc >> 32);
   const uint32_t b_lo = static_cast<uint32_t>(b_desc), b_hi = static_cast<uint32_t>(b_desc >> 32);
   asm volatile(
-      "{\n\t.reg .pred p, pt;\n\t.reg .b32 al, bl;\n\t.reg .b64 ad, bd;\n\t"
-      "setp.ne.b32 p, %6, 0;\n\tsetp.eq.b32 pt, 0, 0;\n\t"
+      "{\n\t.reg .pred p, pt, pe;\n\t.reg .b32 al, bl;\n\t.reg .b64 ad, bd;\n\t"
+      "setp.ne.b32 p, %6, 0;\n\tsetp.eq.b32 pt, 0, 0;\n\telect.sync _|pe, 0xffffffff;\n\t"
       "add.u32 al, %1, 0;\n\tadd.u32 bl, %3, 0;\n\tmov.b64 ad, {al, %2};\n\tmov.b64 bd, {bl, %4};\n\t"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], ad, bd, %5, p;\n\t"
+      "@pe tcgen05.mma.cta_group::1.kind::f16 [%0], ad, bd, %5, p;\n\t"
       "add.u32 al, %1, 2;\n\tadd.u32 bl, %3, 2;\n\tmov.b64 ad, {al, %2};\n\tmov.b64 bd, {bl, %4};\n\t"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], ad, bd, %5, pt;\n\t"
+      "@pe tcgen05.mma.cta_group::1.kind::f16 [%0], ad, bd, %5, pt;\n\t"
       "add.u32 al, %1, 4;\n\tadd.u32 bl, %3, 4;\n\tmov.b64 ad, {al, %2};\n\tmov.b64 bd, {bl, %4};\n\t"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], ad, bd, %5, pt;\n\t"
+      "@pe tcgen05.mma.cta_group::1.kind::f16 [%0], ad, bd, %5, pt;\n\t"
       "add.u32 al, %1, 6;\n\tadd.u32 bl, %3, 6;\n\tmov.b64 ad, {al, %2};\n\tmov.b64 bd, {bl, %4};\n\t"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], ad, bd, %5, pt;\n\t"
+      "@pe tcgen05.mma.cta_group::1.kind::f16 [%0], ad, bd, %5, pt;\n\t"
       "add.u32 al, %1, 1024;\n\tadd.u32 bl, %3, 1024;\n\tmov.b64 ad, {al, %2};\n\tmov.b64 bd, {bl, %4};\n\t"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], ad, bd, %5, pt;\n\t"
+      "@pe tcgen05.mma.cta_group::1.kind::f16 [%0], ad, bd, %5, pt;\n\t"
       "add.u32 al, %1, 1026;\n\tadd.u32 bl, %3, 1026;\n\tmov.b64 ad, {al, %2};\n\tmov.b64 bd, {bl, %4};\n\t"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], ad, bd, %5, pt;\n\t"
+      "@pe tcgen05.mma.cta_group::1.kind::f16 [%0], ad, bd, %5, pt;\n\t"
       "add.u32 al, %1, 1028;\n\tadd.u32 bl, %3, 1028;\n\tmov.b64 ad, {al, %2};\n\tmov.b64 bd, {bl, %4};\n\t"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], ad, bd, %5, pt;\n\t"
+      "@pe tcgen05.mma.cta_group::1.kind::f16 [%0], ad, bd, %5, pt;\n\t"
       "add.u32 al, %1, 1030;\n\tadd.u32 bl, %3, 1030;\n\tmov.b64 ad, {al, %2};\n\tmov.b64 bd, {bl, %4};\n\t"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], ad, bd, %5, pt;\n\t"
+      "@pe tcgen05.mma.cta_group::1.kind::f16 [%0], ad, bd, %5, pt;\n\t"
       "}"
       ::"r"(d_tmem), "r"(a_lo), "r"(a_hi), "r"(b_lo), "r"(b_hi), "r"(idesc), "r"(accumulate)
       : "memory");
@@ -151,16 +170,16 @@ __device__ __forceinline__ void mma_ts_k64(uint32_t d_tmem, uint32_t a_tmem, uin
                                            uint32_t idesc, uint32_t accumulate) {
   const uint32_t b_lo = static_cast<uint32_t>(b_desc), b_hi = static_cast<uint32_t>(b_desc >> 32);
   asm volatile(
-      "{\n\t.reg .pred p, pt;\n\t.reg .b32 at, bl;\n\t.reg .b64 bd;\n\t"
-      "setp.ne.b32 p, %5, 0;\n\tsetp.eq.b32 pt, 0, 0;\n\t"
+      "{\n\t.reg .pred p, pt, pe;\n\t.reg .b32 at, bl;\n\t.reg .b64 bd;\n\t"
+      "setp.ne.b32 p, %5, 0;\n\tsetp.eq.b32 pt, 0, 0;\n\telect.sync _|pe, 0xffffffff;\n\t"
       "add.u32 at, %1, 0;\n\tadd.u32 bl, %2, 0;\n\tmov.b64 bd, {bl, %3};\n\t"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], [at], bd, %4, p;\n\t"
+      "@pe tcgen05.mma.cta_group::1.kind::f16 [%0], [at], bd, %4, p;\n\t"
       "add.u32 at, %1, 8;\n\tadd.u32 bl, %2, 128;\n\tmov.b64 bd, {bl, %3};\n\t"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], [at], bd, %4, pt;\n\t"
+      "@pe tcgen05.mma.cta_group::1.kind::f16 [%0], [at], bd, %4, pt;\n\t"
       "add.u32 at, %1, 16;\n\tadd.u32 bl, %2, 256;\n\tmov.b64 bd, {bl, %3};\n\t"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], [at], bd, %4, pt;\n\t"
+      "@pe tcgen05.mma.cta_group::1.kind::f16 [%0], [at], bd, %4, pt;\n\t"
       "add.u32 at, %1, 24;\n\tadd.u32 bl, %2, 384;\n\tmov.b64 bd, {bl, %3};\n\t"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], [at], bd, %4, pt;\n\t"
+      "@pe tcgen05.mma.cta_group::1.kind::f16 [%0], [at], bd, %4, pt;\n\t"
       "}"
       ::"r"(d_tmem), "r"(a_tmem), "r"(b_lo), "r"(b_hi), "r"(idesc), "r"(accumulate)
       : "memory");
@@ -211,6 +230,24 @@ __device__ __forceinline__ void tmem_st32(uint32_t taddr, const uint32_t* r) {
       "r"(r[22]), "r"(r[23]), "r"(r[24]), "r"(r[25]), "r"(r[26]), "r"(r[27]), "r"(r[28]),
       "r"(r[29]), "r"(r[30]), "r"(r[31])
       : "memory");
+}
+// The same for 8 columns.
+__device__ __forceinline__ void tmem_ld8(uint32_t taddr, uint32_t* r) {
+  asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
+               : "r"(taddr)
+               : "memory");
+}
+__device__ __forceinline__ void tc_wait_ld8(uint32_t* r) {
+  asm volatile("tcgen05.wait::ld.sync.aligned;"
+               : "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3]), "+r"(r[4]), "+r"(r[5]), "+r"(r[6]), "+r"(r[7])
+               :
+               : "memory");
+}
+__device__ __forceinline__ void tmem_st8(uint32_t taddr, const uint32_t* r) {
+  asm volatile("tcgen05.st.sync.aligned.32x32b.x8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"r"(taddr), "r"(r[0]),
+               "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7])
+               : "memory");
 }
 // One 32-byte store (the address must be 32-byte aligned).
 __device__ __forceinline__ void st_global_32(void* p, const uint32_t* r) {
