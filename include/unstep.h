@@ -223,7 +223,9 @@ int unstep_window_attn_noalloc(const unstep_shape_t* shape, const int32_t* start
  * over is split along the keys in one of two ways, whichever is estimated to be shorter: every item
  * into the same number of parts (one or more), one part per worker; or all its steps as one sequence
  * cut into equal contiguous shares, one per worker, so that an item falls into as many parts as shares
- * touch it.  The parts of an item are merged by the worker that finishes last.
+ * touch it.  The parts of an item are merged by the worker that finishes last.  (A launch of no more
+ * items than workers may instead cut every item into 2 to 8 parts that are one thread-block cluster, if the
+ * device runs that many clusters at once; this list, which asks no device, has the split without clusters.)
  *
  *   segs     : HOST int32 [max_segs][10], written (may be NULL when max_segs is 0).  One row per
  *              segment in the order the worker walks them: worker, stream, head, query pair,

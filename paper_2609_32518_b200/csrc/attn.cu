@@ -308,6 +308,16 @@ struct ValidKeys {
   }
 };
 
+// Partial results exchanged inside a cluster: where the K and V tiles were, O of both query tiles as
+// [tile][col / 4][row][col % 4], then (m, l) as [tile][row].
+constexpr int kSwapTileBytes = 128 * 128 * 4;
+constexpr int kSwapMl = 2 * kSwapTileBytes;
+static_assert(kSwapMl + 2 * 128 * 8 <= kStages * kTileBytes, "the exchange does not fit the K and V stages");
+
+// kCluster: a launch of one part per block, in which the parts of an item are a cluster and merge through each
+// other's shared memory.  The other form merges through global memory, where a part's stores, the fence
+// with its count and the last part's loads took 5-10 us one after the other.
+template <bool kCluster>
 __global__ void __launch_bounds__(kThreads, 1)
 window_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_k,
                    const __grid_constant__ CUtensorMap tm_v, const __grid_constant__ CUtensorMap tm_kf,
@@ -528,6 +538,7 @@ window_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
     const uint32_t t_S = t_lane + kTmemS, t_P = t_lane + kTmemP + a * 64, t_O = t_lane + kTmemO + a * 128;
     Sched sched(p, static_cast<int>(blockIdx.x));
     Seg s;
+    Seg seg = {};        // of a cluster's block: its only one
     uint32_t it = 0, s_seen = 0;
     bool ok = true;
     int seg_no = 0;
@@ -536,6 +547,7 @@ window_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
     // it still meets its group and its issuer at every named barrier.  ok is the same in all threads
     // of a warp: barriers and TMEM accesses are instructions of the whole warp.
     while (sched.next(s)) {
+      if (kCluster) seg = s;
       if (a >= s.nq) continue;             // a lone last query tile: nothing for group 1
       float m_run = -INFINITY, l_run = 0.f;
       const ValidKeys valid_of(p, s.b);
@@ -587,7 +599,7 @@ window_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
       // Part of a split item: the arrival counter, looked at under the wait for the last P V
       auto counter = [&] { return p.counters + 2 * s.item + a; };
       int seen = 0;
-      if (!whole && row == 0) {
+      if (!kCluster && !whole && row == 0) {
 #ifdef UNSTEP_CHECK
         if (2 * s.item + a >= p.extent_counters) atomicExch(p.status, static_cast<int>(UNSTEP_ERR_BOUNDS));
 #endif
@@ -614,7 +626,23 @@ window_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
           UNSTEP_STORE(out_v, d + i, p.extent_out, make_uint4(w[4 * i], w[4 * i + 1], w[4 * i + 2], w[4 * i + 3]),
                        p.status);
       };
-      if (whole) {
+      if (kCluster) {
+        // Every block of a cluster holds one part of the same item.  Each puts its part into its own shared memory and
+        // then merges a share of the columns of all rows, in part order, reading the others' parts there.
+        if (s.nq == 2) asm volatile("bar.sync %0, 256;" ::"r"(kSwapBarrier) : "memory");   // the stages are free behind both P V
+        const uint32_t mine = sKV + a * kSwapTileBytes + row * 16;
+        if (ok) {
+#pragma unroll
+          for (int q = 0; q < 4; ++q) {
+            uint32_t o[32];
+            tmem_ld32(t_O + q * 32, o);
+            tc_wait_ld32(o);
+#pragma unroll
+            for (int i = 0; i < 8; ++i) st_shared_16(mine + (q * 8 + i) * 2048, o + 4 * i);
+          }
+          st_shared_8(sKV + kSwapMl + a * 1024 + row * 8, __float_as_uint(m_run), __float_as_uint(l_run));
+        }
+      } else if (whole) {
         // O / l -> bf16 -> out[b][n][h][:]: a thread writes its whole 256-byte row
         if (ok) {
           const float inv_l = 1.f / l_run;
@@ -743,6 +771,69 @@ window_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
       CTRACE(3 + seg_no);
       ++seg_no;
     }
+    if (kCluster) {
+      __syncwarp();
+      cluster_sync();   // all parts are in place
+      const int parts = p.parts, part = static_cast<int>(cluster_rank());
+      // a lone query tile is shared out to both groups
+      const int tile = seg.nq == 2 ? a : 0, share = seg.nq == 2 ? part : 2 * part + a, shares = seg.nq == 2 ? parts : 2 * parts;
+      const int n = (2 * seg.qp + tile) * kTileM + row;
+      bool good = seg.nq > 0;
+      for (int c = 0; c < parts; ++c)   // a block that gave up has left no part
+        good = good && ld_cluster_4(cluster_addr(smem_u32(const_cast<int*>(abort_flag)), c)) == 0;
+      if (good && n < p.L) {
+        float2 x[kMaxClusterParts];
+        float m_all = -INFINITY, l_sum = 0.f;
+#pragma unroll
+        for (int c = 0; c < kMaxClusterParts; ++c)
+          x[c] = c < parts ? ld_cluster_8(cluster_addr(sKV + kSwapMl + tile * 1024 + row * 8, c)) : make_float2(-INFINITY, 0.f);
+#pragma unroll
+        for (int c = 0; c < kMaxClusterParts; ++c) m_all = fmaxf(m_all, x[c].x);
+#pragma unroll
+        for (int c = 0; c < kMaxClusterParts; ++c)
+          if (c < parts) {
+            x[c].x = ex2((x[c].x - m_all) * p.scale_log2e);
+            l_sum += x[c].y * x[c].x;
+          }
+        const float inv_l = 1.f / l_sum;
+        uint4* const out_v = reinterpret_cast<uint4*>(out);
+        const int64_t dst = ((static_cast<int64_t>(seg.b) * p.L + n) * p.Hn + seg.h) * (kHeadDim / 8);   // 16-byte vectors
+        const uint32_t from = sKV + tile * kSwapTileBytes + row * 16;
+#pragma unroll 2
+        for (int v = 16 * share / shares; v < 16 * (share + 1) / shares; ++v) {
+          float acc[8];
+#pragma unroll
+          for (int i = 0; i < 8; ++i) acc[i] = 0.f;
+#pragma unroll
+          for (int c = 0; c < kMaxClusterParts; ++c)
+            if (c < parts) {
+              const uint32_t at = cluster_addr(from + v * 4096, c);
+              const float4 u0 = ld_cluster_16(at), u1 = ld_cluster_16(at + 2048);
+              acc[0] = fmaf(u0.x, x[c].x, acc[0]);
+              acc[1] = fmaf(u0.y, x[c].x, acc[1]);
+              acc[2] = fmaf(u0.z, x[c].x, acc[2]);
+              acc[3] = fmaf(u0.w, x[c].x, acc[3]);
+              acc[4] = fmaf(u1.x, x[c].x, acc[4]);
+              acc[5] = fmaf(u1.y, x[c].x, acc[5]);
+              acc[6] = fmaf(u1.z, x[c].x, acc[6]);
+              acc[7] = fmaf(u1.w, x[c].x, acc[7]);
+            }
+          UNSTEP_STORE(out_v, dst + v, p.extent_out,
+                       make_uint4(pack_bf16x2(acc[0] * inv_l, acc[1] * inv_l), pack_bf16x2(acc[2] * inv_l, acc[3] * inv_l),
+                                  pack_bf16x2(acc[4] * inv_l, acc[5] * inv_l), pack_bf16x2(acc[6] * inv_l, acc[7] * inv_l)),
+                       p.status);
+        }
+      }
+    }
+  }
+  // The other roles meet the softmax groups at the cluster's barrier, and no block leaves while another reads its part.
+  if (kCluster) {
+    if (warp >= 8) {
+      __syncwarp();
+      cluster_sync();
+    }
+    __syncwarp();
+    cluster_sync();
   }
 
   // ---- teardown: every role ends here, also after a timed-out wait --------------------
@@ -819,6 +910,7 @@ static bool make_map(CUtensorMap* m, const void* base, int rank, const uint64_t*
 struct DeviceInfo {
   bool ok = false;
   int sm_count = 0;
+  int32_t clusters[kMaxClusterParts + 1] = {};   // clusters of that many blocks which the device runs at the same time
 };
 
 static const DeviceInfo& device_info() {
@@ -831,8 +923,28 @@ static const DeviceInfo& device_info() {
   }
   if (dev != cached_dev) {
     info.ok = cudaDeviceGetAttribute(&info.sm_count, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess &&
-              cudaFuncSetAttribute(window_attn_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+              cudaFuncSetAttribute(window_attn_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                   kAttnSmemBytes) == cudaSuccess &&
+              cudaFuncSetAttribute(window_attn_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                    kAttnSmemBytes) == cudaSuccess;
+    for (int parts = 2; parts <= kMaxClusterParts; ++parts) {
+      cudaLaunchAttribute attr;
+      attr.id = cudaLaunchAttributeClusterDimension;
+      attr.val.clusterDim.x = parts;
+      attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
+      cudaLaunchConfig_t cfg = {};
+      cfg.gridDim = dim3(parts);
+      cfg.blockDim = dim3(kThreads);
+      cfg.dynamicSmemBytes = kAttnSmemBytes;
+      cfg.attrs = &attr;
+      cfg.numAttrs = 1;
+      int n = 0;
+      if (!info.ok || cudaOccupancyMaxActiveClusters(&n, window_attn_kernel<true>, &cfg) != cudaSuccess) {
+        cudaGetLastError();
+        n = 0;
+      }
+      info.clusters[parts] = n;
+    }
     cached_dev = dev;
   }
   return info;
@@ -958,7 +1070,8 @@ static int window_attn_run(const unstep_shape_t* shape, const int32_t* start_fra
   plan_shape(p, shape, sink_frames);
   for (int b0 = 0; b0 < shape->batch; b0 += kMaxStreamsPerLaunch) {
     const int nb = shape->batch - b0 < kMaxStreamsPerLaunch ? shape->batch - b0 : kMaxStreamsPerLaunch;
-    rc = plan_launch(p, shape, start_frame + b0, nb, window_frames, sink_frames, sink_attend, info.sm_count);
+    rc = plan_launch(p, shape, start_frame + b0, nb, window_frames, sink_frames, sink_attend, info.sm_count,
+                     info.clusters);
     if (rc != UNSTEP_OK) return rc;
     Workspace ws;
     rc = scratch(st, 2 * static_cast<size_t>(info.sm_count), 2 * static_cast<size_t>(nb) * p.items_per_stream, &ws);
@@ -995,8 +1108,9 @@ static int window_attn_run(const unstep_shape_t* shape, const int32_t* start_fra
     // the idling it takes away.  The line lies about where the gain of short runs (0.6 % at 57 steps) has
     // come down to the loss of runs at the cap (0.4 %).
     const bool brief = p.all_steps < static_cast<int64_t>(kOverlapSteps) * p.n_workers;
-    const cudaError_t err = launch_overlapped(brief, window_attn_kernel, p.n_workers, kThreads, kAttnSmemBytes, st, tm_q,
-                                              tm_k, tm_v, tm_kf, tm_vf, p, ob);
+    const cudaError_t err =
+        launch_clusters(brief, p.cluster ? p.parts : 1, p.cluster ? window_attn_kernel<true> : window_attn_kernel<false>,
+                        p.n_workers, kThreads, kAttnSmemBytes, st, tm_q, tm_k, tm_v, tm_kf, tm_vf, p, ob);
     g_launches.fetch_add(1);
     if (err != cudaSuccess) return UNSTEP_ERR_CUDA;
   }

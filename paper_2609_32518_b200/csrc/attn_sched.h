@@ -20,6 +20,7 @@ namespace unstep {
 constexpr int kTileM = 128;                 // queries per tile (two tiles per work item)
 constexpr int kTileN = 128;                 // keys per tile
 constexpr int kMinStepsPerWorker = 4;       // shortest share of the remainder that may cross items
+constexpr int kMaxClusterParts = 8;         // largest portable cluster
 
 struct AttnParams {
   int32_t Hn, L, T, C;
@@ -34,6 +35,7 @@ struct AttnParams {
   int32_t full_rounds;      // whole rounds per stream, n_workers items each
   int32_t leftover;         // items per stream behind the whole rounds: the remainder
   int32_t parts;            // > 0: every item of the remainder is cut into this many parts, one per worker
+  int32_t cluster;          // 1: the parts of an item are a cluster (no whole rounds, 2 <= parts <= kMaxClusterParts)
   int32_t n_active;         // parts == 0: workers that take a share of the remainder, >= 1
   int64_t all_steps;        // key tiles of all items of the launch
   int32_t narrow;           // 1: total_steps * n_active fits 32 bits, and so does every index of the shares
@@ -114,12 +116,13 @@ UNSTEP_HD TileInfo tile_info(const AttnParams& p, int b, int j) {
 //      fetched from HBM once and then hit in L2 by the other workers of the head.
 //   2. Remainder: the leftover items of all streams (fewer than n_workers per stream), split along
 //      their keys in one of two ways (plan_launch chooses):
-//      - p.parts > 0: every item is cut into p.parts parts and each worker takes one of them;
+//      - p.parts > 0: every item is cut into p.parts parts and each worker takes one of them (in a
+//        launch without whole rounds the parts of an item may be a cluster of blocks: p.cluster);
 //      - p.parts == 0: the items form one sequence of (item, key tile) steps, and each of the first
 //        n_active workers takes an equal contiguous share of it (n_active <= total_steps, so no
 //        share is empty and the workers that hold parts of an item are exactly those between the
 //        owners of its first and last step).
-//      The parts of an item are merged by whichever worker finishes last.
+//      The parts of an item are merged by whichever worker finishes last, or by its cluster.
 struct Sched {
   int64_t lo, hi, cur;
   int b_round, round;   // position in the whole rounds
@@ -224,7 +227,7 @@ UNSTEP_HD int part_slot(const AttnParams& p, int c, int64_t item_step0) {
 // steps 82 whole, 5 parts 33, 6 parts 31, 8 parts 33, 86 shares of 4 steps 35; 40 items x 16 steps 35
 // whole, 3 parts 25, 148 shares 36; 80 items x 37 steps behind a whole round: shares.
 inline int32_t remainder_parts(int64_t items, int64_t steps, int32_t least, int32_t most, int max_workers,
-                               int32_t* shares) {
+                               int32_t* shares, double* us) {
   int64_t n = steps / kMinStepsPerWorker;
   n = n < 1 ? 1 : (n > max_workers ? max_workers : n);
   *shares = static_cast<int32_t>(n);
@@ -239,15 +242,37 @@ inline int32_t remainder_parts(int64_t items, int64_t steps, int32_t least, int3
       best = parts;
     }
   }
+  *us = lowest;
+  return best;
+}
+
+// The same for parts that form a cluster, which merges them through shared memory: 0 where that is not
+// shorter than `us`.  clusters[n]: clusters of n blocks that the device runs at the same time (148 SMs: 74, 45,
+// 33, 26, 22, 15, 15 of 2 to 8 blocks).  The merge costs about 2.5 us however many the parts, as each merges a share
+// of the columns.  Attention alone, us, parts merged through global memory or shares -> clusters: 8 items x 40 steps
+// 28.2 -> 20.0, 8 x 28 25.2 -> 18.6, 15 x 113 46.3 -> 37.1, 20 x 16 21.0 -> 17.8, 36 x 18 24.7 -> 22.1, 40 x 43 38.3
+// -> 35.5, 57 x 37 42.7 -> 41.7, 2 x 6 11.6 -> 10.0; 38 items x 256 steps: shares 138, 3 parts 153.
+inline int32_t cluster_parts(int64_t items, int32_t least, int32_t most, const int32_t* clusters, double us) {
+  int32_t best = 0;
+  for (int32_t parts = 2; parts <= kMaxClusterParts && parts <= least; ++parts) {
+    if (items > clusters[parts] || static_cast<int64_t>(most) * parts > INT32_MAX) continue;
+    const double cost = 1.6 * ((most + parts - 1) / parts) + 2.5;
+    if (cost < us) {
+      us = cost;
+      best = parts;
+    }
+  }
   return best;
 }
 
 // Fills the per-launch part of `p` for streams [b0, b0 + nb): the attended frames of each stream
 // cut into runs of consecutive cache slots, the key tiles, and the split of the work over at
 // most `max_workers` workers.  The shape-wide fields (Hn, L, T, C, q_tiles, q_pairs,
-// tiles_per_frame, flat, items_per_stream, sink) must already be set.  Host only.
+// tiles_per_frame, flat, items_per_stream, sink) must already be set.  `clusters` as in cluster_parts;
+// without it no part is in a cluster.  Host only.
 inline int plan_launch(AttnParams& p, const unstep_shape_t* shape, const int32_t* start_frame, int nb,
-                       int32_t window_frames, int32_t sink_frames, int32_t sink_attend, int max_workers) {
+                       int32_t window_frames, int32_t sink_frames, int32_t sink_attend, int max_workers,
+                       const int32_t* clusters = nullptr) {
   p.n_streams = nb;
   for (int i = 0; i < nb; ++i) {
     const int hi = start_frame[i] + shape->chunk_frames;
@@ -297,11 +322,18 @@ inline int plan_launch(AttnParams& p, const unstep_shape_t* shape, const int32_t
   }
   p.total_steps = steps;
   p.parts = 0;
+  p.cluster = 0;
   p.n_active = 1;
   p.narrow = 1;
   if (steps > 0) {
     const int64_t items = static_cast<int64_t>(nb) * p.leftover;
-    p.parts = remainder_parts(items, steps, least, most, max_workers, &p.n_active);
+    double us = 0.0;
+    p.parts = remainder_parts(items, steps, least, most, max_workers, &p.n_active, &us);
+    if (clusters != nullptr && p.full_rounds == 0) {
+      const int32_t parts = cluster_parts(items, least, most, clusters, us);
+      p.cluster = parts > 0;
+      if (p.cluster) p.parts = parts;
+    }
     p.narrow = steps * p.n_active <= INT32_MAX;
     if (p.full_rounds == 0) p.n_workers = p.parts > 0 ? static_cast<int32_t>(items) * p.parts : p.n_active;
   }

@@ -14,8 +14,9 @@
 
 namespace unstep {
 
-// Barrier 0 is __syncthreads.  Group barriers: the 4 warps of softmax group a.
-constexpr int kGroupBarrier = 1, kPReadyBarrier = 3, kSFreeBarrier = 7;
+// Barrier 0 is __syncthreads.  Group barriers: the 4 warps of softmax group a.  Swap barrier: all 8, in front of
+// the exchange of partial results in a cluster.
+constexpr int kGroupBarrier = 1, kPReadyBarrier = 3, kSFreeBarrier = 7, kSwapBarrier = 11;
 
 // Per key tile of group a: S read (its 4 warps and the Q K^T issuer) and then P of the tile ready (its 4 warps
 // and the P V issuer), two barriers of each kind per group used in turn.  The issuers always wait at the

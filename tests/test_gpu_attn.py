@@ -284,6 +284,17 @@ def test_items_cut_into_equal_parts(batch, heads, grid, fc, ring, win, history, 
     run(wl)
 
 
+# Items of 135-token frames, two query tiles and a lone one of 14 rows per head, cut into 2 to 8 parts that are a
+# cluster (on 148 SMs, which hold 74, 45, 33, 26, 22, 15, 15 clusters of 2 to 8 blocks).
+@pytest.mark.parametrize("heads,frames,parts", [(25, 3, 2), (20, 8, 3), (15, 7, 4), (12, 9, 5), (10, 11, 6), (7, 6, 7),
+                                                (7, 7, 8)])
+def test_items_whose_parts_are_a_cluster(heads, frames, parts):
+    sh = W.Shape(batch=1, heads=heads, chunk_frames=2, grid_h=9, grid_w=15, ring_frames=frames)
+    wl = W.Workload(f"cluster{parts}", sh, seed=33, history_starts=(tuple(range(0, frames - 2, 2)),),
+                    measured_starts=(frames - 2,), window_frames=(frames,), k_scale=4.0)
+    run(wl)
+
+
 @pytest.mark.parametrize("grid,fc,ring,history,start,keys", [
     ((8, 8), 2, 6, (0, 2), 4, (33, 63)),               # tiles of 64 keys: past the first 32 of a tile
     ((8, 8), 2, 6, (0, 2), 4, (31, 64 + 40)),          # and in the tile behind it
