@@ -913,6 +913,38 @@ struct DeviceInfo {
   int32_t clusters[kMaxClusterParts + 1] = {};   // clusters of that many blocks which the device runs at the same time
 };
 
+// Set up and queried once per device and process; each thread keeps a copy for the device it uses.
+static DeviceInfo query_device(int dev) {
+  static std::mutex mutex;
+  static std::map<int, DeviceInfo> known;
+  std::lock_guard<std::mutex> lock(mutex);
+  auto it = known.find(dev);
+  if (it != known.end()) return it->second;
+  DeviceInfo info;
+  info.ok = cudaDeviceGetAttribute(&info.sm_count, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess &&
+            cudaFuncSetAttribute(window_attn_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 kAttnSmemBytes) == cudaSuccess &&
+            cudaFuncSetAttribute(window_attn_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 kAttnSmemBytes) == cudaSuccess;
+  if (!info.ok) return info;
+  for (int parts = 2; parts <= kMaxClusterParts; ++parts) {
+    cudaLaunchAttribute attr;
+    attr.id = cudaLaunchAttributeClusterDimension;
+    attr.val.clusterDim.x = parts;
+    attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(parts);
+    cfg.blockDim = dim3(kThreads);
+    cfg.dynamicSmemBytes = kAttnSmemBytes;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    int n = 0;
+    if (cudaOccupancyMaxActiveClusters(&n, window_attn_kernel<true>, &cfg) == cudaSuccess) info.clusters[parts] = n;
+    else cudaGetLastError();   // no clusters of that size, then
+  }
+  return known[dev] = info;
+}
+
 static const DeviceInfo& device_info() {
   static thread_local int cached_dev = -1;
   static thread_local DeviceInfo info;
@@ -921,30 +953,8 @@ static const DeviceInfo& device_info() {
     info.ok = false;
     return info;
   }
-  if (dev != cached_dev) {
-    info.ok = cudaDeviceGetAttribute(&info.sm_count, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess &&
-              cudaFuncSetAttribute(window_attn_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                   kAttnSmemBytes) == cudaSuccess &&
-              cudaFuncSetAttribute(window_attn_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                   kAttnSmemBytes) == cudaSuccess;
-    for (int parts = 2; parts <= kMaxClusterParts; ++parts) {
-      cudaLaunchAttribute attr;
-      attr.id = cudaLaunchAttributeClusterDimension;
-      attr.val.clusterDim.x = parts;
-      attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
-      cudaLaunchConfig_t cfg = {};
-      cfg.gridDim = dim3(parts);
-      cfg.blockDim = dim3(kThreads);
-      cfg.dynamicSmemBytes = kAttnSmemBytes;
-      cfg.attrs = &attr;
-      cfg.numAttrs = 1;
-      int n = 0;
-      if (!info.ok || cudaOccupancyMaxActiveClusters(&n, window_attn_kernel<true>, &cfg) != cudaSuccess) {
-        cudaGetLastError();
-        n = 0;
-      }
-      info.clusters[parts] = n;
-    }
+  if (dev != cached_dev || !info.ok) {
+    info = query_device(dev);
     cached_dev = dev;
   }
   return info;
