@@ -1109,7 +1109,8 @@ static int window_attn_run(const unstep_shape_t* shape, const int32_t* start_fra
         !make_map(&tm_v, vb, 5, rdims, rstr, 2) || !make_map(&tm_kf, kb, 4, fdims, fstr, 2) ||
         !make_map(&tm_vf, vb, 4, fdims, fstr, 2))
       return UNSTEP_ERR_CUDA;
-    // Set up under the append before it where the launch is short.  Append and attention, us not
+    // Set up under the append before it where the launch is short.  Append and attention (with the pipeline of one
+    // S per query tile, 10 % slower per step), us not
     // overlapped -> overlapped, by steps per worker: in runs of 20 (full clock) 24: 78.9 -> 76.5, 35:
     // 94.6 -> 92.6, 57: 143.1 -> 142.3, 114: 242.0 -> 240.6, 226: 446.1 -> 445.5, 394: 754.9 -> 763.7; run
     // on end at the power cap 24: 80.2 -> 79.8 (1912 -> 1867 MHz), 57: 155.2 -> 155.8 (1792 -> 1776), 114:
