@@ -201,10 +201,12 @@ __device__ __forceinline__ void mask_block32(uint32_t* s, int col0, int nvalid) 
 //
 // The reference is the maximum of the segment's first key tile, so that the largest weight there is exactly 1 (with
 // the maximum of 32 scores the error of peaked rows against float64 grew from 2.17e-3 to 2.32e-3).  It moves
-// only where a later tile has a score more than kJump = 64 (log2 units) above it: up to there P (bf16)
-// and the float32 sums are as accurate as near 1 (same relative precision, no overflow: 32760 keys of 2^64
-// times |v| stay far below 2^127), and what was accumulated before such a jump is negligible exactly as in
-// the true softmax.  The scores have left TMEM by the time a sum of P could tell, so the maximum is looked
+// only where a later tile has a score more than kJump = 57 (log2 units) above it: up to there P (bf16) and the
+// float32 sums are as accurate as near 1 (same relative precision), and what was accumulated before such a jump
+// is negligible exactly as in the true softmax.  A tile's sum of P is at most 128 * 2^57 = 2^64, the sum of n keys
+// at most n * 2^57, and O that times |v|: finite for any window that the entry points take (2^30 keys) up to
+// |v| = 2^40, for 32760 keys up to 2^55.  (A score may be 64 above the reference with |v| 2^7 smaller; the results of
+// ordinary keys are the same.)  The scores have left TMEM by the time a sum of P could tell, so the maximum is looked
 // for in front: 64 three-input maxima in the shadow of the other group's exponentials.
 //
 // P may be stored, and O rescaled, once the P V of the tile before has run.  That barrier, and the one of the next
@@ -212,7 +214,7 @@ __device__ __forceinline__ void mask_block32(uint32_t* s, int col0, int nvalid) 
 // almost always finds what it looks for.
 // Tiles of at most 64 keys (frames of up to 64 tokens, the end of a run) leave the other half of the columns
 // alone.
-constexpr float kJump = 64.f;
+constexpr float kJump = 57.f;
 
 template <bool kMasked, int kCols, bool kTight>   // kCols: score columns that hold keys, 64 or 128; kTight: not a segment's first tile
 __device__ __forceinline__ bool softmax_row_tile(uint32_t t_S, uint32_t t_P, uint32_t t_O, float c, int nvalid,

@@ -257,6 +257,29 @@ def test_single_huge_key_in_a_late_tile_is_caught():
     assert U.poll_status() == 0
 
 
+def test_many_weights_far_above_the_reference_do_not_overflow():
+    # 150 items of 12 full key tiles on 148 blocks: whole items, and two leftover ones in parts.  A segment's first tile
+    # has scores 0, all others 61.97 log2 units above it, and |v| is about 2^60: weights of 2^62 against the first
+    # tile's maximum would add up to more than float32 holds within one tile.
+    heads, frames = 150, 12
+    sh = W.Shape(batch=1, heads=heads, chunk_frames=1, grid_h=8, grid_w=16, ring_frames=frames)
+    dev, ora = DevicePath(sh), OraclePath(sh)
+    segs = U.window_attn_plan(dev.abi, [frames - 1], frames, U.attn_workers()[0])
+    assert {s[7] for s in segs} == {frames} and min(s[6] - s[5] for s in segs) >= 3
+    assert {s[8] == 1 for s in segs} == {True, False}                 # whole items, and parts through the scratch
+    dev.ring_k.fill_(3.796875)                                        # x 128 / sqrt(128) x log2(e) = 61.97
+    for s in segs:
+        dev.ring_k[:, s[5], :, s[2]] = 0.0
+    dev.ring_v.copy_((2.0 ** 60 * (1.0 + torch.arange(128, device="cuda") % 4 / 4)).to(torch.bfloat16).expand_as(dev.ring_v))
+    ora.ring.ring_k[...], ora.ring.ring_v[...] = to_bits(dev.ring_k), to_bits(dev.ring_v)
+    q = torch.ones((1, sh.chunk_tokens, heads, 128), dtype=torch.bfloat16, device="cuda")
+    out = to_bits(dev.attend([frames - 1], frames, q))
+    some = [0, 1, 147, 148, 149]
+    _, _, rel = attn_errors(out[:, :, some], ora.attend([frames - 1], frames, to_bits(q), heads=some))
+    assert np.isfinite(O.bf16_bits_to_f32(out)).all() and rel <= REL_L2, rel
+    assert U.poll_status() == 0
+
+
 def test_remainder_smaller_than_the_grid():
     # Work splits whose remainder has fewer steps than there are thread blocks: 11 heads of one
     # query tile over 2 key tiles (the launch shrinks to a few blocks), and 10 heads x 15 query
