@@ -220,34 +220,49 @@ int unstep_window_attn_noalloc(const unstep_shape_t* shape, const int32_t* start
  * The launch is cut into work items (stream, head, pair of 128-query tiles); an item has one step
  * per 128-key tile of its window.  Each of at most `max_workers` workers (one per SM) first takes
  * whole items round-robin (a launch of no more items than workers has no such rounds).  What is left
- * over is split along the keys in one of two ways, whichever is estimated to be shorter: every item
- * into the same number of parts (one or more), one part per worker; or all its steps as one sequence
+ * over is split along the keys in one of three ways, whichever is estimated to be shortest: every item
+ * into the same number of parts (one or more), one part per worker; all its steps as one sequence
  * cut into equal contiguous shares, one per worker, so that an item falls into as many parts as shares
- * touch it.  The parts of an item are merged by the worker that finishes last.  (A launch of no more
- * items than workers may instead cut every item into 2 to 8 parts that are one thread-block cluster, if the
- * device runs that many clusters at once; this list, which asks no device, has the split without clusters.)
+ * touch it; or, in a launch without whole rounds, every item into 2 to 8 parts that are one thread-block
+ * cluster.  The parts of an item are merged through scratch by the worker that finishes last, those
+ * of a cluster through its shared memory.
  *
+ *   clusters : HOST int32 [9]: clusters[n], n = 2 .. 8, is the number of clusters of n thread blocks that
+ *              the device runs at the same time (unstep_attn_clusters; the others are ignored).  NULL: none.
  *   segs     : HOST int32 [max_segs][10], written (may be NULL when max_segs is 0).  One row per
  *              segment in the order the worker walks them: worker, stream, head, query pair,
  *              query tiles in the pair (1 or 2), first key tile, end key tile (exclusive), key
  *              tiles of the whole item, number of parts the item is split into (1 = whole), and the
- *              scratch slot (0 or 1) the part is published in (-1 for a whole item).
+ *              scratch slot (0 or 1) the part is published in (-1 for a whole item and for a part of a cluster).
  *   n_segs   : HOST int32, written: the number of segments of the launch (may exceed max_segs; only
  *              the first max_segs rows are written).
  * Only the first launch of the call is listed (the first 32 streams).  Arguments are checked as in
  * unstep_window_attn_sink; sink_frames = 0 lists the plain rolling window.
+ *
+ * With the workers and clusters of a device (the two functions below) the list is the launch on it.
+ * unstep_window_attn_plan is the list for a device that runs no clusters.
  */
+int unstep_window_attn_plan_clusters(const unstep_shape_t* shape, int32_t sink_frames, const int32_t* start_frame,
+                                     int32_t recent_frames, int32_t sink_attend, int32_t max_workers,
+                                     const int32_t* clusters, int32_t* segs, int32_t max_segs, int32_t* n_segs);
 int unstep_window_attn_plan(const unstep_shape_t* shape, int32_t sink_frames, const int32_t* start_frame,
                             int32_t recent_frames, int32_t sink_attend, int32_t max_workers,
                             int32_t* segs, int32_t max_segs, int32_t* n_segs);
 
 /*
  * How the attention calls will use the current device (the paper has no counterpart): the number
- * of workers of a full-size launch (the `max_workers` to give unstep_window_attn_plan: one per SM)
+ * of workers of a full-size launch (the `max_workers` to give the plan functions: one per SM)
  * and the thread blocks per worker (1: every worker is one persistent thread block).
  *   workers, ctas_per_worker : HOST int32, written.
  */
 int unstep_attn_workers(int32_t* workers, int32_t* ctas_per_worker);
+
+/*
+ * The clusters of n attention thread blocks that the current device runs at the same time, n = 2 .. 8: the
+ * `clusters` to give unstep_window_attn_plan_clusters.
+ *   clusters : HOST int32 [9], written (0 in the first two).
+ */
+int unstep_attn_clusters(int32_t* clusters);
 
 /* Static, human-readable text for a status code. */
 const char* unstep_strerror(int code);

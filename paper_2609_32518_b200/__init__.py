@@ -17,6 +17,7 @@ from .binding import (  # noqa: F401
     rmsnorm_rope_kv_append,
     window_attn_plan,
     attn_workers,
+    attn_clusters,
     poll_status,
     shutdown,
     selftest_wait_limit,

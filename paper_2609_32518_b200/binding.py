@@ -14,7 +14,9 @@ from . import build as _build
 
 EXPORTS = ("unstep_rope_table", "unstep_rope_kv_append", "unstep_window_attn",
            "unstep_window_attn_noalloc", "unstep_rope_kv_append_sink", "unstep_window_attn_sink",
-           "unstep_rmsnorm_rope_kv_append", "unstep_window_attn_plan", "unstep_attn_workers", "unstep_selftest_wait_limit", "unstep_shutdown", "unstep_strerror", "unstep_poll_status", "unstep_launch_count")
+           "unstep_rmsnorm_rope_kv_append", "unstep_window_attn_plan", "unstep_window_attn_plan_clusters",
+           "unstep_attn_workers", "unstep_attn_clusters", "unstep_selftest_wait_limit", "unstep_shutdown",
+           "unstep_strerror", "unstep_poll_status", "unstep_launch_count")
 
 
 class UnstepError(RuntimeError):
@@ -89,6 +91,12 @@ def lib() -> ctypes.CDLL:
         L.unstep_window_attn_plan.restype = c_int
         L.unstep_window_attn_plan.argtypes = [POINTER(Shape), c_int32, POINTER(c_int32), c_int32, c_int32,
                                               c_int32, POINTER(c_int32), c_int32, POINTER(c_int32)]
+        L.unstep_window_attn_plan_clusters.restype = c_int
+        L.unstep_window_attn_plan_clusters.argtypes = [POINTER(Shape), c_int32, POINTER(c_int32), c_int32, c_int32,
+                                                       c_int32, POINTER(c_int32), POINTER(c_int32), c_int32,
+                                                       POINTER(c_int32)]
+        L.unstep_attn_clusters.restype = c_int
+        L.unstep_attn_clusters.argtypes = [POINTER(c_int32)]
         L.unstep_attn_workers.restype = c_int
         L.unstep_attn_workers.argtypes = [POINTER(c_int32), POINTER(c_int32)]
         L.unstep_selftest_wait_limit.restype = c_int
@@ -341,17 +349,23 @@ def _general_window_attn_sink(shape, sink_frames, start_frame, recent_frames, si
 
 
 def window_attn_plan(shape: Shape, start_frame, recent_frames: int, max_workers: int, sink_frames: int = 0,
-                     sink_attend: int = 0):
-    """unstep_window_attn_plan: the segments of one attention launch as rows of 10 ints (worker,
-    stream, head, query pair, query tiles, first key tile, end key tile, tiles of the item, parts,
-    scratch slot).  Host only."""
+                     sink_attend: int = 0, clusters=None):
+    """unstep_window_attn_plan_clusters: the segments of one attention launch as rows of 10 ints (worker,
+    stream, head, query pair, query tiles, first key tile, end key tile, tiles of the item, parts, scratch
+    slot, -1 for a whole item or a part of a cluster).  `clusters`: the limits as attn_clusters() returns
+    them, None for a device that runs no clusters.  Host only."""
     n = c_int32(0)
     starts = _starts(shape, start_frame)
+    if clusters is not None:
+        if len(clusters) != 9:
+            raise ValueError("clusters needs 9 entries")
+        clusters = (c_int32 * 9)(*clusters)
     args = (ctypes.byref(shape), int(sink_frames), starts, int(recent_frames), int(sink_attend),
-            int(max_workers))
-    _check(lib().unstep_window_attn_plan(*args, None, 0, ctypes.byref(n)), "unstep_window_attn_plan")
+            int(max_workers), clusters)
+    where = "unstep_window_attn_plan_clusters"
+    _check(lib().unstep_window_attn_plan_clusters(*args, None, 0, ctypes.byref(n)), where)
     buf = (c_int32 * (10 * max(n.value, 1)))()
-    _check(lib().unstep_window_attn_plan(*args, buf, n.value, ctypes.byref(n)), "unstep_window_attn_plan")
+    _check(lib().unstep_window_attn_plan_clusters(*args, buf, n.value, ctypes.byref(n)), where)
     return [tuple(buf[10 * i:10 * i + 10]) for i in range(n.value)]
 
 
@@ -360,6 +374,13 @@ def attn_workers():
     a, b = c_int32(0), c_int32(0)
     _check(lib().unstep_attn_workers(ctypes.byref(a), ctypes.byref(b)), "unstep_attn_workers")
     return a.value, b.value
+
+
+def attn_clusters():
+    """unstep_attn_clusters: how many clusters of n attention blocks run at the same time, at index n (2 .. 8)."""
+    buf = (c_int32 * 9)()
+    _check(lib().unstep_attn_clusters(buf), "unstep_attn_clusters")
+    return list(buf)
 
 
 def selftest_wait_limit(limit_cycles: int, stream=None):

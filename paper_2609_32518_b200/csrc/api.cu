@@ -24,10 +24,10 @@ extern "C" int64_t unstep_launch_count(void) { return unstep::g_launches.load();
 
 // The work split of an attention launch, listed on the host with the same code the kernel's
 // roles run on the device.
-extern "C" int unstep_window_attn_plan(const unstep_shape_t* shape, int32_t sink_frames,
-                                       const int32_t* start_frame, int32_t recent_frames,
-                                       int32_t sink_attend, int32_t max_workers, int32_t* segs,
-                                       int32_t max_segs, int32_t* n_segs) {
+extern "C" int unstep_window_attn_plan_clusters(const unstep_shape_t* shape, int32_t sink_frames,
+                                                const int32_t* start_frame, int32_t recent_frames,
+                                                int32_t sink_attend, int32_t max_workers, const int32_t* clusters,
+                                                int32_t* segs, int32_t max_segs, int32_t* n_segs) {
   using namespace unstep;
   int rc = check_attn_args(shape, start_frame, recent_frames, sink_frames, sink_attend);
   if (rc != UNSTEP_OK) return rc;
@@ -37,7 +37,7 @@ extern "C" int unstep_window_attn_plan(const unstep_shape_t* shape, int32_t sink
   AttnParams p;
   plan_shape(p, shape, sink_frames);
   const int nb = shape->batch < kMaxStreamsPerLaunch ? shape->batch : kMaxStreamsPerLaunch;
-  rc = plan_launch(p, shape, start_frame, nb, recent_frames, sink_frames, sink_attend, max_workers);
+  rc = plan_launch(p, shape, start_frame, nb, recent_frames, sink_frames, sink_attend, max_workers, clusters);
   if (rc != UNSTEP_OK) return rc;
   int64_t n = 0;
   for (int w = 0; w < p.n_workers; ++w) {
@@ -56,7 +56,7 @@ extern "C" int unstep_window_attn_plan(const unstep_shape_t* shape, int32_t sink
         o[6] = s.t1;
         o[7] = s.tiles;
         o[8] = whole ? 1 : last_part_worker(p, s) - first_part_worker(p, s) + 1;
-        o[9] = whole ? -1 : part_slot(p, w, s.item_step0);
+        o[9] = whole || p.cluster ? -1 : part_slot(p, w, s.item_step0);
       }
       ++n;
     }
@@ -64,4 +64,12 @@ extern "C" int unstep_window_attn_plan(const unstep_shape_t* shape, int32_t sink
   if (n > INT32_MAX) return UNSTEP_ERR_INVALID_ARG;
   *n_segs = static_cast<int32_t>(n);
   return UNSTEP_OK;
+}
+
+extern "C" int unstep_window_attn_plan(const unstep_shape_t* shape, int32_t sink_frames,
+                                       const int32_t* start_frame, int32_t recent_frames,
+                                       int32_t sink_attend, int32_t max_workers, int32_t* segs,
+                                       int32_t max_segs, int32_t* n_segs) {
+  return unstep_window_attn_plan_clusters(shape, sink_frames, start_frame, recent_frames, sink_attend, max_workers,
+                                          nullptr, segs, max_segs, n_segs);
 }

@@ -1237,6 +1237,16 @@ extern "C" int unstep_attn_workers(int32_t* workers, int32_t* ctas_per_worker) {
   return UNSTEP_OK;
 }
 
+extern "C" int unstep_attn_clusters(int32_t* clusters) {
+  if (clusters == nullptr) return UNSTEP_ERR_INVALID_ARG;
+  const int rc = check_device();
+  if (rc != UNSTEP_OK) return rc;
+  const DeviceInfo& info = device_info();
+  if (!info.ok) return UNSTEP_ERR_CUDA;
+  for (int n = 0; n <= kMaxClusterParts; ++n) clusters[n] = info.clusters[n];
+  return UNSTEP_OK;
+}
+
 #ifdef UNSTEP_CHECK
 namespace unstep {
 // One store just past the end of a 4-element buffer: a checking build must skip it and record it.

@@ -1,11 +1,13 @@
 """The work split of the attention kernel, replayed on the host (no GPU).
 
-The kernel's roles all walk the same integer schedule; `unstep_window_attn_plan` lists it with the
+The kernel's roles all walk the same integer schedule; `unstep_window_attn_plan(_clusters)` lists it with the
 same code compiled for the host.  Whatever the shape, window and worker count, every (item, key
 tile) step must be covered exactly once, a split item's parts must be counted correctly (a part
 that waits for more parts than exist would never merge, and its rows would never be written), and
-no two parts of one worker may share a scratch slot."""
+no two parts of one worker may share a scratch slot.  Parts that are a cluster take no slot: they are one
+segment per worker, and the parts of an item the blocks of one cluster, in order."""
 
+import ctypes
 import itertools
 
 import pytest
@@ -13,8 +15,13 @@ import pytest
 import paper_2609_32518_b200 as U
 
 
-def check_plan(shape, starts, window, workers, sink=0, sink_attend=0):
-    segs = U.window_attn_plan(shape, starts, window, workers, sink, sink_attend)
+CLUSTERS = [0, 0, 74, 45, 33, 26, 22, 15, 15]   # clusters of n blocks that the 148 SMs of a B200 run at once
+
+
+def check_plan(shape, starts, window, workers, sink=0, sink_attend=0, clusters=None):
+    segs = U.window_attn_plan(shape, starts, window, workers, sink, sink_attend, clusters)
+    in_cluster = any(s[8] > 1 and s[9] == -1 for s in segs)
+    assert clusters is not None or not in_cluster
     T = shape.grid_h * shape.grid_w
     q_tiles = -(-shape.chunk_frames * T // 128)
     q_pairs = (q_tiles + 1) // 2
@@ -30,8 +37,11 @@ def check_plan(shape, starts, window, workers, sink=0, sink_attend=0):
             assert (item, t) not in covered, f"step {(item, t)} given to two workers"
             covered[(item, t)] = w
         whole = t0 == 0 and t1 == tiles
-        assert (parts == 1 and slot == -1) if whole else (parts >= 2 and slot in (0, 1))
-        if not whole:
+        assert (parts == 1 and slot == -1) if whole else (parts >= 2 and slot in ((-1,) if in_cluster else (0, 1)))
+        if in_cluster:
+            assert parts == segs[0][8] and t1 - t0 in (tiles // parts, tiles // parts + 1)
+            parts_seen.setdefault(item, []).append((w, parts))
+        elif not whole:
             parts_seen.setdefault(item, []).append((w, parts))
             assert slot not in slots_of_worker.setdefault(w, set()), f"worker {w} reuses scratch slot {slot}"
             slots_of_worker[w].add(slot)
@@ -52,6 +62,11 @@ def check_plan(shape, starts, window, workers, sink=0, sink_attend=0):
         ws = sorted(w for w, _ in lst)
         assert all(n == len(lst) for _, n in lst), f"item {item}: {len(lst)} parts, expected {[n for _, n in lst]}"
         assert ws == list(range(ws[0], ws[0] + len(ws)))
+        if in_cluster:   # the blocks of a cluster are neighbours from a multiple of its size on, its parts in their order
+            assert ws[0] % len(ws) == 0
+            assert [s[5] for s in segs if (s[1], s[2], s[3]) == item] == sorted(s[5] for s in segs if (s[1], s[2], s[3]) == item)
+    if in_cluster:
+        assert [s[0] for s in segs] == list(range(n_items * segs[0][8])) and n_items <= clusters[segs[0][8]]
     return segs
 
 
@@ -159,3 +174,44 @@ def test_workers_rise_and_fall_along_a_clip_within_the_grid():
             workers[heads, start] = 1 + max(s[0] for s in segs)
     assert workers[3, 0] < workers[3, 3] and workers[1, 20] < workers[1, 19]
     assert max(workers.values()) <= 148
+
+
+def form(segs):
+    """How a launch is split: "cluster", "scratch" (parts or shares through global memory) or "whole"."""
+    return "cluster" if any(s[8] > 1 and s[9] == -1 for s in segs) else "scratch" if any(s[8] > 1 for s in segs) else "whole"
+
+
+def test_sweep_of_small_shapes_on_a_device_that_runs_clusters():
+    # two streams at different fill levels, without and with sink frames
+    seen = {}
+    for heads, (gh, gw), fc, win, sink in itertools.product((1, 2, 7, 25, 50, 80), ((8, 8), (3, 5), (9, 15), (16, 20)),
+                                                            (1, 3), (0, 6), (0, 2)):
+        ring = fc + win
+        sh = U.Shape.make(batch=2, heads=heads, chunk_frames=fc, grid_h=gh, grid_w=gw, ring_frames=ring)
+        segs = check_plan(sh, [ring + 3, 0], ring, 148, sink, sink, CLUSTERS)
+        seen.setdefault(form(segs), set()).add(max(s[8] for s in segs))
+    assert seen["cluster"] >= {2, 3, 4, 5, 6, 8} and seen["whole"] == {1} and len(seen["scratch"]) > 1
+
+
+def test_limits_of_the_device_decide_which_clusters_a_launch_has():
+    sh = U.Shape.make(batch=1, heads=8, chunk_frames=2, grid_h=9, grid_w=15, ring_frames=9)   # 16 items of 10 tiles
+    parts = lambda clusters: {s[8] for s in check_plan(sh, [7], 9, 148, clusters=clusters)}   # noqa: E731
+    assert parts(CLUSTERS) == {5} and parts([0] * 6 + [0, 0, 16]) == {8}
+    none = check_plan(sh, [7], 9, 148, clusters=[0] * 9)
+    assert none == check_plan(sh, [7], 9, 148) and {s[9] for s in none} == {0}
+    # no clusters behind whole rounds, nor of more parts than the shortest stream has tiles
+    sh = U.Shape.make(batch=1, heads=150, chunk_frames=1, grid_h=10, grid_w=20, ring_frames=9)
+    assert form(check_plan(sh, [8], 9, 148, clusters=CLUSTERS)) == "scratch"
+    sh = U.Shape.make(batch=2, heads=1, chunk_frames=1, grid_h=8, grid_w=8, ring_frames=9)
+    assert {s[8] for s in check_plan(sh, [8, 2], 9, 148, clusters=CLUSTERS)} == {3}
+
+
+def test_the_list_without_clusters_and_its_arguments():
+    sh = U.Shape.make(batch=1, heads=8, chunk_frames=2, grid_h=9, grid_w=15, ring_frames=9)
+    want = [x for s in U.window_attn_plan(sh, [7], 9, 148) for x in s]
+    buf, n, start = (ctypes.c_int32 * len(want))(), ctypes.c_int32(0), (ctypes.c_int32 * 1)(7)
+    rc = U.lib().unstep_window_attn_plan(ctypes.byref(sh), 0, start, 9, 0, 148, buf, len(want) // 10, ctypes.byref(n))
+    assert rc == 0 and 10 * n.value == len(want) and list(buf) == want
+    with pytest.raises(ValueError):
+        U.window_attn_plan(sh, [7], 9, 148, clusters=[0, 0, 74])
+    assert U.lib().unstep_attn_clusters(None) == -1
