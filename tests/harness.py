@@ -114,6 +114,27 @@ class OraclePath:
                              rows=rows, heads=heads)
 
 
+def random_layer(sh: W.Shape, seed: int, k_scale: float = 1.0):
+    """A layer whose caches hold the same random keys and values on both sides, and rotated queries: (device path,
+    oracle path, queries, their bits)."""
+    dev, ora = DevicePath(sh), OraclePath(sh)
+    gen = torch.Generator(device="cuda").manual_seed(seed)
+    for ring, scale in ((dev.ring_k, k_scale), (dev.ring_v, 1.0)):
+        ring.copy_(scale * torch.randn(ring.shape, generator=gen, device="cuda"))
+    share_caches(dev, ora)
+    q = torch.randn((sh.batch, sh.chunk_tokens, sh.heads, sh.head_dim), generator=gen, device="cuda").to(torch.bfloat16)
+    return dev, ora, q, to_bits(q)
+
+
+def share_caches(dev: DevicePath, ora: OraclePath):
+    """The oracle's caches take the device's bytes."""
+    ora.ring.ring_k[...], ora.ring.ring_v[...] = to_bits(dev.ring_k), to_bits(dev.ring_v)
+
+
+def some_heads(sh: W.Shape):
+    return sorted({0, sh.heads // 2, max(sh.heads - 2, 0), sh.heads - 1})
+
+
 def stream_history(wl: W.Workload, dev: DevicePath, ora: OraclePath, check_ring: bool = True):
     """Append every history chunk of every stream on both sides (streams advance
     together where their schedules allow, else one by one is emulated by re-appending)."""

@@ -13,9 +13,7 @@ import itertools
 import pytest
 
 import paper_2609_32518_b200 as U
-
-
-CLUSTERS = [0, 0, 74, 45, 33, 26, 22, 15, 15]   # clusters of n blocks that the 148 SMs of a B200 run at once
+from splits import CLUSTERS, EQUAL_PARTS, SPLITS, forms
 
 
 def check_plan(shape, starts, window, workers, sink=0, sink_attend=0, clusters=None):
@@ -176,11 +174,6 @@ def test_workers_rise_and_fall_along_a_clip_within_the_grid():
     assert max(workers.values()) <= 148
 
 
-def form(segs):
-    """How a launch is split: "cluster", "scratch" (parts or shares through global memory) or "whole"."""
-    return "cluster" if any(s[8] > 1 and s[9] == -1 for s in segs) else "scratch" if any(s[8] > 1 for s in segs) else "whole"
-
-
 def test_sweep_of_small_shapes_on_a_device_that_runs_clusters():
     # two streams at different fill levels, without and with sink frames
     seen = {}
@@ -189,8 +182,9 @@ def test_sweep_of_small_shapes_on_a_device_that_runs_clusters():
         ring = fc + win
         sh = U.Shape.make(batch=2, heads=heads, chunk_frames=fc, grid_h=gh, grid_w=gw, ring_frames=ring)
         segs = check_plan(sh, [ring + 3, 0], ring, 148, sink, sink, CLUSTERS)
-        seen.setdefault(form(segs), set()).add(max(s[8] for s in segs))
-    assert seen["cluster"] >= {2, 3, 4, 5, 6, 8} and seen["whole"] == {1} and len(seen["scratch"]) > 1
+        for f in forms(segs):
+            seen.setdefault(f, set()).add(max(s[8] for s in segs))
+    assert seen["cluster"] >= {2, 3, 4, 5, 6, 8} and "whole" in seen and len(seen["scratch"]) > 1
 
 
 def test_limits_of_the_device_decide_which_clusters_a_launch_has():
@@ -201,7 +195,7 @@ def test_limits_of_the_device_decide_which_clusters_a_launch_has():
     assert none == check_plan(sh, [7], 9, 148) and {s[9] for s in none} == {0}
     # no clusters behind whole rounds, nor of more parts than the shortest stream has tiles
     sh = U.Shape.make(batch=1, heads=150, chunk_frames=1, grid_h=10, grid_w=20, ring_frames=9)
-    assert form(check_plan(sh, [8], 9, 148, clusters=CLUSTERS)) == "scratch"
+    assert forms(check_plan(sh, [8], 9, 148, clusters=CLUSTERS)) == {"whole", "scratch"}
     sh = U.Shape.make(batch=2, heads=1, chunk_frames=1, grid_h=8, grid_w=8, ring_frames=9)
     assert {s[8] for s in check_plan(sh, [8, 2], 9, 148, clusters=CLUSTERS)} == {3}
 
@@ -215,3 +209,20 @@ def test_the_list_without_clusters_and_its_arguments():
     with pytest.raises(ValueError):
         U.window_attn_plan(sh, [7], 9, 148, clusters=[0, 0, 74])
     assert U.lib().unstep_attn_clusters(None) == -1
+
+
+@pytest.mark.parametrize("name", list(SPLITS))
+def test_launches_that_the_gpu_tests_rely_on(name):
+    (batch, heads, grid, fc, ring, starts), want, parts = SPLITS[name]
+    sh = U.Shape.make(batch=batch, heads=heads, chunk_frames=fc, grid_h=grid[0], grid_w=grid[1], ring_frames=ring)
+    segs = U.window_attn_plan(sh, starts, ring, 148, clusters=CLUSTERS)
+    assert forms(segs) == want and max(s[8] for s in segs) == parts
+    if batch <= 32:
+        check_plan(sh, starts, ring, 148, clusters=CLUSTERS)
+
+
+@pytest.mark.parametrize("batch,heads,grid,fc,ring,win,history,starts,parts", EQUAL_PARTS)
+def test_launches_of_equal_parts_are_clusters(batch, heads, grid, fc, ring, win, history, starts, parts):
+    sh = U.Shape.make(batch=batch, heads=heads, chunk_frames=fc, grid_h=grid[0], grid_w=grid[1], ring_frames=ring)
+    segs = check_plan(sh, starts, win, 148, clusters=CLUSTERS)
+    assert forms(segs) == {"cluster"} and {s[8] for s in segs} == {parts}

@@ -13,7 +13,9 @@ import torch
 import oracle as O
 import paper_2609_32518_b200 as U
 import workloads as W
-from harness import (DevicePath, OraclePath, assert_ring_equal, attn_errors, stream_history, to_bits)
+from harness import (DevicePath, OraclePath, assert_ring_equal, attn_errors, random_layer, share_caches, some_heads,
+                     stream_history, to_bits)
+from splits import EQUAL_PARTS, SPLITS, forms, shortest_part, split_on_device
 
 pytestmark = pytest.mark.gpu
 
@@ -218,28 +220,27 @@ def test_split_items_merge_in_a_fixed_order_bitwise_repeatable():
     assert U.poll_status() == 0
 
 
-def test_scores_far_above_the_first_tiles_maximum_take_the_redo_path():
-    # Later key tiles are exponentiated against the first tile's row maximum and only checked
-    # afterwards; scores more than 64 (log2 units) above it make the kernel find the true
-    # maximum, rescale and redo the tile.  History with ordinary keys, then a chunk whose keys are
-    # 64 times larger: its scores have a standard deviation of ~90 log2 units.
+def test_parts_whose_maxima_lie_far_apart():
+    # History with ordinary keys, then a chunk whose keys are 64 times larger: its scores have a standard
+    # deviation of ~90 log2 units.  On a B200 every key tile is a part of its own here, with a maximum of its own, and
+    # the merge of the cluster has to cope with weights that differ by more than float32 holds.  (A jump inside a
+    # segment: test_keys_far_above_the_reference_in_segments_of_several_tiles.)
     base = W.WORKLOADS["cfg1"]
     dev, ora = DevicePath(base.shape), OraclePath(base.shape)
     stream_history(base, dev, ora)
     big = W.Workload("huge_keys", base.shape, seed=26, history_starts=base.history_starts,
                      measured_starts=base.measured_starts, window_frames=(6, 4), k_scale=64.0)
     run(big, dev=dev, ora=ora)
-    # and back to ordinary keys on top of the huge ones (the reference maximum is now far too high
-    # for most rows of the newest keys: their weights underflow, as in the exact softmax)
+    # and back to ordinary keys on top of the huge ones (the weights of the newest keys underflow for most
+    # rows, as in the exact softmax)
     after = W.Workload("after_huge", base.shape, seed=27, history_starts=base.history_starts,
                        measured_starts=(6,), window_frames=(6, 2))
     run(after, dev=dev, ora=ora)
 
 
-def test_single_huge_key_in_a_late_tile_is_caught():
-    # One key of a late tile scores hundreds of log2 units above everything else for about half of
-    # the rows (its exponential against the first tile's maximum overflows to inf): those rows
-    # must be redone against the true maximum.
+def test_single_huge_key_in_the_last_part():
+    # One key of the last tile, a part of its own on a B200, scores hundreds of log2 units above everything else for
+    # about half of the rows: the other parts' weights vanish there and decide the other rows.
     wl = W.WORKLOADS["cfg1"]
     dev, ora = DevicePath(wl.shape), OraclePath(wl.shape)
     stream_history(wl, dev, ora)             # 4 frames of 64 tokens = two full key tiles
@@ -271,7 +272,7 @@ def test_many_weights_far_above_the_reference_do_not_overflow():
     for s in segs:
         dev.ring_k[:, s[5], :, s[2]] = 0.0
     dev.ring_v.copy_((2.0 ** 60 * (1.0 + torch.arange(128, device="cuda") % 4 / 4)).to(torch.bfloat16).expand_as(dev.ring_v))
-    ora.ring.ring_k[...], ora.ring.ring_v[...] = to_bits(dev.ring_k), to_bits(dev.ring_v)
+    share_caches(dev, ora)
     q = torch.ones((1, sh.chunk_tokens, heads, 128), dtype=torch.bfloat16, device="cuda")
     out = to_bits(dev.attend([frames - 1], frames, q))
     some = [0, 1, 147, 148, 149]
@@ -293,18 +294,42 @@ def test_remainder_smaller_than_the_grid():
     run(wl, rows_fn=lambda L: np.concatenate([W.sample_rows(L, per_tile=2), np.arange(3328, L, 7)]), heads=[0, 9])
 
 
-@pytest.mark.parametrize("batch,heads,grid,fc,ring,win,history,starts", [
-    (2, 5, (17, 23), 2, 7, 5, ((4, 6, 8, 10), (2, 4, 6)), (12, 8)),        # 3 parts, 16 and 17 key tiles
-    (1, 1, (20, 30), 3, 9, 9, ((3, 6, 9),), (12,)),                        # 5 parts
-    (3, 1, (11, 13), 3, 9, 9, ((), (0, 3), (3, 6, 9)), (0, 6, 12)),        # 3 parts, 4 and 11 key tiles
-    (2, 4, (16, 24), 1, 6, 6, (tuple(range(3, 9)), (0,)), (9, 1)),         # 4 parts, a lone query tile
-    (1, 3, (9, 14), 1, 5, 5, ((1, 2, 3, 4, 5),), (6,)),                    # whole items, frames below a tile
-])
-def test_items_cut_into_equal_parts(batch, heads, grid, fc, ring, win, history, starts):
+@pytest.mark.parametrize("batch,heads,grid,fc,ring,win,history,starts,parts", EQUAL_PARTS)   # clusters on a B200
+def test_items_cut_into_equal_parts(batch, heads, grid, fc, ring, win, history, starts, parts):
     sh = W.Shape(batch=batch, heads=heads, chunk_frames=fc, grid_h=grid[0], grid_w=grid[1], ring_frames=ring)
     wl = W.Workload("parts", sh, seed=31, history_starts=history, measured_starts=starts, window_frames=(win,),
                     k_scale=4.0)
     run(wl)
+
+
+def layer_of(name, seed, k_scale):
+    """One launch of SPLITS, which must be split as its name says on this device."""
+    (batch, heads, grid, fc, ring, starts), want, _ = SPLITS[name]
+    sh = W.Shape(batch=batch, heads=heads, chunk_frames=fc, grid_h=grid[0], grid_w=grid[1], ring_frames=ring)
+    dev, ora, q, q_bits = random_layer(sh, seed, k_scale)
+    segs = split_on_device(dev.abi, starts, ring)
+    assert forms(segs) == want, (name, U.attn_clusters())
+    return sh, starts, segs, dev, ora, q, q_bits
+
+
+@pytest.mark.parametrize("name", list(SPLITS))
+def test_every_form_of_the_split(name):
+    # whole items, parts and shares merged through scratch (up to and beyond four parts, streams of unequal
+    # length), clusters: against the oracle, and the same bits whichever part finishes last
+    sh, starts, _, dev, ora, q, q_bits = layer_of(name, 41, 4.0)
+    heads = some_heads(sh)
+    out = to_bits(dev.attend(starts, sh.ring_frames, q))
+    check(out[:, :, heads], ora.attend(starts, sh.ring_frames, q_bits, heads=heads), name, strict=False)
+    assert np.isfinite(O.bf16_bits_to_f32(out)).all()
+    for _ in range(3):
+        assert np.array_equal(to_bits(dev.attend(starts, sh.ring_frames, q)), out)
+    assert U.poll_status() == 0
+
+
+def test_cluster_limits_of_the_device():
+    workers, limits = U.attn_workers()[0], U.attn_clusters()
+    assert len(limits) == 9 and limits[:2] == [0, 0]
+    assert all(0 <= limits[n] <= workers // n for n in range(2, 9)) and limits[2] > 0
 
 
 # Items of 135-token frames, two query tiles and a lone one of 14 rows per head, cut into 2 to 8 parts that are a
@@ -328,9 +353,9 @@ def test_items_whose_parts_are_a_cluster(heads, frames, parts):
     ((9, 14), 1, 4, (0, 1, 2), 3, (32, 125)),          # frames just below a tile
 ])
 def test_keys_far_above_the_reference_wherever_they_sit(grid, fc, ring, history, start, keys):
-    # The reference of a segment is the maximum of its first tile.  Single keys 256 times larger score
-    # hundreds of log2 units above the others (for about half of the rows): in the first tile they must
-    # be found, in a later one the tile must be redone, in tiles of up to 64 keys and in full ones.
+    # Single keys 256 times larger score hundreds of log2 units above the others (for about half of the
+    # rows), in tiles of up to 64 keys and in full ones.  On a B200 every tile is a part of its own here and its
+    # first, so they must be found among its columns; the test below has segments of several tiles.
     sh = W.Shape(batch=1, heads=2, chunk_frames=fc, grid_h=grid[0], grid_w=grid[1], ring_frames=ring)
     wl = W.Workload("far_keys", sh, seed=32, history_starts=(history,), measured_starts=(start,), window_frames=(ring,))
     T = sh.tokens_per_frame
@@ -347,6 +372,37 @@ def test_keys_far_above_the_reference_wherever_they_sit(grid, fc, ring, history,
     assert np.array_equal(to_bits(q_dev), q_ref)
     check(to_bits(dev.attend([start], ring, q_dev)), ora.attend([start], ring, q_ref), f"keys {keys}")
     assert U.poll_status() == 0
+
+
+@pytest.mark.parametrize("name", ["whole_and_parts", "four_parts", "cluster"])
+@pytest.mark.parametrize("place", ["first", "full", "ragged", "rising"])
+def test_keys_far_above_the_reference_in_segments_of_several_tiles(name, place):
+    # The reference of a segment is the maximum of its first tile, and moves where a later tile has a score more than 57
+    # (log2 units) above it: O is rescaled then.  Keys 256 times larger (hundreds of units for about half of the rows)
+    # in the first tile, where they must be found, in a full tile and in the last, ragged one, where the
+    # reference must move; "rising" moves it in every tile.
+    sh, starts, segs, dev, ora, q, q_bits = layer_of(name, 42, 1.0)
+    frames, T, heads = sh.ring_frames, sh.tokens_per_frame, some_heads(sh)
+    keys = frames * T
+    assert starts[0] == frames - 1 and keys % 128 != 0        # the cache in order; a ragged last tile
+    assert min(s[6] - s[5] for s in segs) >= 3
+    K = dev.ring_k.view(keys, sh.heads, 128)
+    moves = []
+    for s in segs:
+        h, t0, t1 = s[2], s[5], s[6]
+        at = {"first": [(t0 * 128 + 33, 256.0)], "full": [(t0 * 128 + 128 + 100, 256.0)],
+              "ragged": [(keys - 1, 256.0)] if t1 == s[7] else [],
+              "rising": [(t * 128 + 5, 64.0 * (1 + t - t0)) for t in range(t0, t1)]}[place]
+        for key, scale in at:
+            K[key, h] = (K[key, h].float() * scale).to(torch.bfloat16)
+        if h in heads and at:
+            scores = q[0, :, h].float() @ K[t0 * 128:min(t1 * 128, keys), h].float().T * 0.12751743
+            moves.append(bool((scores[:, 128:].amax(1) - scores[:, :128].amax(1) > 57).any()))
+    assert moves and all(m == (place != "first") for m in moves)
+    share_caches(dev, ora)
+    out = to_bits(dev.attend(starts, frames, q))
+    check(out[:, :, heads], ora.attend(starts, frames, q_bits, heads=heads), f"{name} {place}", strict=False)
+    assert np.isfinite(O.bf16_bits_to_f32(out)).all() and U.poll_status() == 0
 
 
 @pytest.mark.parametrize("heads,grid,ring", [(2, (8, 8), 6), (12, (30, 52), 9)])   # parts, and whole items as well

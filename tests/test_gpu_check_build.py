@@ -4,7 +4,7 @@ No memory checker can be run on the kernels here, so the library carries its own
 build every global store of the three kernels is tested against the extent of the buffer it
 belongs to, and a store outside is skipped and reported through the status word instead of being
 made.  This file runs the shapes with the most index arithmetic (tiny, ragged tiles, more streams
-than one launch carries, a sink prefix, the fused norm) through that build, with every output
+than one launch carries, a sink prefix, the fused norm, parts merged in clusters and through scratch) through that build, with every output
 placed between two bands of sentinel values, and asserts: status 0 (no store was refused), bands
 intact (no store landed outside), results equal to the oracle.  The checking build is loaded in a
 child process (UNSTEP_LIB_VARIANT=check), so the normal library of this process is untouched.
@@ -31,6 +31,7 @@ def _child():
     import paper_2609_32518_b200 as U
     import workloads as W
     from harness import OraclePath, abi_shape, attn_errors, to_dev
+    from splits import forms, split_on_device
 
     assert os.path.basename(U.lib()._name) == "libunstep_check.so"
 
@@ -51,9 +52,11 @@ def _child():
         def bits(self):
             return self.t.contiguous().view(torch.int16).cpu().numpy().view(np.uint16)
 
-    def run(wl, extra_history=(), sink=0, sink_attend=0, norm=False, out_offset=0):
+    def run(wl, extra_history=(), sink=0, sink_attend=0, norm=False, out_offset=0, split=None):
         sh = wl.shape
         abi = abi_shape(sh)
+        if split is not None:
+            assert forms(split_on_device(abi, wl.measured_starts, wl.window_frames[0])) == split, wl.name
         cache_shape = (sh.batch, sink + sh.ring_frames, sh.tokens_per_frame, sh.heads, sh.head_dim)
         act_shape = (sh.batch, sh.chunk_tokens, sh.heads, sh.head_dim)
         ck, cv = Guarded(cache_shape), Guarded(cache_shape)
@@ -176,6 +179,14 @@ def _child():
     sh = W.Shape(batch=2, heads=3, chunk_frames=2, grid_h=3, grid_w=5, ring_frames=6)
     run(W.Workload("norm", sh, seed=35, history_starts=((), ()), measured_starts=(6, 2), window_frames=(6, 2)),
         extra_history=[[0, 0], [2, 0], [4, 0]], norm=True)
+    # parts and shares merged through scratch: 150 items, the last two in parts behind a whole round, and 80 items of
+    # 20 key tiles as shares
+    sh = W.Shape(batch=1, heads=150, chunk_frames=4, grid_h=5, grid_w=8, ring_frames=8)
+    run(W.Workload("scratch_parts", sh, seed=36, history_starts=((),), measured_starts=(4,), window_frames=(8,)),
+        extra_history=[[0]], split={"whole", "scratch"})
+    sh = W.Shape(batch=1, heads=80, chunk_frames=5, grid_h=5, grid_w=8, ring_frames=20)
+    run(W.Workload("scratch_shares", sh, seed=37, history_starts=((),), measured_starts=(15,), window_frames=(20,)),
+        extra_history=[[0], [5], [10]], split={"scratch"})
     print("all ok")
 
 

@@ -5,6 +5,7 @@ import pytest
 import torch
 
 import paper_2609_32518_b200 as U
+from splits import forms, split_on_device
 
 pytestmark = pytest.mark.gpu
 BF16 = torch.bfloat16
@@ -24,6 +25,8 @@ class Layer:
         self.cos, self.sin = (torch.zeros(self.sh.chunk_tokens, 64, device="cuda") for _ in range(2))
         self.q_rot, self.out = torch.zeros_like(self.q), torch.zeros_like(self.q)
         self.norm, self.attn = norm, U.window_attn_noalloc if noalloc else U.window_attn
+        # 77 heads and more are 154 items and more: a whole round, and parts merged through scratch behind it
+        assert ("scratch" in forms(split_on_device(self.sh, [6], 6))) == (heads >= 77)
 
     def steps(self):
         # every call reads what the one before it wrote, and writes what the one before that read
@@ -53,14 +56,14 @@ def same(a, b):
     return all(torch.equal(x.view(torch.uint8), y.view(torch.uint8)) for x, y in zip(a, b))
 
 
-@pytest.mark.parametrize("norm", [False, True])
+@pytest.mark.parametrize("norm,heads", [(False, 3), (True, 3), (False, 80)])
 @pytest.mark.parametrize("noalloc", [False, True])
-def test_dependent_calls_back_to_back(norm, noalloc):
-    want = Layer(1, norm=norm, noalloc=noalloc)
+def test_dependent_calls_back_to_back(norm, noalloc, heads):
+    want = Layer(1, heads, norm=norm, noalloc=noalloc)
     for _ in range(3):
         want.run(sync=True)
     for _ in range(4):
-        got = Layer(1, norm=norm, noalloc=noalloc)
+        got = Layer(1, heads, norm=norm, noalloc=noalloc)
         torch.cuda.synchronize()
         for _ in range(3):
             got.run()
@@ -69,9 +72,10 @@ def test_dependent_calls_back_to_back(norm, noalloc):
     assert U.poll_status() == 0
 
 
-def test_two_streams_at_once():
-    want = [Layer(s, heads=h) for s, h in ((2, 3), (3, 12))]
-    got = [Layer(s, heads=h) for s, h in ((2, 3), (3, 12))]
+@pytest.mark.parametrize("heads", [(3, 12), (77, 80)])   # clusters, and parts in the scratch of either stream
+def test_two_streams_at_once(heads):
+    want = [Layer(s, heads=h) for s, h in zip((2, 3), heads)]
+    got = [Layer(s, heads=h) for s, h in zip((2, 3), heads)]
     for layer in want:
         layer.run(sync=True)
     torch.cuda.synchronize()
@@ -83,12 +87,12 @@ def test_two_streams_at_once():
         assert same(g.state(), w.state())
 
 
-@pytest.mark.parametrize("noalloc", [False, True])
-def test_under_capture_with_a_fork_and_a_join(noalloc):
-    want, got = Layer(4, noalloc=noalloc), Layer(4, noalloc=noalloc)
-    other_want, other = Layer(5), Layer(5)
+@pytest.mark.parametrize("noalloc,heads", [(False, 3), (True, 3), (False, 77), (True, 77)])
+def test_under_capture_with_a_fork_and_a_join(noalloc, heads):
+    want, got = Layer(4, heads, noalloc=noalloc), Layer(4, heads, noalloc=noalloc)
+    other_want, other = Layer(5, heads), Layer(5, heads)
     main, side = torch.cuda.Stream(), torch.cuda.Stream()
-    for stream, layer in ((main, Layer(6, noalloc=noalloc)), (side, Layer(7))):   # scratch of both streams
+    for stream, layer in ((main, Layer(6, heads, noalloc=noalloc)), (side, Layer(7, heads))):   # scratch of both streams
         with torch.cuda.stream(stream):
             layer.run()
     torch.cuda.synchronize()

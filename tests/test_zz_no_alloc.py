@@ -16,7 +16,8 @@ import torch
 import oracle as O
 import paper_2609_32518_b200 as U
 import workloads as W
-from harness import DevicePath, OraclePath, to_bits
+from harness import DevicePath, OraclePath, random_layer, some_heads, to_bits
+from splits import SPLITS, forms, split_on_device
 
 FAKE = 0x10000
 
@@ -45,8 +46,8 @@ def _check_against_oracle(got_bits, ref, what):
 
 @pytest.mark.gpu
 def test_noalloc_entry_point_matches_the_oracle_and_the_regular_one_twice_in_a_row():
-    # 2 streams x 3 heads x 3 query pairs of 14 ragged key tiles over ~31 CTAs: most items are
-    # split across CTAs, so both calls go through the scratch (partials, counters, merge)
+    # 2 streams x 3 heads x 3 query pairs of 5 to 11 ragged key tiles: clusters on a B200, which merge their parts
+    # in shared memory (launches through the fixed array: test_parts_and_counters_in_the_fixed_array)
     sh = W.Shape(batch=2, heads=3, chunk_frames=3, grid_h=8, grid_w=25, ring_frames=7)
     wl = W.Workload("noalloc", sh, seed=31, history_starts=((), ()), measured_starts=(9, 3),
                     window_frames=(7,), k_scale=4.0)
@@ -72,8 +73,7 @@ def test_noalloc_entry_point_matches_the_oracle_and_the_regular_one_twice_in_a_r
 
 @pytest.mark.gpu
 def test_noalloc_with_more_streams_than_one_launch_carries():
-    # 33 streams: two kernel launches of one call, back to back on one stream, share the array
-    # (the second clears and reuses the counters the first has just used)
+    # 33 streams: two kernel launches of one call, back to back on one stream, clusters both on a B200
     sh = W.Shape(batch=33, heads=2, chunk_frames=1, grid_h=8, grid_w=20, ring_frames=3)
     starts = tuple(2 + (b % 3) for b in range(33))
     wl = W.Workload("noalloc33", sh, seed=32, history_starts=((),) * 33, measured_starts=starts,
@@ -95,3 +95,25 @@ def test_noalloc_with_more_streams_than_one_launch_carries():
         assert U.poll_status() == 0
         _check_against_oracle(to_bits(got), ref, f"33 streams, call {rep}")
         assert np.array_equal(to_bits(dev.attend(starts, 3, q_rot)), to_bits(got))
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("name", ["whole_and_parts", "shares", "many_parts", "shares_of_32_streams"])
+def test_parts_and_counters_in_the_fixed_array(name):
+    # Launches whose parts are merged through the array, two calls in a row with other queries: the second finds
+    # the partial results and counters of the first there.  33 streams are two launches of one call.  The split goes by
+    # 160 and more items, or by items of very many tiles, and does not depend on the clusters that a device runs.
+    (batch, heads, grid, fc, ring, starts), want, _ = SPLITS[name]
+    sh = W.Shape(batch=batch, heads=heads, chunk_frames=fc, grid_h=grid[0], grid_w=grid[1], ring_frames=ring)
+    dev, ora, q, _ = random_layer(sh, 43)
+    assert forms(split_on_device(dev.abi, starts, ring)) == want and "scratch" in want
+    some = some_heads(sh)
+    for rep in range(2):
+        q = q if rep == 0 else q.flip(1).contiguous()
+        regular = to_bits(dev.attend(starts, ring, q))
+        got = torch.full_like(q.view(torch.int16), 0x7FC1).view(torch.bfloat16)
+        U.window_attn_noalloc(dev.abi, list(starts), ring, q, dev.ring_k, dev.ring_v, got)
+        torch.cuda.synchronize()
+        assert U.poll_status() == 0
+        assert np.array_equal(regular, to_bits(got)), f"call {rep}: results differ bitwise"
+        _check_against_oracle(to_bits(got)[:, :, some], ora.attend(starts, ring, to_bits(q), heads=some), f"{name}, call {rep}")
