@@ -19,9 +19,11 @@ static int n_tiles, segment, n_groups, n_warps;
 
 struct Rule {
   const char* name;
-  bool two;   // two barriers of a kind per group, or one
+  bool two;             // two barriers of a kind per group, or one
+  bool gave_up_waits;   // a warp that gave up waits at the barriers (the kernel's rule), or only arrives there too
   int s_free(int a, int tile) const { return unstep::s_free_barrier(a, two ? tile : 0); }
   int p_ready(int a, int tile) const { return unstep::p_ready_barrier(a, two ? tile : 0); }
+  bool waits(bool gave_up) const { return gave_up_waits && unstep::p_ready_waits(gave_up); }
 };
 
 enum Stage : int8_t { kWaitS, kAtS, kWaitPv, kAtP, kEpilogue, kAtGroup };   // kAt*: waiting at a barrier
@@ -101,7 +103,7 @@ static std::vector<State> successors(const State& s, const Rule& r) {
       if (!w.gave && !seen) continue;
       State t = s;
       Warp& x = t.w[a][k];
-      const bool waits = unstep::p_ready_waits(w.gave);
+      const bool waits = r.waits(w.gave);
       int b;
       if (w.stage == kWaitS) {
         b = r.s_free(a, w.tile);
@@ -142,7 +144,8 @@ static std::vector<State> successors(const State& s, const Rule& r) {
 int main(int argc, char** argv) {
   if (argc != 5) return 2;
   n_tiles = atoi(argv[1]), segment = atoi(argv[2]), n_groups = atoi(argv[3]), n_warps = atoi(argv[4]);
-  for (const Rule& r : {Rule{"kernel", true}, Rule{"one_barrier", false}}) {
+  for (const Rule& r : {Rule{"kernel", true, true}, Rule{"one_barrier", false, true}, Rule{"one_barrier_arrive", false, false},
+                        Rule{"two_barriers_arrive", true, false}}) {
     std::set<std::vector<int8_t>> seen;
     std::vector<State> todo = {State()};
     seen.insert(State().flat());

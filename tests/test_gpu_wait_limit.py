@@ -1,6 +1,6 @@
 """Bounded device-side waits: a wait that can never be satisfied gives up, reports it through
 the status word and leaves the context usable (no trap, no hang).  The probe is the wait alone; what the
-attention kernel's roles do behind a wait that gave up is shown on the CPU (test_hand_over.py)."""
+attention kernel's roles do behind a wait that gave up is shown on the CPU (test_score_hand_over.py)."""
 
 import time
 

@@ -1,6 +1,7 @@
 """S goes back to the Q K^T issuer and P on to the P V issuer through named barriers, which have no bounded
 wait: whatever wait gave up where, every warp must get past all of them.  A model of the barriers' counts
-walks through all orders, with the kernel's own rule (csrc/handover.h) and with one barrier of each kind."""
+walks through all orders, with the kernel's own rule (csrc/handover.h) and with rules that leave somebody behind: one
+barrier of each kind, and warps that gave up and do not wait at the barriers."""
 
 import os
 import shutil
@@ -31,5 +32,9 @@ def test_no_order_leaves_a_warp_at_a_barrier(model, tiles, segment, groups, warp
                          text=True).stdout
     blocked = {line.split()[0]: int(line.split()[2]) for line in out.splitlines()}
     assert blocked["kernel"] == 0
+    if tiles > 1:
+        assert blocked["one_barrier_arrive"] > 0
     if tiles > 1 and warps > 1:
         assert blocked["one_barrier"] > 0
+    if tiles > 2:
+        assert blocked["two_barriers_arrive"] > 0
