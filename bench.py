@@ -48,7 +48,7 @@ L2_BYTES = 126e6
 # dram__bytes_read.sum + dram__bytes_write.sum of one window_attn launch at cfg2 from the ncu
 # capture summarised in profiles/window_attn_cfg2_ncu_full.txt, and the range seen over all
 # captures of that kernel at that workload (the L2 state at the start of the launch differs)
-ATTN_DRAM_TRAFFIC = {"bytes": 336_592_128, "capture": "profiles/window_attn_cfg2_ncu_full.txt",
+ATTN_DRAM_TRAFFIC = {"bytes": 362_149_120, "capture": "profiles/window_attn_cfg2_ncu_full.txt",
                      "range_over_captures_mb": [286, 402],
                      "note": "one launch under ncu, which replays it: parts of K and V may be in L2 when it begins"}
 
@@ -552,7 +552,6 @@ def run_ours(args):
                      "frac_of_nominal_2250": attn_tflops / 2250.0,
                      "traffic": ATTN_DRAM_TRAFFIC["bytes"] if default_cfg else None,
                      "traffic_source": ATTN_DRAM_TRAFFIC if default_cfg else None,
-                     "mcycles_per_launch": (t_attn * 1e3 * clocks["sm_mhz"] / 1e6) if clocks and clocks.get("sm_mhz") else None,
                      "sustained": sustained},
         "append_roofline": {"kernel": "rmsnorm_rope_kv_append_token_kernel" if args.rmsnorm else "rope_kv_append_kernel",
                             "bound": "hbm", "achieved": append_bytes / (t_append * 1e-3) / 1e9,
