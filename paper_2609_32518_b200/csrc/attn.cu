@@ -13,8 +13,8 @@
 // follows when P is there.  So the next scores are there when a group is done with its tile, and the
 // two groups share the MUFU pipe without waiting for the tensor core.  (With an S for each tile and P over
 // S, a tile's next Q K^T had to wait for its P V: exponentials, hand-over, P V and Q K^T were one
-// chain of ~3500 clk per key tile.  12 heads, 4680 queries, 32760 keys: 1422 -> 1184 thousand
-// cycles, 878 -> 800 us run on end at the power cap, 754 -> 693 us in a burst.)
+// chain of ~3500 clk per key tile.  12 heads, 4680 queries, 32760 keys: 1423-1431 -> 1184-1219 thousand
+// cycles and 881-884 -> 808-815 us run on end at the power cap, 755-757 -> 694-697 us in runs of 20.)
 //
 // What a group does per key tile is as long as the period, so it counts how fast it is fetched: its
 // loop over the full tiles is kept short and free of taken branches (rare cases are out of line, one
@@ -205,9 +205,9 @@ __device__ __forceinline__ void mask_block32(uint32_t* s, int col0, int nvalid) 
 // float32 sums are as accurate as near 1 (same relative precision), and what was accumulated before such a jump
 // is negligible exactly as in the true softmax.  A tile's sum of P is at most 128 * 2^57 = 2^64, the sum of n keys
 // at most n * 2^57, and O that times |v|: finite for any window that the entry points take (2^30 keys) up to
-// |v| = 2^40, for 32760 keys up to 2^55.  (A score may be 64 above the reference with |v| 2^7 smaller; the results of
-// ordinary keys are the same.)  The scores have left TMEM by the time a sum of P could tell, so the maximum is looked
-// for in front: 64 three-input maxima in the shadow of the other group's exponentials.
+// |v| = 2^40, for 32760 keys up to 2^55.  (With kJump = 64, tiles of 128 keys 62 above the reference overflowed with |v| =
+// 2^60.)  The scores have left TMEM by the time a sum of P could tell, so the maximum is looked for in front: 64
+// three-input maxima in the shadow of the other group's exponentials.
 //
 // P may be stored, and O rescaled, once the P V of the tile before has run.  That barrier, and the one of the next
 // tile's scores, are looked at once, ahead of time: the look takes 100-200 clk under the MMAs' traffic, and

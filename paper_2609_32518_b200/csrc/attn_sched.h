@@ -253,6 +253,11 @@ inline int32_t remainder_parts(int64_t items, int64_t steps, int32_t least, int3
 // of the columns.  Attention alone, us, parts merged through global memory or shares -> clusters: 8 items x 40 steps
 // 28.2 -> 20.0, 8 x 28 25.2 -> 18.6, 15 x 113 46.3 -> 37.1, 20 x 16 21.0 -> 17.8, 36 x 18 24.7 -> 22.1, 40 x 43 38.3
 // -> 35.5, 57 x 37 42.7 -> 41.7, 2 x 6 11.6 -> 10.0; 38 items x 256 steps: shares 138, 3 parts 153.
+// That is the time of one launch.  The finer cut takes more SMs for it, and launches of several streams side by side
+// lose where two no longer fit the device at once: per launch, us, 1 / 2 / 3 streams, parts through global memory
+// -> clusters: 20 x 16 21.8 / 12.2 / 9.7 -> 18.4 / 13.9 / 13.7 (80 -> 120 blocks), 24 x 7 20.0 / 10.0 / 6.9 -> 15.4 / 10.0 /
+// 9.0 (48 -> 96), 2 x 6 13.1 / 6.7 / 4.7 -> 10.2 / 5.3 / 3.7 (6 -> 12).  Streams that are served together go into one
+// launch, so the line is drawn by the single launch.
 inline int32_t cluster_parts(int64_t items, int32_t least, int32_t most, const int32_t* clusters, double us) {
   int32_t best = 0;
   for (int32_t parts = 2; parts <= kMaxClusterParts && parts <= least; ++parts) {
