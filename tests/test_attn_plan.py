@@ -64,7 +64,9 @@ def check_plan(shape, starts, window, workers, sink=0, sink_attend=0, clusters=N
             assert ws[0] % len(ws) == 0
             assert [s[5] for s in segs if (s[1], s[2], s[3]) == item] == sorted(s[5] for s in segs if (s[1], s[2], s[3]) == item)
     if in_cluster:
-        assert [s[0] for s in segs] == list(range(n_items * segs[0][8])) and n_items <= clusters[segs[0][8]]
+        parts = segs[0][8]
+        assert [s[0] for s in segs] == list(range(n_items * parts))
+        assert n_items <= clusters[parts] - 3 * (parts % 2)   # room for odd ones
     return segs
 
 
@@ -198,6 +200,15 @@ def test_limits_of_the_device_decide_which_clusters_a_launch_has():
     assert forms(check_plan(sh, [8], 9, 148, clusters=CLUSTERS)) == {"whole", "scratch"}
     sh = U.Shape.make(batch=2, heads=1, chunk_frames=1, grid_h=8, grid_w=8, ring_frames=9)
     assert {s[8] for s in check_plan(sh, [8, 2], 9, 148, clusters=CLUSTERS)} == {3}
+
+
+@pytest.mark.parametrize("parts,most", [(3, 42), (5, 23), (7, 12)])
+def test_clusters_of_odd_size_leave_room(parts, most):
+    # 13 key tiles; with all 45 clusters of 3, or 26 of 5, a launch under the one before it ran in two waves
+    for items in range(most - 2, CLUSTERS[parts] + 1):
+        sh = U.Shape.make(batch=1, heads=items, chunk_frames=2, grid_h=8, grid_w=15, ring_frames=13)
+        segs = check_plan(sh, [11], 13, 148, clusters=CLUSTERS)
+        assert (forms(segs) == {"cluster"} and segs[0][8] == parts) == (items <= most), items
 
 
 def test_the_list_without_clusters_and_its_arguments():
