@@ -228,7 +228,7 @@ UNSTEP_HD int part_slot(const AttnParams& p, int c, int64_t item_step0) {
 // steps 82 whole, 5 parts 33, 6 parts 31, 8 parts 33, 86 shares of 4 steps 35; 40 items x 16 steps 35
 // whole, 3 parts 25, 148 shares 36; 80 items x 37 steps behind a whole round: shares.
 inline int32_t remainder_parts(int64_t items, int64_t steps, int32_t least, int32_t most, int max_workers,
-                               int32_t* shares, double* us) {
+                               int32_t* shares) {
   int64_t n = steps / kMinStepsPerWorker;
   n = n < 1 ? 1 : (n > max_workers ? max_workers : n);
   *shares = static_cast<int32_t>(n);
@@ -243,7 +243,6 @@ inline int32_t remainder_parts(int64_t items, int64_t steps, int32_t least, int3
       best = parts;
     }
   }
-  *us = lowest;
   return best;
 }
 
@@ -258,22 +257,40 @@ inline int32_t cluster_limit(const int32_t* clusters, int32_t parts) {
   return parts % 2 != 0 ? clusters[parts] - 3 : clusters[parts];
 }
 
-// The same for parts that form a cluster, which merges them through shared memory: 0 where that is not
-// shorter than `us`.  clusters[n]: clusters of n blocks that the device runs at the same time (148 SMs: 74, 45,
-// 33, 26, 22, 15, 15 of 2 to 8 blocks).  The merge costs about 2.5 us however many the parts, as each merges a share
-// of the columns.  Attention alone, us, parts merged through global memory or shares -> clusters: 8 items x 40 steps
-// 28.2 -> 20.0, 8 x 28 25.2 -> 18.6, 15 x 113 46.3 -> 37.1, 20 x 16 21.0 -> 17.8, 36 x 18 24.7 -> 22.1, 40 x 43 38.3
-// -> 35.5, 57 x 37 42.7 -> 41.7, 2 x 6 11.6 -> 10.0; 38 items x 256 steps: shares 138, 3 parts 153.
+// Parts that form a cluster, which merges them through shared memory: how many, or 0 where the split that
+// remainder_parts chose (p.parts, p.n_active) is shorter.  clusters[n]: clusters of n blocks that the device runs at the
+// same time (148 SMs: 74, 45, 33, 26, 22, 15, 15 of 2 to 8 blocks).  The estimates (us) are fitted to append and attention
+// of 930 launches of 1 to 74 items of 2 to 183 key tiles, each split in every way.  With two query tiles an item, one in
+// brackets: a step 1.35 (1.0), in frames of 65 to 127 tokens, whose tiles all take the masked code, 1.9 (1.4), in a cluster
+// 4 % more; the merge of a cluster 4.1 (2.5) however many the parts, as each merges a share of the columns; through
+// global memory 5.2 (4.1) and 1.3 (1.1) for each part beyond the second; either way 0.024 for each further block.
+// Measured, us, global memory, whole or shares -> clusters: 8 items x 41 key tiles 26.0 -> 22.2, 20 x 40 31.6 -> 26.1, 40 x 41
+// 42.0 -> 40.5, 52 x 40 45.6 -> 43.4, 2 items of a toy layer 14.1 -> 11.2.  Whole and shorter: 74 x 4 16.1, clusters of 2
+// 21.4; 33 x 4 13.3, of 4 16.2; 41 of a toy layer x 3 10.4, of 3 12.6.  Through global memory and shorter, as a long
+// part gains little by the merge: 70 x 183 162-186, of 2 174-207; 72 x 123 114-129, 122-142; 64 x 65 67.4, 71.3.  With one
+// estimate for all (a step 1.6, a merge 2.5, nothing for a block) 19 % of the launches were slower than without clusters,
+// by up to 33 %; 0.8 % are now, by up to 8 %, and all of them take 2 % less on average.
 // That is the time of one launch.  The finer cut takes more SMs for it, and launches of several streams side by side
 // lose where two no longer fit the device at once: per launch, us, 1 / 2 / 3 streams, parts through global memory
 // -> clusters: 20 x 16 21.8 / 12.2 / 9.7 -> 18.4 / 13.9 / 13.7 (80 -> 120 blocks), 24 x 7 20.0 / 10.0 / 6.9 -> 15.4 / 10.0 /
 // 9.0 (48 -> 96), 2 x 6 13.1 / 6.7 / 4.7 -> 10.2 / 5.3 / 3.7 (6 -> 12).  Streams that are served together go into one
 // launch, so the line is drawn by the single launch.
-inline int32_t cluster_parts(int64_t items, int32_t least, int32_t most, const int32_t* clusters, double us) {
+inline int32_t cluster_parts(const AttnParams& p, int64_t items, int64_t steps, int32_t least, int32_t most,
+                             const int32_t* clusters) {
+  const bool lone = p.q_tiles == 1, masked = !p.flat && p.T > kTileN / 2;
+  const double step = masked ? (lone ? 1.4 : 1.9) : (lone ? 1.0 : 1.35), block = 0.024 * static_cast<double>(items);
+  double us;
+  if (p.parts > 0) {
+    us = step * ((most + p.parts - 1) / p.parts) +
+         (p.parts > 1 ? (lone ? 4.1 : 5.2) + (lone ? 1.1 : 1.3) * (p.parts - 2) + block * (p.parts - 1) : 0.0);
+  } else {
+    const double share = static_cast<double>((steps + p.n_active - 1) / p.n_active);
+    us = step * share + 6.0 + 2.2 * (static_cast<double>(steps) / static_cast<double>(items) / share + 1.0);
+  }
   int32_t best = 0;
   for (int32_t parts = 2; parts <= kMaxClusterParts && parts <= least; ++parts) {
     if (items > cluster_limit(clusters, parts) || static_cast<int64_t>(most) * parts > INT32_MAX) continue;
-    const double cost = 1.6 * ((most + parts - 1) / parts) + 2.5;
+    const double cost = 1.04 * step * ((most + parts - 1) / parts) + (lone ? 2.5 : 4.1) + block * (parts - 1);
     if (cost < us) {
       us = cost;
       best = parts;
@@ -344,10 +361,9 @@ inline int plan_launch(AttnParams& p, const unstep_shape_t* shape, const int32_t
   p.narrow = 1;
   if (steps > 0) {
     const int64_t items = static_cast<int64_t>(nb) * p.leftover;
-    double us = 0.0;
-    p.parts = remainder_parts(items, steps, least, most, max_workers, &p.n_active, &us);
+    p.parts = remainder_parts(items, steps, least, most, max_workers, &p.n_active);
     if (clusters != nullptr && p.full_rounds == 0) {
-      const int32_t parts = cluster_parts(items, least, most, clusters, us);
+      const int32_t parts = cluster_parts(p, items, steps, least, most, clusters);
       p.cluster = parts > 0;
       if (p.cluster) p.parts = parts;
     }

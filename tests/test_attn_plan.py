@@ -211,6 +211,17 @@ def test_clusters_of_odd_size_leave_room(parts, most):
         assert (forms(segs) == {"cluster"} and segs[0][8] == parts) == (items <= most), items
 
 
+@pytest.mark.parametrize("heads,grid,fc,ring,form,parts", [
+    (74, (10, 20), 1, 2, "whole", 1), (33, (10, 20), 1, 2, "whole", 1), (41, (8, 8), 2, 3, "whole", 1),   # 4, 4, 3 tiles
+    (2, (8, 8), 2, 6, "cluster", 6), (5, (17, 23), 2, 13, "cluster", 6),                # 2 items of 6 tiles, 20 of 40
+    (10, (17, 23), 2, 5, "cluster", 3), (13, (17, 23), 2, 13, "cluster", 2),            # 40 items of 16 tiles, 52 of 40
+    (10, (30, 52), 1, 15, "scratch", 2), (16, (17, 23), 2, 21, "scratch", 2)])          # 70 items of 183 tiles, 64 of 65
+def test_the_split_is_the_one_that_was_measured_to_be_shortest(heads, grid, fc, ring, form, parts):
+    sh = U.Shape.make(batch=1, heads=heads, chunk_frames=fc, grid_h=grid[0], grid_w=grid[1], ring_frames=ring)
+    segs = check_plan(sh, [ring - fc], ring, 148, clusters=CLUSTERS)
+    assert forms(segs) == {form} and max(s[8] for s in segs) == parts
+
+
 def test_the_list_without_clusters_and_its_arguments():
     sh = U.Shape.make(batch=1, heads=8, chunk_frames=2, grid_h=9, grid_w=15, ring_frames=9)
     want = [x for s in U.window_attn_plan(sh, [7], 9, 148) for x in s]

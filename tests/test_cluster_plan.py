@@ -28,7 +28,7 @@ def plan(tmp_path_factory):
 
 
 @pytest.mark.parametrize("heads,grid,chunk,frames,start,parts", [
-    (25, (9, 15), 2, 3, 1, 2), (20, (9, 15), 2, 8, 6, 3), (15, (9, 15), 2, 7, 5, 4), (11, (9, 15), 2, 9, 7, 5),
+    (25, (9, 15), 2, 10, 8, 2), (20, (9, 15), 2, 8, 6, 3), (15, (9, 15), 2, 7, 5, 4), (11, (9, 15), 2, 9, 7, 5),
     (10, (9, 15), 2, 11, 9, 6), (6, (9, 15), 2, 6, 4, 7), (7, (9, 15), 2, 7, 5, 8), (2, (8, 8), 2, 6, 4, 6),
     (1, (8, 8), 1, 2, 1, 0), (2, (30, 52), 3, 21, 18, 0), (12, (30, 52), 3, 3, 0, 0)])
 def test_every_block_has_one_part(plan, heads, grid, chunk, frames, start, parts):

@@ -334,7 +334,7 @@ def test_cluster_limits_of_the_device():
 
 # Items of 135-token frames, two query tiles and a lone one of 14 rows per head, cut into 2 to 8 parts that are a
 # cluster (on 148 SMs, which hold 74, 45, 33, 26, 22, 15, 15 clusters of 2 to 8 blocks).
-@pytest.mark.parametrize("heads,frames,parts", [(25, 3, 2), (20, 8, 3), (15, 7, 4), (11, 9, 5), (10, 11, 6), (6, 6, 7),
+@pytest.mark.parametrize("heads,frames,parts", [(25, 10, 2), (20, 8, 3), (15, 7, 4), (11, 9, 5), (10, 11, 6), (6, 6, 7),
                                                 (7, 7, 8)])
 def test_items_whose_parts_are_a_cluster(heads, frames, parts):
     sh = W.Shape(batch=1, heads=heads, chunk_frames=2, grid_h=9, grid_w=15, ring_frames=frames)
