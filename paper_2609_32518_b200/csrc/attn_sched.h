@@ -246,15 +246,15 @@ inline int32_t remainder_parts(int64_t items, int64_t steps, int32_t least, int3
   return best;
 }
 
-// How many clusters of `parts` blocks a launch may have: all that the device runs at the same time, but of an odd
-// size three less (42 of 45 clusters of 3, 23 of 26 of 5, 12 of 15 of 7).  A launch that is set up under the kernel in
-// front of it gets the SMs one by one as that one leaves, odd clusters are placed where three or five happen to be
-// free, and the last ones found no place until the first had ended.  Append and attention of 13 key tiles, us, median:
-// clusters of 3: 41 items 24.3, 42 26.3, 43 28.0, 44 35.2, 45 42.3; of 5: 23 20.3, 24 22.9, 25 25.9, 26 24.7.  Over other
-// shapes 42 clusters of 3 are shorter than 42 of 2 (by 9 % on average, 6 % longer at worst), 44 longer; 24 and 25 of 5 are
-// longer than those of 4, 14 and 15 of 7 than those of 8.  Clusters of 2, 4, 6 and 8 never did that, up to 148 blocks.
+// How many clusters of `parts` blocks a launch may have: all that the device runs at the same time, but of 3 and of 5
+// three less (42 of 45, 23 of 26).  A launch that is set up under the kernel in front of it gets the SMs one by one as
+// that one leaves, odd clusters are placed where three or five happen to be free, and the last ones found no place
+// until the first had ended.  Append and attention of 13 key tiles, us, median: clusters of 3: 41 items 24.3, 42 26.3,
+// 43 28.0, 44 35.2, 45 42.3; of 5: 23 20.3, 24 22.9, 25 25.9, 26 24.7.  Over other shapes 42 clusters of 3 are shorter than
+// 42 of 2 (by 9 % on average, 6 % longer at worst), 44 longer; 24 and 25 of 5 are longer than those of 4.  Clusters of 2, 4,
+// 6 and 8 never did that, up to 148 blocks, nor did those of 7, which are 105 blocks at most.
 inline int32_t cluster_limit(const int32_t* clusters, int32_t parts) {
-  return parts % 2 != 0 ? clusters[parts] - 3 : clusters[parts];
+  return parts == 3 || parts == 5 ? clusters[parts] - 3 : clusters[parts];
 }
 
 // Parts that form a cluster, which merges them through shared memory: how many, or 0 where the split that

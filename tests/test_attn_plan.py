@@ -66,7 +66,7 @@ def check_plan(shape, starts, window, workers, sink=0, sink_attend=0, clusters=N
     if in_cluster:
         parts = segs[0][8]
         assert [s[0] for s in segs] == list(range(n_items * parts))
-        assert n_items <= clusters[parts] - 3 * (parts % 2)   # room for odd ones
+        assert n_items <= clusters[parts] - (3 if parts in (3, 5) else 0)   # room for odd ones
     return segs
 
 
@@ -202,13 +202,16 @@ def test_limits_of_the_device_decide_which_clusters_a_launch_has():
     assert {s[8] for s in check_plan(sh, [8, 2], 9, 148, clusters=CLUSTERS)} == {3}
 
 
-@pytest.mark.parametrize("parts,most", [(3, 42), (5, 23), (7, 12)])
+@pytest.mark.parametrize("parts,most", [(3, 42), (5, 23)])
 def test_clusters_of_odd_size_leave_room(parts, most):
     # 13 key tiles; with all 45 clusters of 3, or 26 of 5, a launch under the one before it ran in two waves
+    # (15 of 7 are 105 blocks and never did)
     for items in range(most - 2, CLUSTERS[parts] + 1):
         sh = U.Shape.make(batch=1, heads=items, chunk_frames=2, grid_h=8, grid_w=15, ring_frames=13)
         segs = check_plan(sh, [11], 13, 148, clusters=CLUSTERS)
         assert (forms(segs) == {"cluster"} and segs[0][8] == parts) == (items <= most), items
+    sh = U.Shape.make(batch=1, heads=15, chunk_frames=2, grid_h=8, grid_w=15, ring_frames=13)
+    assert {s[8] for s in check_plan(sh, [11], 13, 148, clusters=CLUSTERS)} == {7}
 
 
 @pytest.mark.parametrize("heads,grid,fc,ring,form,parts", [
