@@ -222,8 +222,8 @@ UNSTEP_HD int part_slot(const AttnParams& p, int c, int64_t item_step0) {
 // parts per item, or 0 for `*shares` equal shares across the items.  Parts leave a worker with one
 // part of one item; shares give the workers less to do, but each then holds parts of two items, one
 // after the other, each with a hand-over, and an item falls into more parts.  The estimates (us)
-// are fitted to launches of 2 to 40 items of 6 to 85 key tiles on a B200 (with the pipeline of one S per query
-// tile; a step takes 1.4 to 1.6 now): a step 1.6; a second part
+// are fitted to launches of 2 to 40 items of 6 to 85 key tiles on a B200, with the pipeline of one S per query
+// tile (the present one's are in cluster_parts): a step 1.6; a second part
 // 3.4, each further one 1.6; shares 6 and 2.2 for each part of an item.  Measured, us: 8 items x 43
 // steps 82 whole, 5 parts 33, 6 parts 31, 8 parts 33, 86 shares of 4 steps 35; 40 items x 16 steps 35
 // whole, 3 parts 25, 148 shares 36; 80 items x 37 steps behind a whole round: shares.
